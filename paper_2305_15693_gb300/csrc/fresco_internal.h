@@ -17,7 +17,7 @@ constexpr int kMaxWidth = 16;     // largest ES kernel width instantiated
 constexpr int kMinWidth = 2;
 constexpr int kMaxTileEdge = 255; // tile-relative cell must fit the 8-bit field of a packed coordinate
 constexpr int kTileCursors = 4;   // placement cursors per tile of a single plan (Geom.sub)
-constexpr int kZSegment = 6;      // 3D single plans: tiles per z-column segment (Geom.zseg)
+constexpr int kZSegmentMax = 16;  // 3D single plans: most tiles per z-column segment (Geom.zseg)
 constexpr int kColMaxPlanes = 64; // column spread: tiles with tmax_z + w above this spread one by one
 constexpr int kDirectPointsPerThread = 8;   // points in flight per thread of k_place_direct
 // fresco_loss_grad_host copies the points in up to kHostChunks pieces of at least

@@ -543,6 +543,130 @@ __device__ __forceinline__ int residue_lists(const typename PT<T>::U *__restrict
     return p1 - p0;
 }
 
+// ---------------------------------------------------------------------------------------------
+// FP64 tiles, points taken by the whole block. An FP64 tile is small (three FP64 fields of its
+// region fill the shared memory in 3D) and holds few points (about 20 in 3D at the usual mask
+// densities), so one thread per point leaves most of the block idle, and FP64 shared-memory
+// atomics are compare-and-swap loops. Here the block takes kOwnedChunk points at a time: (point,
+// axis) tasks evaluate the kernel weights into shared memory, then every point's window is split
+// over the threads. What bounds it is the FP64 pipe (two lanes per clock and SM): one fused
+// multiply-add per window cell.
+constexpr int kOwnedChunk = 32;       // spread: points whose weights are staged at once
+constexpr int kOwnedChunkInterp = 8;  // interpolation: one point per warp (the field leaves little room)
+// Interpolation tiles of more points than this go back to one thread per point: a full block of
+// 256 points takes 472 us (direct) or 353 us (kernel derivative) at w = 13 on one SM, a point
+// taken by a warp 2.7 us.
+constexpr int kWarpPointMax = 128;
+
+// bytes of the staged weights (and derivatives) and window starts of n points, 16-byte aligned
+__host__ __device__ inline size_t owned_bytes(int n, int dim, int w, bool deriv) {
+    return ((size_t)n * dim * w * 8 * (deriv ? 2 : 1) + (size_t)n * 16 + 15) & ~(size_t)15;
+}
+
+// Weights of points p .. p + n - 1: sw[((q * D + a) * (DERIV ? 2 : 1) + der) * W + k] and window
+// starts (region cells) si[4 q + a]. The caller synchronises the block before reading them.
+template <int W, int D, bool DERIV>
+__device__ __forceinline__ void stage_point_weights(const EsPoly<double> &ep,
+                                                    const uint64_t *__restrict__ sorted, int p,
+                                                    int n, double *sw, int *si) {
+    constexpr int HL = W / 2, RW = D == 3 ? 4 : 2;   // words per sorted record
+    constexpr int P = PolyDeg<double>::value, KP = (W + 1) / 2;
+    constexpr int PE = P & ~1, PO = (P & 1) ? P : P - 1;
+    // one task per (point, axis, mirrored pair of kernel intervals): the arithmetic of es_weights
+    // and es_weights_d, spread over the block so that the few points of a chunk do not leave the
+    // evaluation to one warp
+    for (int u = threadIdx.x; u < n * D * KP; u += blockDim.x) {
+        const int t = u / KP, k = u - t * KP;
+        const int q = t / D, a = t - q * D;
+        int rel;
+        double f, x1;
+        unpack_coord<double>(sorted[(int64_t)(p + q) * RW + a], rel, f);
+        const int i0 = rel + support_start<double, W>(f, x1) + HL;
+        if (k == 0) si[4 * q + a] = i0;
+        const double tau = 2.0 * x1 + (double)(W - 1);
+        const double s = tau * tau;
+        double *out = sw + (size_t)t * (DERIV ? 2 : 1) * W;
+        double e = ep.c[k][PE], de = 0.0, o = ep.c[k][PO], dO = 0.0;
+#pragma unroll
+        for (int j = PE - 2; j >= 0; j -= 2) {
+            if (DERIV) de = fma(de, s, e);
+            e = fma(e, s, ep.c[k][j]);
+        }
+#pragma unroll
+        for (int j = PO - 2; j >= 1; j -= 2) {
+            if (DERIV) dO = fma(dO, s, o);
+            o = fma(o, s, ep.c[k][j]);
+        }
+        const double da = (tau + tau) * de, db = fma(s + s, dO, o);
+        if (2 * k + 1 == W) {
+            out[k] = e;
+            if (DERIV) out[W + k] = da;
+        } else {
+            out[k] = fma(tau, o, e);
+            out[W - 1 - k] = fma(-tau, o, e);
+            if (DERIV) {
+                out[W + k] = da + db;
+                out[W + W - 1 - k] = da - db;
+            }
+        }
+    }
+}
+
+// The FP64 spread takes a tile's points this way when a window row pair fills enough threads; with
+// narrow kernels (W^2 < 64 threads of 256) one thread per point with atomics is the better one.
+template <typename T, int W>
+constexpr bool kOwnedSpread = sizeof(T) == 8 && W >= 8;
+
+// Adds the windows of points [p0, p1) to the region (planes of Sxy elements, rows of Ex) without
+// atomics: thread (a, b) owns every cell with x = a and y = b modulo W, of which each window holds
+// exactly one per plane, so no two threads ever add to the same cell and the points need no barrier
+// between them. NP: planes of a circular buffer (column spread), r0 the buffer plane of the
+// region's first plane; NP = 0: planes in order. Measured on GB300, 3D, 20011 points, w = 13:
+// spread stage with its folds 2174 -> 228 us.
+template <int W, int D>
+__device__ __forceinline__ void spread_points_owned(const EsPoly<double> &ep,
+                                                    const uint64_t *__restrict__ sorted, int p0,
+                                                    int p1, int Ex, int Sxy, int NP, int r0,
+                                                    double *ftile, unsigned char *stage) {
+    double *sw = reinterpret_cast<double *>(stage);
+    int *si = reinterpret_cast<int *>(sw + kOwnedChunk * D * W);
+    const int b = threadIdx.x / W, a = threadIdx.x - b * W;
+    for (int p = p0; p < p1; p += kOwnedChunk) {
+        const int n = min(kOwnedChunk, p1 - p);
+        stage_point_weights<W, D, false>(ep, sorted, p, n, sw, si);
+        __syncthreads();
+        if (b < W) {
+            for (int q = 0; q < n; ++q) {
+                const int ix = si[4 * q], iy = si[4 * q + 1];
+                int kx = a - ix % W, ky = b - iy % W;
+                kx += kx < 0 ? W : 0;
+                ky += ky < 0 ? W : 0;
+                const double *w = sw + q * D * W;
+                const double wxy = w[kx] * w[W + ky];
+                double *cell = ftile + (iy + ky) * Ex + ix + kx;
+                if constexpr (D == 2) {
+                    *cell += wxy;
+                } else {
+                    int pl = r0 + si[4 * q + 2];
+                    if (NP) pl -= pl >= NP ? NP : 0;
+                    double v[W];
+                    int o[W];
+#pragma unroll
+                    for (int c = 0; c < W; ++c) {
+                        o[c] = pl * Sxy;
+                        v[c] = cell[o[c]];
+                        ++pl;
+                        if (NP) pl -= pl >= NP ? NP : 0;
+                    }
+#pragma unroll
+                    for (int c = 0; c < W; ++c) cell[o[c]] = fma(wxy, w[2 * W + c], v[c]);
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
 template <typename T, int W, int D>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_spread_own(
     Geom g, EsPoly<T> ep, const typename PT<T>::U *__restrict__ sorted,
@@ -597,6 +721,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_spread_own(
             for (int a = 0; a < D; ++a) x1[a] = (T)l_x1[a * cap + h];
             spread_point_own<T, W, D>(ep, i0, x1, Ex, Exy, ftile, itile, true, fscale);
         }
+    } else if constexpr (kOwnedSpread<T, W>) {
+        spread_points_owned<W, D>(ep, sorted, p0, p1, Ex, Exy, 0, 0, ftile,
+                                  sm_raw + spread_own_tile_bytes(g, sizeof(T)));
     } else {
         for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
             U u[3];
@@ -828,6 +955,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k_spread_col(
                 pl -= pl >= NP ? NP : 0;
                 spread_point_col<T, W>(ep, i0, x1, Ex, Sxy, NP, pl, ftile, itile, true, fscale);
             }
+        } else if constexpr (kOwnedSpread<T, W>) {
+            spread_points_owned<W, D>(ep, sorted, p0, p1, Ex, Sxy, NP, r0, ftile,
+                                      sm_raw + spread_col_tile_bytes(g, sizeof(T)));
         } else {
             for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
                 U u[3];
