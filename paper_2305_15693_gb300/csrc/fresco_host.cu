@@ -521,6 +521,7 @@ void release(fresco_plan_s *p) {
     cufftHandle hs[] = {p->fft_rows, p->fft_cols, p->ifft_cols, p->ifft_rows};
     for (int i = 0; i < 4; ++i)
         if (p->have_fft[i]) cufftDestroy(hs[i]);
+    fresco::direct_free(p->direct);
     p->prof.release();
     delete p;
 }
@@ -899,6 +900,23 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
     const Geom &g = p->geom;
     const MaskGeom &m = p->mgeom;
     cudaStream_t s = p->stream;
+    if (p->direct) {
+        if (h_pts)
+            FR_CUDA(cudaMemcpyAsync(const_cast<T *>(pts), h_pts,
+                                    sizeof(T) * (size_t)(p->n_points * p->dim),
+                                    cudaMemcpyHostToDevice, s));
+        {
+            StageScope sc(p->prof, s, ST_SPREAD);
+            FR_CUDA(fresco::direct_rho<T>(p->direct, pts, p->d_err, s));
+        }
+        {
+            StageScope sc(p->prof, s, ST_MASK);
+            FR_CUDA(fresco::direct_mask<T>(p->direct, loss, s));
+        }
+        p->launches += 2;
+        p->forward_done = true;
+        return FRESCO_OK;
+    }
     {
         StageScope sc(p->prof, p->stream, ST_SORT);
         int nl = 0;
@@ -978,6 +996,12 @@ fresco_status backward_impl(fresco_plan_s *p, const double *grad_out, T *grad) {
     const Geom &g = p->geom;
     const MaskGeom &m = p->mgeom;
     cudaStream_t s = p->stream;
+    if (p->direct) {
+        StageScope sc(p->prof, s, ST_INTERP);
+        FR_CUDA(fresco::direct_grad<T>(p->direct, grad_out, grad, s));
+        p->launches += 1;
+        return FRESCO_OK;
+    }
     if (m.kderiv) {
         {
             StageScope sc(p->prof, p->stream, ST_FFT_INV);
@@ -1297,7 +1321,19 @@ fresco_status fresco_plan(fresco_plan_t *out, int dim, const double *box, int64_
         delete p;
         return FRESCO_ERR_OOM;
     }
-    st = P.precision == FRESCO_F64 ? build_plan<double>(p, P, F) : build_plan<float>(p, P, F);
+    fresco_opts o;
+    fresco_opts_default(&o);
+    if (opts) o = *opts;
+    if (fresco::direct_wanted(n_points, o, P.precision, P.tol))
+        st = fresco::direct_build(&p->direct, dim, n_points, box, P.precision, mask, n_k, F.n, F.s0,
+                                  F.w, F.loss_const);
+    if (!st && p->direct) {
+        p->device_bytes += fresco::direct_bytes(p->direct);
+        st = dalloc(p, &p->d_err, sizeof(int));
+        if (!st) st = cuda_status(cudaMemset(p->d_err, 0, sizeof(int)));
+    } else if (!st) {
+        st = P.precision == FRESCO_F64 ? build_plan<double>(p, P, F) : build_plan<float>(p, P, F);
+    }
     if (st) {
         release(p);
         return st;
@@ -1352,6 +1388,13 @@ fresco_status fresco_get_rho_S(fresco_plan_t p, void *d_rho, void *d_S) {
     fresco::clear_pending_error();
     if (!p || !p->forward_done) return FRESCO_ERR_ARG;
     if (!d_rho && !d_S) return FRESCO_OK;
+    if (p->direct) {
+        p->launches += 1;
+        return cuda_status(
+            p->precision == FRESCO_F64
+                ? fresco::direct_rho_s<double>(p->direct, (double *)d_rho, (double *)d_S, p->stream)
+                : fresco::direct_rho_s<float>(p->direct, (float *)d_rho, (float *)d_S, p->stream));
+    }
     if (!p->d_mask_orig) {
         fresco_status st = dalloc(p, &p->d_mask_orig, sizeof(int) * p->h_mask.size());
         if (st) return st;

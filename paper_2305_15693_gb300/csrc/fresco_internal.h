@@ -337,6 +337,26 @@ inline void clear_pending_error() { (void)cudaGetLastError(); }
 void es_poly_table(int w, double beta, EsPoly<float> &out);
 void es_poly_table(int w, double beta, EsPoly<double> &out);
 
+// Direct sums for small plans (fresco_direct.cu). direct_wanted: the plan's options leave the choice
+// to the library; direct_build leaves *out null where the problem is large enough for the NUFFT.
+struct DirectPlan;
+bool direct_wanted(int64_t n_points, const fresco_opts &o, int precision, double tol);
+fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const double *box,
+                           int precision, const int32_t *mask, int64_t n_k,
+                           const std::vector<int32_t> &rep_n, const std::vector<double> &rep_s0,
+                           const std::vector<double> &rep_w, double loss_const);
+void direct_free(DirectPlan *d);
+int64_t direct_bytes(const DirectPlan *d);
+// sums over the points; S, the loss and the gradient coefficients; the gradient; rho and S
+template <typename T>
+cudaError_t direct_rho(DirectPlan *d, const T *pts, int *err, cudaStream_t s);
+template <typename T>
+cudaError_t direct_mask(DirectPlan *d, double *loss, cudaStream_t s);
+template <typename T>
+cudaError_t direct_grad(DirectPlan *d, const double *grad_out, T *grad, cudaStream_t s);
+template <typename T>
+cudaError_t direct_rho_s(DirectPlan *d, T *rho, T *S, cudaStream_t s);
+
 #ifdef __CUDACC__
 // Knuth's two-sum: s + e == a + b exactly (round to nearest, no overflow)
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
@@ -436,6 +456,7 @@ struct fresco_plan_s {
     cufftHandle ifft_rows = 0;       // C2C inverse along x, all rows (kderiv: nf0/2, in place)
     bool have_fft[4] = {false, false, false, false};
 
+    fresco::DirectPlan *direct = nullptr;   // small problems: direct sums, none of the above
     fresco::StageProfile prof;
     int64_t launches = 0;
     bool forward_done = false;

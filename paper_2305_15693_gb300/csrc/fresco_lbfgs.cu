@@ -455,6 +455,7 @@ fresco_status fresco_lbfgs_create(fresco_lbfgs_t *out, fresco_plan_t plan,
     }
     fresco_lbfgs_s *s = new (std::nothrow) fresco_lbfgs_s();
     if (!s) return FRESCO_ERR_OOM;
+    if (plan->direct) o.tile_order = 0;   // direct sums have no tiles: the caller's order is as good
     s->plan = plan;
     s->opts = o;
     s->n = info.n_points * info.dim;
