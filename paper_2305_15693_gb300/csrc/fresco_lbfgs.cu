@@ -3,9 +3,10 @@
 //
 // All vectors (positions, gradients, search direction, the m (s, y) history pairs) stay on the
 // device in the plan's precision; every inner product keeps FP64 accuracy (per thread a float
-// pair for FP32 vectors, fresco::DotAcc) and is reduced in FP64 in a fixed two-stage order. The two-loop recursion keeps its scalars (rho_i, alpha_i, beta, gamma) in
-// device memory, so it runs without host round trips; the host reads back two scalars per
-// line-search trial (the trial loss and, once per iteration, the slope and the step bound).
+// pair for FP32 vectors, fresco::DotAcc) and is reduced in FP64 in a fixed order. The two-loop
+// recursion, the step bound and the first trial point are one launch (or one per pair and
+// direction on long vectors), the trial's pair and its products another; the host reads the
+// scalars once per trial and decides.
 //
 // Algorithm (Nocedal & Wright, Numerical Optimization, Alg. 7.4 / 7.5):
 //   d = -H g by the two-loop recursion over the stored pairs, H0 = (s.y)/(y.y) I;
@@ -13,8 +14,10 @@
 //   t0 = min(1, max_step / max_j |d_j|)        (no coordinate moves more than max_step);
 //   t = t0, t0/2, ... until L(x + t d) <= L(x) + c1 t g.d (at most max_backtrack halvings);
 //   s = t d, y = g(x + t d) - g(x); the pair is stored only if s.y > 0.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -28,99 +31,285 @@ namespace {
 constexpr int kRedBlocks = 1024;
 constexpr int kRedThreads = 256;
 
+// Device scalars; the first SL_READ of them are what the host reads, in one copy per trial.
 enum Slot {
-    SL_TMP = 0,     // scratch dot
-    SL_GAMMA_NUM,   // s.y of the newest pair
-    SL_GAMMA_DEN,   // y.y of the newest pair
-    SL_BETA,
-    SL_GD,          // g.d
+    SL_GD = 0,      // g.d
     SL_DMAX,        // max |d_j|
-    SL_GG,          // g.g
+    SL_LOSS,        // loss at the trial point
     SL_SY,          // s.y of the candidate pair
-    SL_RHO0,        // rho_i at SL_RHO0 + i, alpha_i at SL_RHO0 + m + i, i = 0..m-1
+    SL_YY,          // y.y of the candidate pair
+    SL_GG,          // g.g at the trial point (or at the start point)
+    SL_READ,
+    SL_BETA = SL_READ,
+    SL_GAMMA,       // s.y / y.y of the newest stored pair at SL_GAMMA + slot; then, likewise per
+                    // slot, rho = 1 / s.y and alpha (slots() entries each)
 };
 
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_dot_part(const T *__restrict__ a,
-                                                          const T *__restrict__ b, int64_t n,
-                                                          double *__restrict__ part) {
-    __shared__ double ws[kRedThreads / 32];
-    fresco::DotAcc<T> dot;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        dot.add(a[i], b[i]);
-    double acc = dot.value();
+// Block sums (or maxima) of NV values; results in thread 0
+template <int NV, int NT>
+__device__ __forceinline__ void block_reduce(double (&v)[NV], bool is_max) {
+    __shared__ double ws[NV][NT / 32];
+    __syncthreads();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kRedThreads / 32; ++w) s += ws[w];
-        part[blockIdx.x] = s;
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_absmax_part(const T *__restrict__ a, int64_t n,
-                                                             double *__restrict__ part) {
-    __shared__ double ws[kRedThreads / 32];
-    T mt = T(0);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        mt = fmax(mt, fabs(a[i]));
-    double m = (double)mt;
+    for (int k = 0; k < NV; ++k) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = m;
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v[k], o);
+            v[k] = is_max ? fmax(v[k], u) : v[k] + u;
+        }
+        if ((threadIdx.x & 31) == 0) ws[k][threadIdx.x >> 5] = v[k];
+    }
     __syncthreads();
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            double r = ws[k][0];
+            for (int w = 1; w < NT / 32; ++w) r = is_max ? fmax(r, ws[k][w]) : r + ws[k][w];
+            v[k] = r;
+        }
+}
+
+// Grid sums (or maxima) of NV values: every block leaves its own, the block that finishes last adds
+// them in block order (so the result repeats) and returns true in its thread 0, with the totals in
+// v. done is zero before the launch and after it.
+template <int NV>
+__device__ __forceinline__ bool grid_reduce(double (&v)[NV], bool is_max,
+                                            double *__restrict__ part,
+                                            unsigned *__restrict__ done) {
+    __shared__ bool s_last;
+    block_reduce<NV, kRedThreads>(v, is_max);
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kRedThreads / 32; ++w) s = fmax(s, ws[w]);
-        part[blockIdx.x] = s;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) part[(int64_t)k * gridDim.x + blockIdx.x] = v[k];
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
     }
-}
-
-// out = (sum or max of part[0..nb)) * (mul ? *mul : 1); fixed order
-__global__ void __launch_bounds__(256) k_final(const double *__restrict__ part, int nb, int is_max,
-                                               const double *__restrict__ mul,
-                                               double *__restrict__ out) {
-    __shared__ double sm[256];
-    double v = 0.0;
-    for (int i = threadIdx.x; i < nb; i += 256) v = is_max ? fmax(v, part[i]) : v + part[i];
-    sm[threadIdx.x] = v;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-            sm[threadIdx.x] = is_max ? fmax(sm[threadIdx.x], sm[threadIdx.x + o])
-                                     : sm[threadIdx.x] + sm[threadIdx.x + o];
-        __syncthreads();
+    if (!s_last) return false;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        double r = 0.0;   // (maxima are of absolute values)
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedThreads) {
+            const double u = __ldcg(part + (int64_t)k * gridDim.x + i);
+            r = is_max ? fmax(r, u) : r + u;
+        }
+        v[k] = r;
     }
-    if (threadIdx.x == 0) *out = sm[0] * (mul ? *mul : 1.0);
+    block_reduce<NV, kRedThreads>(v, is_max);
+    if (threadIdx.x == 0) *done = 0;
+    return threadIdx.x == 0;
 }
 
-// y += sign * (*a - (b ? *b : 0)) * x
+// *out = a.b
 template <typename T>
-__global__ void k_axpy_dev(T *__restrict__ y, const T *__restrict__ x, int64_t n,
-                           const double *__restrict__ a, const double *__restrict__ b,
-                           double sign) {
-    const T c = (T)(sign * (*a - (b ? *b : 0.0)));
+__global__ void __launch_bounds__(kRedThreads) k_dot(const T *__restrict__ a,
+                                                     const T *__restrict__ b, int64_t n,
+                                                     double *__restrict__ part,
+                                                     unsigned *__restrict__ done,
+                                                     double *__restrict__ out) {
+    fresco::DotAcc<T> acc;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = fma(c, x[i], y[i]);
+        acc.add(a[i], b[i]);
+    double v[1] = {acc.value()};
+    if (grid_reduce<1>(v, false, part, done)) *out = v[0];
 }
 
-// y = scale * x, scale = (num ? *num / *den : s0); non-positive denominators give scale 1
 template <typename T>
-__global__ void k_scale_copy(T *y, const T *x, int64_t n,
-                             const double *__restrict__ num, const double *__restrict__ den,
-                             double s0) {
-    double c = s0;
-    if (num) c = (*den > 0.0 && *num > 0.0) ? *num / *den : 1.0;
-    const T ct = (T)c;
+__global__ void __launch_bounds__(kRedThreads) k_absmax(const T *__restrict__ a, int64_t n,
+                                                        double *__restrict__ part,
+                                                        unsigned *__restrict__ done,
+                                                        double *__restrict__ out) {
+    T m = T(0);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        m = fmax(m, fabs(a[i]));
+    double v[1] = {(double)m};
+    if (grid_reduce<1>(v, true, part, done)) *out = v[0];
+}
+
+// The candidate pair of a trial point: s = xt - x, y = gt - g, with s.y, y.y and gt.gt in the same
+// pass, and 1 / s.y, s.y / y.y for the slot it would take.
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) k_candidate(
+    T *__restrict__ s, T *__restrict__ y, const T *__restrict__ xt, const T *__restrict__ x,
+    const T *__restrict__ gt, const T *__restrict__ g, int64_t n, double *__restrict__ part,
+    unsigned *__restrict__ done, double *__restrict__ sc, double *__restrict__ gamma,
+    double *__restrict__ rho) {
+    fresco::DotAcc<T> sy, yy, gg;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const T gi = gt[i];
+        const T si = fma(T(-1), x[i], xt[i]), yi = fma(T(-1), g[i], gi);
+        s[i] = si;
+        y[i] = yi;
+        sy.add(si, yi);
+        yy.add(yi, yi);
+        gg.add(gi, gi);
+    }
+    double v[3] = {sy.value(), yy.value(), gg.value()};
+    if (grid_reduce<3>(v, false, part, done)) {
+        sc[SL_SY] = v[0];
+        sc[SL_YY] = v[1];
+        sc[SL_GG] = v[2];
+        // (non-positive products give scale 1; the pair is stored only if s.y > 0)
+        *gamma = (v[1] > 0.0 && v[0] > 0.0) ? v[0] / v[1] : 1.0;
+        *rho = 1.0 / v[0];
+    }
+}
+
+// The stored pairs, newest first, passed by value; gamma, rho and alpha lie in the device scalars.
+constexpr int kMaxHistory = 64;
+struct History {
+    int count;
+    int slot[kMaxHistory];
+    const void *s[kMaxHistory], *y[kMaxHistory];
+};
+
+// Two-loop recursion, d = -H g, with g.d, max |d|, and the first trial point xt = x + t d,
+// t = min(1, max_step / max |d|), for vectors that fit the registers of one cluster: kTlBlocks
+// blocks of kTlThreads threads with up to E elements each. Every dot product is a block sum and one
+// exchange over the cluster's shared memory. A launch per vector operation costs more than these
+// operations up to about 3e4 elements (20 points of history: 60 launches, 190 us, against one of
+// 25 us at 2048 FP64 elements); beyond, k_two_loop_step does one launch per pair and direction.
+constexpr int kTlBlocks = 8, kTlThreads = 256;
+
+template <typename T, int E>
+__global__ void __cluster_dims__(kTlBlocks, 1, 1) __launch_bounds__(kTlThreads)
+    k_two_loop(const __grid_constant__ History hist, const T *__restrict__ g,
+               const T *__restrict__ x, T *__restrict__ d, T *__restrict__ xt, int64_t n,
+               double max_step, double *__restrict__ sc, const double *__restrict__ gamma,
+               const double *__restrict__ rho) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ double slot[2][2];
+    __shared__ double alpha[kMaxHistory];
+    const int64_t i0 = (int64_t)blockIdx.x * kTlThreads + threadIdx.x;
+    constexpr int64_t ST = kTlBlocks * kTlThreads;
+    int phase = 0;
+    // sums (or maxima) over the cluster of one value per thread, the same in every thread
+    auto total = [&](double v0, bool is_max) -> double {
+        double v[1] = {v0};
+        block_reduce<1, kTlThreads>(v, is_max);
+        if (threadIdx.x == 0) slot[phase][0] = v[0];
+        cl.sync();
+        double r = 0.0;
+#pragma unroll
+        for (int b = 0; b < kTlBlocks; ++b) {
+            const double u = *cl.map_shared_rank(&slot[phase][0], b);
+            r = is_max ? fmax(r, u) : r + u;
+        }
+        phase ^= 1;   // the other buffer next: a block writes this one again only after the next
+        return r;     // exchange, which every block reaches after this read
+    };
+    auto dot = [&](const T (&v)[E], const T *__restrict__ b) -> double {
+        fresco::DotAcc<T> acc;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (i0 + e * ST < n) acc.add(b[i0 + e * ST], v[e]);
+        return total(acc.value(), false);
+    };
+    auto axpy = [&](T (&v)[E], const T *__restrict__ b, double c) {
+        const T ct = (T)c;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (i0 + e * ST < n) v[e] = fma(ct, b[i0 + e * ST], v[e]);
+    };
+    T v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = i0 + e * ST < n ? g[i0 + e * ST] : T(0);
+    const int m = hist.count;
+    for (int k = 0; k < m; ++k) {              // newest to oldest
+        const double a = dot(v, (const T *)hist.s[k]) * rho[hist.slot[k]];
+        if (threadIdx.x == 0) alpha[k] = a;
+        axpy(v, (const T *)hist.y[k], -a);
+    }
+    if (m) {
+        const T ct = (T)gamma[hist.slot[0]];
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = ct * v[e];
+    }
+    __syncthreads();
+    for (int k = m - 1; k >= 0; --k) {         // oldest to newest
+        const double b = dot(v, (const T *)hist.y[k]) * rho[hist.slot[k]];
+        axpy(v, (const T *)hist.s[k], alpha[k] - b);
+    }
+    T mx = T(0);
+    fresco::DotAcc<T> acc;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        v[e] = T(-1) * v[e];
+        if (i0 + e * ST < n) {
+            acc.add(g[i0 + e * ST], v[e]);
+            mx = fmax(mx, fabs(v[e]));
+        }
+    }
+    const double gd = total(acc.value(), false);
+    const double dmax = total((double)mx, true);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc[SL_GD] = gd;
+        sc[SL_DMAX] = dmax;
+    }
+    const T t = (T)fmin(1.0, max_step / dmax);
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (i0 + e * ST < n) {
+            d[i0 + e * ST] = v[e];
+            xt[i0 + e * ST] = fma(t, v[e], x[i0 + e * ST]);
+        }
+    cl.sync();   // no block leaves while another may still read its shared memory
+}
+
+// One step of the recursion over a vector of any length: v = in (+ c a), c = sign (*c0 - *c1),
+// times *scale, negated if neg; then, in the same pass, v.b times *mul into *out and, if out_max,
+// max |v|. Null pointers leave their part out.
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads) k_two_loop_step(
+    T *__restrict__ v, const T *in, const T *__restrict__ a, const double *__restrict__ c0,
+    const double *__restrict__ c1, double sign, const double *__restrict__ scale, int neg,
+    const T *__restrict__ b, const double *__restrict__ mul, int64_t n, double *__restrict__ part,
+    unsigned *__restrict__ done, double *__restrict__ out, double *__restrict__ out_max) {
+    const T c = a ? (T)(sign * (*c0 - (c1 ? *c1 : 0.0))) : T(0);
+    const T st = scale ? (T)*scale : T(1);
+    fresco::DotAcc<T> acc;
+    T mx = T(0);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        T u = in[i];
+        if (a) u = fma(c, a[i], u);
+        if (scale) u = st * u;
+        if (neg) u = T(-1) * u;
+        v[i] = u;
+        if (b) acc.add(b[i], u);
+        mx = fmax(mx, fabs(u));
+    }
+    double r[1] = {acc.value()};
+    if (b && grid_reduce<1>(r, false, part, done)) *out = r[0] * (mul ? *mul : 1.0);
+    if (!out_max) return;
+    // (a second pass over the blocks' counters: the sum's is zero again only once its last block
+    // is done, so the maximum has its own)
+    double q[1] = {(double)mx};
+    if (grid_reduce<1>(q, true, part + gridDim.x, done + 1)) *out_max = q[0];
+}
+
+// y = s0 x
+template <typename T>
+__global__ void k_scale_copy(T *y, const T *x, int64_t n, double s0) {
+    const T ct = (T)s0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         y[i] = ct * x[i];
+}
+
+// z = x + min(1, max_step / *dmax) b
+template <typename T>
+__global__ void k_first_trial(T *__restrict__ z, const T *__restrict__ x, const T *__restrict__ b,
+                              int64_t n, double max_step, const double *__restrict__ dmax) {
+    const T tt = (T)fmin(1.0, max_step / *dmax);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        z[i] = fma(tt, b[i], x[i]);
 }
 
 // z = a + t * b
@@ -132,8 +321,6 @@ __global__ void k_lincomb(T *__restrict__ z, const T *__restrict__ a, const T *_
          i += (int64_t)gridDim.x * blockDim.x)
         z[i] = fma(tt, b[i], a[i]);
 }
-
-__global__ void k_set(double *__restrict__ p, double v) { *p = v; }
 
 }  // namespace
 
@@ -150,10 +337,13 @@ struct fresco_lbfgs_s {
     bool have_order = false;
     void *g = nullptr, *d = nullptr, *xt = nullptr, *gt = nullptr;
     std::vector<void *> S, Y;
-    double *scal = nullptr;   // device scalars
+    double *scal = nullptr;   // device scalars (Slot)
     double *part = nullptr;   // reduction partials
-    double *loss_x = nullptr, *loss_t = nullptr;   // device losses
-    int count = 0, head = 0;  // stored pairs, index of the next slot
+    unsigned *done = nullptr; // blocks finished in the running reductions
+    double *h_scal = nullptr; // pinned host copy of the first SL_READ scalars
+    // stored pairs; head is the slot the next candidate pair is written to. There is one slot more
+    // than the history holds, so a candidate that is not accepted overwrites no stored pair
+    int count = 0, head = 0;
     int64_t evals = 0, iters = 0;
 };
 
@@ -166,22 +356,82 @@ struct Ops {
         int64_t b = (s->n + kRedThreads - 1) / kRedThreads;
         return (int)std::max<int64_t>(1, std::min<int64_t>(b, kRedBlocks));
     }
-    void dot(const void *a, const void *b, double *out, const double *mul = nullptr) {
-        k_dot_part<T><<<grid(), kRedThreads, 0, s->stream>>>((const T *)a, (const T *)b, s->n,
-                                                             s->part);
-        k_final<<<1, 256, 0, s->stream>>>(s->part, grid(), 0, mul, out);
+    void dot(const void *a, const void *b, double *out) {
+        k_dot<T><<<grid(), kRedThreads, 0, s->stream>>>((const T *)a, (const T *)b, s->n, s->part,
+                                                        s->done, out);
     }
     void absmax(const void *a, double *out) {
-        k_absmax_part<T><<<grid(), kRedThreads, 0, s->stream>>>((const T *)a, s->n, s->part);
-        k_final<<<1, 256, 0, s->stream>>>(s->part, grid(), 1, nullptr, out);
+        k_absmax<T><<<grid(), kRedThreads, 0, s->stream>>>((const T *)a, s->n, s->part, s->done,
+                                                           out);
     }
-    void axpy(void *y, const void *x, const double *a, const double *b, double sign) {
-        k_axpy_dev<T><<<grid(), kRedThreads, 0, s->stream>>>((T *)y, (const T *)x, s->n, a, b,
-                                                             sign);
+    void scale_copy(void *y, const void *x, double s0) {
+        k_scale_copy<T><<<grid(), kRedThreads, 0, s->stream>>>((T *)y, (const T *)x, s->n, s0);
     }
-    void scale_copy(void *y, const void *x, const double *num, const double *den, double s0) {
-        k_scale_copy<T><<<grid(), kRedThreads, 0, s->stream>>>((T *)y, (const T *)x, s->n, num,
-                                                               den, s0);
+    int slots() const { return s->opts.history + 1; }
+    double *gamma() const { return s->scal + SL_GAMMA; }
+    double *rho() const { return gamma() + slots(); }
+    double *alpha() const { return rho() + slots(); }
+    // d = -H g, g.d, max |d| and the first trial point xt
+    void direction(const void *x) {
+        History h;
+        h.count = s->count;
+        for (int k = 0; k < s->count; ++k) {
+            h.slot[k] = (s->head - 1 - k + slots()) % slots();
+            h.s[k] = s->S[h.slot[k]];
+            h.y[k] = s->Y[h.slot[k]];
+        }
+        const T *g = (const T *)s->g, *xp = (const T *)x;
+        T *d = (T *)s->d, *xt = (T *)s->xt;
+        constexpr int64_t per = kTlBlocks * kTlThreads;
+        if (s->n <= 16 * per) {
+            const auto kern = s->n <= 4 * per ? k_two_loop<T, 4> : k_two_loop<T, 16>;
+            kern<<<kTlBlocks, kTlThreads, 0, s->stream>>>(h, g, xp, d, xt, s->n, s->opts.max_step,
+                                                          s->scal, gamma(), rho());
+            return;
+        }
+        const int m = h.count;
+        auto step = [&](const T *in, const T *a, const double *c0, const double *c1, double sign,
+                        const double *scale, int neg, const T *b, const double *mul, double *out,
+                        double *out_max) {
+            k_two_loop_step<T><<<grid(), kRedThreads, 0, s->stream>>>(
+                d, in, a, c0, c1, sign, scale, neg, b, mul, s->n, s->part, s->done, out, out_max);
+        };
+        double *sc = s->scal;
+        if (!m) {
+            step(g, nullptr, nullptr, nullptr, 1.0, nullptr, 1, g, nullptr, sc + SL_GD,
+                 sc + SL_DMAX);
+        } else {
+            // q = g, with the newest pair's alpha; then q -= alpha y, each with the next product
+            step(g, nullptr, nullptr, nullptr, 1.0, nullptr, 0, (const T *)h.s[0],
+                 rho() + h.slot[0], alpha(), nullptr);
+            for (int k = 0; k < m; ++k) {
+                const bool last = k + 1 == m;
+                step(d, (const T *)h.y[k], alpha() + k, nullptr, -1.0,
+                     last ? gamma() + h.slot[0] : nullptr, 0,
+                     (const T *)(last ? h.y[k] : h.s[k + 1]), rho() + h.slot[last ? k : k + 1],
+                     last ? sc + SL_BETA : alpha() + k + 1, nullptr);
+            }
+            for (int k = m - 1; k >= 0; --k) {
+                // beta of the next pair goes to the other of two words: this step still reads its own
+                double *beta = sc + SL_BETA, *spare = alpha() + slots();
+                double *now = (m - 1 - k) & 1 ? spare : beta, *next = (m - 1 - k) & 1 ? beta : spare;
+                if (k)
+                    step(d, (const T *)h.s[k], alpha() + k, now, 1.0, nullptr, 0,
+                         (const T *)h.y[k - 1], rho() + h.slot[k - 1], next, nullptr);
+                else
+                    step(d, (const T *)h.s[k], alpha() + k, now, 1.0, nullptr, 1, g, nullptr,
+                         sc + SL_GD, sc + SL_DMAX);
+            }
+        }
+        k_first_trial<T><<<grid(), kRedThreads, 0, s->stream>>>(xt, xp, d, s->n, s->opts.max_step,
+                                                                sc + SL_DMAX);
+    }
+    // the trial point's candidate pair, in the free slot
+    void candidate(const void *x) {
+        const int h = s->head;
+        k_candidate<T><<<grid(), kRedThreads, 0, s->stream>>>(
+            (T *)s->S[h], (T *)s->Y[h], (const T *)s->xt, (const T *)x, (const T *)s->gt,
+            (const T *)s->g, s->n, s->part, s->done, s->scal, gamma() + h, rho() + h);
     }
     void lincomb(void *z, const void *a, const void *b, double t) {
         k_lincomb<T><<<grid(), kRedThreads, 0, s->stream>>>((T *)z, (const T *)a, (const T *)b,
@@ -266,11 +516,12 @@ fresco_status cerr(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? FRESCO_ERR_OOM : FRESCO_ERR_CUDA;
 }
 
-double host_read(fresco_lbfgs_s *s, const double *dev) {
-    double v = 0.0;
-    cudaMemcpyAsync(&v, dev, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
+// The scalars a trial leaves for the host (one copy, one wait).
+const double *read_scalars(fresco_lbfgs_s *s) {
+    cudaMemcpyAsync(s->h_scal, s->scal, sizeof(double) * SL_READ, cudaMemcpyDeviceToHost,
+                    s->stream);
     cudaStreamSynchronize(s->stream);
-    return v;
+    return s->h_scal;
 }
 
 // loss and gradient of the minimised function: the structure-factor loss, plus the pair term
@@ -294,7 +545,7 @@ fresco_status run_impl(fresco_lbfgs_s *s, void *x_caller, int64_t max_iter,
     // loss and gradient at the start point
     if (s->opts.tile_order && !s->have_order) {
         // evaluate in caller order once; its tile order becomes the solver's order
-        if ((st = evaluate(s, x_caller, s->loss_x, s->gt))) return st;
+        if ((st = evaluate(s, x_caller, sc + SL_LOSS, s->gt))) return st;
         const int64_t nt = s->plan->geom.n_tiles;
         k_tile_prefix<<<1, 1024, 0, s->stream>>>(s->plan->d_tr, nt, s->tpre);
         k_order_from_plan<T><<<pb, 256, 0, s->stream>>>(s->plan->d_sorted, s->plan->d_perm,
@@ -306,96 +557,80 @@ fresco_status run_impl(fresco_lbfgs_s *s, void *x_caller, int64_t max_iter,
     } else if (s->opts.tile_order) {
         k_permute<T><<<pb, 256, 0, s->stream>>>(s->order, np, dim, (T *)x_caller, (T *)s->xs, 1);
         x = s->xs;
-        if ((st = evaluate(s, x, s->loss_x, s->g))) return st;
+        if ((st = evaluate(s, x, sc + SL_LOSS, s->g))) return st;
     } else {
-        if ((st = evaluate(s, x, s->loss_x, s->g))) return st;
+        if ((st = evaluate(s, x, sc + SL_LOSS, s->g))) return st;
     }
     ++s->evals;
-    double fx = host_read(s, s->loss_x);
+    op.dot(s->g, s->g, sc + SL_GG);
+    const double *hs = read_scalars(s);
+    double fx = hs[SL_LOSS], gg = hs[SL_GG];
     int status = 0;
+    // One trial: the loss and gradient at xt and, ahead of the decision on it, the pair it would
+    // give, so that the host waits once per trial.
+    auto trial = [&]() -> fresco_status {
+        const fresco_status e = evaluate(s, s->xt, sc + SL_LOSS, s->gt);
+        if (e) return e;
+        op.candidate(x);
+        read_scalars(s);
+        return FRESCO_OK;
+    };
     for (int64_t it = 0; it < max_iter; ++it) {
-        op.dot(s->g, s->g, sc + SL_GG);
-        const double gg = host_read(s, sc + SL_GG);
         const double grms = std::sqrt(gg / (double)s->n);
         if (s->opts.gtol > 0.0 && grms < s->opts.gtol) { status = 1; break; }
         if (s->opts.ftol > 0.0 && fx < s->opts.ftol) { status = 2; break; }
-        // two-loop recursion: d = -H g
-        if (s->count == 0) {
-            op.scale_copy(s->d, s->g, nullptr, nullptr, -1.0);
-        } else {
-            op.scale_copy(s->d, s->g, nullptr, nullptr, 1.0);   // q = g
-            for (int k = 0; k < s->count; ++k) {     // newest to oldest
-                const int i = (s->head - 1 - k + m) % m;
-                double *a_i = sc + SL_RHO0 + m + i;  // alpha_i stored after the rho block
-                op.dot(s->S[i], s->d, a_i, sc + SL_RHO0 + i);   // alpha_i = rho_i s_i.q
-                op.axpy(s->d, s->Y[i], a_i, nullptr, -1.0);     // q -= alpha_i y_i
-            }
-            const int newest = (s->head - 1 + m) % m;
-            op.dot(s->S[newest], s->Y[newest], sc + SL_GAMMA_NUM);
-            op.dot(s->Y[newest], s->Y[newest], sc + SL_GAMMA_DEN);
-            op.scale_copy(s->d, s->d, sc + SL_GAMMA_NUM, sc + SL_GAMMA_DEN, 1.0);  // r = gamma q
-            for (int k = s->count - 1; k >= 0; --k) {    // oldest to newest
-                const int i = (s->head - 1 - k + m) % m;
-                op.dot(s->Y[i], s->d, sc + SL_BETA, sc + SL_RHO0 + i);   // beta = rho_i y_i.r
-                op.axpy(s->d, s->S[i], sc + SL_RHO0 + m + i, sc + SL_BETA, 1.0);
-            }
-            op.scale_copy(s->d, s->d, nullptr, nullptr, -1.0);   // d = -r
-        }
-        op.dot(s->g, s->d, sc + SL_GD);
-        double gd = host_read(s, sc + SL_GD);
+        op.direction(x);   // two-loop recursion, and xt at the first step length
+        if ((st = trial())) return st;
+        double gd = hs[SL_GD], dmax = hs[SL_DMAX];
         if (!(gd < 0.0)) {   // not a descent direction: restart from steepest descent
             s->count = 0;
             s->head = 0;
-            op.scale_copy(s->d, s->g, nullptr, nullptr, -1.0);
+            op.scale_copy(s->d, s->g, -1.0);
             gd = -gg;
+            op.absmax(s->d, sc + SL_DMAX);
+            dmax = read_scalars(s)[SL_DMAX];
+            if (dmax > 0.0) {
+                op.lincomb(s->xt, x, s->d, std::min(1.0, s->opts.max_step / dmax));
+                if ((st = trial())) return st;
+            }
         }
-        op.absmax(s->d, sc + SL_DMAX);
-        const double dmax = host_read(s, sc + SL_DMAX);
         if (!(dmax > 0.0)) { status = 1; break; }
         double t = std::min(1.0, s->opts.max_step / dmax);
         bool accepted = false;
         double ft = fx;
-        for (int k = 0; k <= s->opts.max_backtrack; ++k) {
-            op.lincomb(s->xt, x, s->d, t);
-            if ((st = evaluate(s, s->xt, s->loss_t, s->gt))) return st;
+        for (int k = 0;; ++k) {
             ++s->evals;
-            ft = host_read(s, s->loss_t);
+            ft = hs[SL_LOSS];
             if (std::isfinite(ft) && ft <= fx + s->opts.c1 * t * gd) {
                 accepted = true;
                 break;
             }
+            if (k == s->opts.max_backtrack) break;
             t *= 0.5;
+            op.lincomb(s->xt, x, s->d, t);
+            if ((st = trial())) return st;
         }
         if (cudaGetLastError() != cudaSuccess) return FRESCO_ERR_CUDA;
         if (!accepted) { status = 4; break; }
-        // new pair in the ring slot head: s = xt - x, y = gt - g
-        const int h = s->head;
-        op.lincomb(s->S[h], s->xt, x, -1.0);
-        op.lincomb(s->Y[h], s->gt, s->g, -1.0);
-        op.dot(s->S[h], s->Y[h], sc + SL_SY);
-        const double sy = host_read(s, sc + SL_SY);
-        if (sy > 0.0) {
-            k_set<<<1, 1, 0, s->stream>>>(sc + SL_RHO0 + h, 1.0 / sy);
-            s->head = (h + 1) % m;
+        if (hs[SL_SY] > 0.0) {   // store the candidate pair
+            s->head = (s->head + 1) % (m + 1);
             s->count = std::min(s->count + 1, m);
         } else if (s->count == m) {
-            s->count = m - 1;   // the oldest pair's slot was overwritten by the rejected one
+            s->count = m - 1;   // a rejected pair takes the place of the oldest one
         }
         // accept: x = xt, g = gt
         if (cudaMemcpyAsync(x, s->xt, s->es * (size_t)s->n, cudaMemcpyDeviceToDevice,
                             s->stream) != cudaSuccess)
             return FRESCO_ERR_CUDA;
         std::swap(s->g, s->gt);
-        std::swap(s->loss_x, s->loss_t);
         fx = ft;
+        gg = hs[SL_GG];
         ++s->iters;
         if (it + 1 == max_iter) status = 3;
     }
     if (s->opts.tile_order)   // the result back in caller order
         k_permute<T><<<pb, 256, 0, s->stream>>>(s->order, np, dim, (T *)x_caller, (T *)x, 0);
     if (rep) {
-        op.dot(s->g, s->g, sc + SL_GG);
-        const double gg = host_read(s, sc + SL_GG);
         rep->iterations = s->iters;
         rep->evaluations = s->evals;
         rep->loss = fx;
@@ -408,7 +643,8 @@ fresco_status run_impl(fresco_lbfgs_s *s, void *x_caller, int64_t max_iter,
 void lbfgs_free(fresco_lbfgs_s *s) {
     if (!s) return;
     if (s->stream) cudaStreamSynchronize(s->stream);
-    void *bufs[] = {s->g, s->d, s->xt, s->gt, s->scal, s->part, s->loss_x, s->loss_t,
+    if (s->h_scal) cudaFreeHost(s->h_scal);
+    void *bufs[] = {s->g, s->d, s->xt, s->gt, s->scal, s->part, s->done,
                     s->order, s->tpre, s->xs};
     for (void *b : bufs)
         if (b) cudaFree(b);
@@ -470,14 +706,15 @@ fresco_status fresco_lbfgs_create(fresco_lbfgs_t *out, fresco_plan_t plan,
         }
         return true;
     };
+    const size_t n_scal = SL_GAMMA + 3 * (size_t)(o.history + 1) + 1;   // (the last: a spare beta)
     bool ok = alloc(&s->g, vb) && alloc(&s->d, vb) && alloc(&s->xt, vb) && alloc(&s->gt, vb) &&
-              alloc((void **)&s->scal, sizeof(double) * (SL_RHO0 + 2 * o.history)) &&
-              alloc((void **)&s->part, sizeof(double) * kRedBlocks) &&
-              alloc((void **)&s->loss_x, sizeof(double)) &&
-              alloc((void **)&s->loss_t, sizeof(double));
-    s->S.assign(o.history, nullptr);
-    s->Y.assign(o.history, nullptr);
-    for (int i = 0; ok && i < o.history; ++i) ok = alloc(&s->S[i], vb) && alloc(&s->Y[i], vb);
+              alloc((void **)&s->scal, sizeof(double) * n_scal) &&
+              alloc((void **)&s->part, sizeof(double) * 4 * kRedBlocks) &&
+              alloc((void **)&s->done, sizeof(unsigned) * 2) &&
+              cudaMallocHost((void **)&s->h_scal, sizeof(double) * SL_READ) == cudaSuccess;
+    s->S.assign(o.history + 1, nullptr);
+    s->Y.assign(o.history + 1, nullptr);
+    for (int i = 0; ok && i <= o.history; ++i) ok = alloc(&s->S[i], vb) && alloc(&s->Y[i], vb);
     if (ok && o.tile_order)
         ok = alloc((void **)&s->order, sizeof(int) * (size_t)info.n_points) && alloc(&s->xs, vb) &&
              alloc((void **)&s->tpre, sizeof(int) * (size_t)plan->geom.n_tiles);
@@ -485,7 +722,8 @@ fresco_status fresco_lbfgs_create(fresco_lbfgs_t *out, fresco_plan_t plan,
         lbfgs_free(s);
         return FRESCO_ERR_OOM;
     }
-    cudaMemsetAsync(s->scal, 0, sizeof(double) * (SL_RHO0 + 2 * o.history), s->stream);
+    cudaMemsetAsync(s->scal, 0, sizeof(double) * n_scal, s->stream);
+    cudaMemsetAsync(s->done, 0, sizeof(unsigned) * 2, s->stream);
     *out = s;
     return FRESCO_OK;
 }
