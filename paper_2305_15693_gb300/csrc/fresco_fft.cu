@@ -1,0 +1,551 @@
+// Transforms of the FP32 fine grids, fused with the steps around them.
+//
+// With library transforms an evaluation moves the grid through memory once per step: the x pass,
+// the split into half spectra with the transpose, the y pass, the mask, the y pass back, the merge
+// and transpose, the x pass back: fourteen reads or writes of (part of) the grid and seven launches
+// and more. Here they are three kernels that read and write it once each:
+//   k_fft_rows_fwd   real rows in, the needed columns of their half spectra out, transposed;
+//   k_fft_cols       a column in; along y forward, the mask (S, loss, gradient coefficients), along
+//                    y back; a column out;
+//   k_fft_rows_inv   columns in, real rows out (k_fft_rows_inv_c: complex rows, the direct mode).
+// A block holds its rows (or its column) in shared memory and runs the passes in place
+// (fresco_fft.cuh).
+//
+// What bounds them: shared-memory passes and instruction issue at about equal parts (three or four
+// passes, each element read and written once per pass), with the global reads and writes in
+// between (fft_set_build has what they measured against cuFFT and where the line lies).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "fresco_fft.cuh"
+#include "fresco_kernels.cuh"
+
+namespace fresco {
+
+using namespace fft_detail;
+
+namespace {
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_fwd(const __grid_constant__ FftDesc f,
+                                                      const float *__restrict__ grid,
+                                                      float2 *__restrict__ xt,
+                                                      const float2 *__restrict__ tws, int64_t rows,
+                                                      int kx, int64_t grid_stride,
+                                                      int64_t xt_stride) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const int M = f.n, pitch = f.words;
+    const int64_t r0 = (int64_t)blockIdx.x * f.rows;
+    const int nr = (int)min((int64_t)f.rows, rows - r0);
+    const float2 *in =
+        reinterpret_cast<const float2 *>(grid + (int64_t)blockIdx.z * grid_stride) + r0 * M;
+    xt += (int64_t)blockIdx.z * xt_stride + r0;
+    fft_forward(f, nr, s, pitch, [&](int row, int i) { return in[(int64_t)row * M + i]; });
+    // X[k] = E + tau_k O and X[M - k] = conj(E - tau_k O) from Z[k], Z[M - k] (as k_rfft_split_cols)
+    const int half = M / 2, shift = __popc(f.rows - 1);   // f.rows is a power of two
+    for (int t = threadIdx.x; t < (half + 1) << shift; t += blockDim.x) {
+        const int row = t & (f.rows - 1), k = t >> shift;
+        const int km = M - k;
+        if (row >= nr || (k > kx && km > kx)) continue;
+        const float2 a = s[row * pitch + fft_place(f, __ldg(f.pos + k))];
+        const float2 b = s[row * pitch + fft_place(f, __ldg(f.pos + (k == 0 ? 0 : km)))];
+        const float2 w = __ldg(tws + k);
+        const float ex = 0.5f * (a.x + b.x), ey = 0.5f * (a.y - b.y);
+        const float ox = 0.5f * (a.y + b.y), oy = -0.5f * (a.x - b.x);
+        const float px = w.x * ox - w.y * oy, py = w.x * oy + w.y * ox;
+        if (k <= kx) xt[(int64_t)k * rows + row] = {ex + px, ey + py};
+        if (km > half && km <= kx) xt[(int64_t)km * rows + row] = {ex - px, -(ey - py)};
+    }
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_inv(const __grid_constant__ FftDesc f,
+                                                      const float2 *__restrict__ bt,
+                                                      float *__restrict__ grid,
+                                                      const float2 *__restrict__ tws, int64_t rows,
+                                                      int kx, int64_t bt_stride,
+                                                      int64_t grid_stride) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const int M = f.n, pitch = f.words;
+    const int64_t r0 = (int64_t)blockIdx.x * f.rows;
+    const int nr = (int)min((int64_t)f.rows, rows - r0);
+    bt += (int64_t)blockIdx.z * bt_stride + r0;
+    float2 *out = reinterpret_cast<float2 *>(grid + (int64_t)blockIdx.z * grid_stride) + r0 * M;
+    // Z[k] = P + i Q, Z[M - k] = conj P + i conj Q (as k_rfft_merge_rows), parts exchanged
+    const int half = M / 2, shift = __popc(f.rows - 1);
+    for (int t = threadIdx.x; t < (half + 1) << shift; t += blockDim.x) {
+        const int row = t & (f.rows - 1), k = t >> shift;
+        if (row >= nr) continue;
+        const int km = M - k;
+        float2 a = {0.f, 0.f}, b = {0.f, 0.f};
+        if (k <= kx) a = bt[(int64_t)k * rows + row];
+        if (km <= kx) b = bt[(int64_t)km * rows + row];
+        const float2 w = __ldg(tws + k);
+        const float px = a.x + b.x, py = a.y - b.y;
+        const float dx = a.x - b.x, dy = a.y + b.y;
+        const float qx = dx * w.x + dy * w.y, qy = dy * w.x - dx * w.y;
+        s[row * pitch + fft_place(f, __ldg(f.pos + k))] = {py + qx, px - qy};
+        if (km > half && km < M) s[row * pitch + fft_place(f, __ldg(f.pos + km))] = {-py + qx, px + qy};
+    }
+    __syncthreads();
+    fft_adjoint(f, nr, s, pitch,
+                [&](int row, int i, float2 v) { out[(int64_t)row * M + i] = {v.y, v.x}; });
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_inv_c(const __grid_constant__ FftDesc f,
+                                                        const float2 *__restrict__ bt,
+                                                        float2 *__restrict__ g, int64_t rows,
+                                                        int kx, int64_t bt_stride,
+                                                        int64_t g_stride) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const int n = f.n, pitch = f.words;
+    const int64_t r0 = (int64_t)blockIdx.x * f.rows;
+    const int nr = (int)min((int64_t)f.rows, rows - r0);
+    bt += (int64_t)blockIdx.z * bt_stride + r0;
+    g += (int64_t)blockIdx.z * g_stride + r0 * n;
+    const int shift = __popc(f.rows - 1), ncol = 2 * kx + 2;
+    for (int t = threadIdx.x; t < n << shift; t += blockDim.x) {
+        const int row = t & (f.rows - 1), x = t >> shift;
+        if (row >= nr) continue;
+        // x = n_x modulo n; n_x = c - kx - 1
+        const int c = x <= kx ? x + kx + 1 : x - (n - kx - 1);
+        float2 v = {0.f, 0.f};
+        if (c >= 0 && c < ncol) v = bt[(int64_t)c * rows + row];
+        s[row * pitch + fft_place(f, __ldg(f.pos + x))] = {v.y, v.x};
+    }
+    __syncthreads();
+    fft_adjoint(f, nr, s, pitch,
+                [&](int row, int i, float2 v) { g[(int64_t)row * n + i] = {v.y, v.x}; });
+}
+
+// One column of the 2D problem (see k_mask for the mask's arithmetic; the thread's loss terms are an
+// exact float pair). Returns the thread's loss sum.
+template <bool KD>
+__device__ __forceinline__ double cols_column(const FftDesc &f, const MaskGeom &m, int k,
+                                              const float2 *__restrict__ in, float2 *__restrict__ bt,
+                                              const int *__restrict__ rep_n,
+                                              const float *__restrict__ rep_s0,
+                                              const float *__restrict__ rep_w, int e0, int e1,
+                                              const float *__restrict__ ip0,
+                                              const float *__restrict__ ip1) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    const int n = f.n, words = f.words, nbit = (words + 31) / 32;
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    float2 *t = s + words;                                        // direct mode only
+    unsigned *bits = reinterpret_cast<unsigned *>(s + (KD ? 1 : 2) * words);
+    for (int i = threadIdx.x; i < nbit; i += blockDim.x) bits[i] = 0;
+    fft_forward(f, 1, s, 0, [&](int, int i) { return in[i]; });
+    const float inv_n = (float)m.inv_n, ipx = ip0[k];
+    float ah = 0.f, al = 0.f;
+    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+        const int ny = rep_n[2 * e + 1];
+        const int ry = ny < 0 ? ny + n : ny;
+        const int p = fft_place(f, __ldg(f.pos + ry));
+        const float2 F = s[p];
+        const float ip = ipx * ip1[ny < 0 ? -ny : ny];
+        const float re = F.x * ip, im = F.y * ip;
+        const float S = (re * re + im * im) * inv_n;
+        const float wgt = rep_w[e];
+        float dh, dl;
+        two_sum(S, -rep_s0[e], dh, dl);
+        const float pr = dh * dh;
+        const float pl = fmaf(2.f * dh, dl, fmaf(dh, dh, -pr));
+        const float th = wgt * pr;
+        const float tl = fmaf(wgt, pl, fmaf(wgt, pr, -th));
+        float sh, se;
+        two_sum(ah, th, sh, se);
+        ah = sh;
+        al += se + tl;
+        const float E = 4.f * wgt * dh * inv_n;
+        const float h = 0.5f * ip * E;
+        const float er = re * h, ei = im * h;
+        // kderiv: the scalar E / Psi with its parts exchanged; direct: kept for both columns
+        s[p] = KD ? float2{ei, er} : float2{er, ei};
+        atomicOr(&bits[p >> 5], 1u << (p & 31));
+        if (KD && k == 0) {   // the conjugate at -n, which the real inverse along x reads
+            const int p2 = fft_place(f, __ldg(f.pos + (ny > 0 ? n - ny : -ny)));
+            s[p2] = {-ei, er};
+            atomicOr(&bits[p2 >> 5], 1u << (p2 & 31));
+        }
+    }
+    __syncthreads();
+    if constexpr (KD) {
+        for (int i = threadIdx.x; i < words; i += blockDim.x)
+            if (!(bits[i >> 5] >> (i & 31) & 1)) s[i] = {0.f, 0.f};
+        __syncthreads();
+        float2 *out = bt + (int64_t)k * n;
+        fft_adjoint(f, 1, s, 0, [&](int, int i, float2 v) { out[i] = {v.y, v.x}; });
+    } else {
+        // H[n] = (a_x + i a_y) ip / 2 at n and at -n (columns n_x = k and -k)
+        const float kxs = (float)(m.kscale[0] * k);
+#pragma unroll 1
+        for (int side = 0; side < (k ? 2 : 1); ++side) {
+            for (int i = threadIdx.x; i < words; i += blockDim.x) t[i] = {0.f, 0.f};
+            __syncthreads();
+            for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+                const int ny = rep_n[2 * e + 1];
+                const int p = fft_place(f, __ldg(f.pos + (ny < 0 ? ny + n : ny)));
+                const int p2 = fft_place(f, __ldg(f.pos + (ny > 0 ? n - ny : -ny)));
+                const float er = s[p].x, ei = s[p].y, ky = (float)(m.kscale[1] * ny);
+                if (side == 0) t[p] = {er * kxs - ei * ky, -er * ky - ei * kxs};
+                if (side == 1 || k == 0) t[p2] = {-er * kxs - ei * ky, er * ky - ei * kxs};
+            }
+            __syncthreads();
+            float2 *out = bt + (int64_t)((side ? -k : k) + m.kx + 1) * n;
+            fft_adjoint(f, 1, t, 0, [&](int, int i, float2 v) { out[i] = {v.y, v.x}; });
+            __syncthreads();
+        }
+    }
+    return (double)ah + (double)al;
+}
+
+template <bool KD>
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols(const __grid_constant__ FftDesc f,
+                                                  const __grid_constant__ ColsArgs a,
+                                                  double loss_const, double *__restrict__ loss,
+                                                  unsigned *__restrict__ done) {
+    __shared__ bool s_last;
+    const int k = blockIdx.x, e0 = a.rep_first[k], e1 = a.rep_first[k + 1];
+    // (a column without representatives stays zero from plan time)
+    const double l = e0 == e1 ? 0.0
+                              : cols_column<KD>(f, a.m, k, a.xt + (int64_t)k * f.n, a.bt, a.rep_n,
+                                                a.rep_s0, a.rep_w, e0, e1, a.ip0, a.ip1);
+    const double b = block_sum(l);
+    if (threadIdx.x == 0) {
+        a.partial[k] = b;
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // the block that finishes last adds the columns' sums in a fixed order
+    double v = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(a.partial + i);
+    const double t = block_sum(v);
+    if (threadIdx.x == 0) {
+        *loss = t + loss_const;
+        *done = 0;
+    }
+}
+
+template <bool KD>
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols_b(const __grid_constant__ FftDesc f,
+                                                    const __grid_constant__ ColsBatch a) {
+    const int i = a.list[blockIdx.y], k = blockIdx.x;
+    const BInst &I = a.inst[i];
+    const int *first = a.rep_first + a.rep_off[i];
+    const int e0 = first[k], e1 = first[k + 1];
+    const double l =
+        e0 == e1 ? 0.0
+                 : cols_column<KD>(f, I.m, k, a.xt + I.ato + (int64_t)k * f.n, a.bt + I.hco,
+                                   a.rep_n + 2 * I.reo, a.rep_s0 + I.reo, a.rep_w + I.reo, e0, e1,
+                                   a.ip + I.ipo[0], a.ip + I.ipo[1]);
+    const double b = block_sum(l);
+    if (threadIdx.x == 0) a.partial[a.part_off[i] + k] = b;
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols_spec(const __grid_constant__ FftDesc f,
+                                                       const float2 *xt, float2 *out) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const float2 *in = xt + (int64_t)blockIdx.x * f.n;
+    fft_forward(f, 1, s, 0, [&](int, int i) { return in[i]; });
+    for (int i = threadIdx.x; i < f.n; i += blockDim.x)
+        out[(int64_t)blockIdx.x * f.n + i] = s[fft_place(f, __ldg(f.pos + i))];
+}
+
+}  // namespace
+
+// Radices, and the arithmetic of a butterfly with its twiddles per element (instructions, counted
+// from the code).
+constexpr int kRadix[] = {10, 9, 8, 7, 6, 5, 4, 3, 2};
+static double radix_cost(int r) {
+    switch (r) {
+        case 2: return 6.0;
+        case 3: return 12.0;
+        case 4: return 10.0;
+        case 5: return 15.0;
+        case 7: return 21.0;
+        case 8: return 14.5;
+        default: return 9.0 + 1.0 * r;
+    }
+}
+
+// Shared-memory wavefronts per element and pass, read and write, of pass p with the padding shift
+// given: the first warps' accesses (64-bit: half a warp at a time over 16 pairs of banks).
+static double pass_wavefronts(const FftDesc &f, int p, int shift) {
+    const int r = f.r[p], m = f.m[p], nb = f.n / r;
+    double waves = 0.0;
+    int groups = 0;
+    for (int i0 = 0; i0 < std::min(nb, 128); i0 += 16) {
+        int hit[16] = {}, most = 0;
+        for (int i = i0; i < std::min(nb, i0 + 16); ++i) {
+            const int a = i / m * m * r + i % m;
+            most = std::max(most, ++hit[(a + (a >> shift)) & 15]);
+        }
+        waves += most;
+        ++groups;
+    }
+    return waves / groups;
+}
+
+static void set_radices(FftDesc &f, const std::vector<int> &r) {
+    f.np = (int)r.size();
+    int len = f.n;
+    for (int p = 0; p < f.np; ++p) {
+        f.r[p] = r[(size_t)p];
+        f.m[p] = len / f.r[p];
+        len = f.m[p];
+    }
+}
+
+// The factorisation with the least arithmetic, in the order and with the padding that meet the
+// fewest bank conflicts.
+bool fft_describe(int n, FftDesc &f) {
+    f = FftDesc();
+    f.n = n;
+    if (n < 2 || sizeof(float2) * (size_t)n > kFftSmem) return false;
+    std::vector<int> best, cur;
+    double best_cost = 1e300;
+    // (descending radices: every multiset once)
+    auto search = [&](auto &&self, int rest, int from, double cost) -> void {
+        if (cost >= best_cost || (int)cur.size() > kFftMaxPasses) return;
+        if (rest == 1) {
+            best = cur;
+            best_cost = cost;
+            return;
+        }
+        for (int i = from; i < (int)(sizeof(kRadix) / sizeof(kRadix[0])); ++i)
+            if (rest % kRadix[i] == 0) {
+                cur.push_back(kRadix[i]);
+                self(self, rest / kRadix[i], i, cost + radix_cost(kRadix[i]) + 10.0);
+                cur.pop_back();
+            }
+    };
+    search(search, n, 0, 0.0);
+    if (best.empty() || (int)best.size() > kFftMaxPasses) return false;
+    std::sort(best.begin(), best.end());
+    std::vector<int> order;
+    int shift = 31;
+    double waves = 1e300;
+    int tried = 0;
+    do {
+        set_radices(f, best);
+        for (int s : {31, 4, 3, 5}) {
+            if (sizeof(float2) * (size_t)(n + (n >> s) + 1) > kFftSmem) continue;
+            double w = s == 31 ? 0.0 : 0.2 * f.np;   // (the padding's own arithmetic)
+            for (int p = 0; p < f.np; ++p) w += pass_wavefronts(f, p, s);
+            if (w < waves - 1e-9) {
+                waves = w;
+                order = best;
+                shift = s;
+            }
+        }
+    } while (std::next_permutation(best.begin(), best.end()) && ++tried < 120);
+    if (order.empty()) return false;
+    set_radices(f, order);
+    for (int p = 0; p < f.np; ++p) {
+        f.dm[p] = FastDiv(f.m[p]);
+        f.db[p] = FastDiv(n / f.r[p]);
+    }
+    f.shift = shift;
+    f.words = n + (n >> shift) + 1;
+    if (!(f.words & 1)) ++f.words;   // rows of a block start in different banks
+    return sizeof(float2) * (size_t)f.words <= kFftSmem;
+}
+
+fresco_status fft_tables(FftDesc &f, std::vector<void *> &allocs, int64_t &bytes) {
+    std::vector<float2> tw((size_t)f.n);
+    std::vector<int> pos((size_t)f.n);
+    for (int k = 0; k < f.n; ++k) {
+        const double a = 2.0 * M_PI * (double)k / (double)f.n;
+        tw[(size_t)k] = make_float2((float)std::cos(a), (float)-std::sin(a));
+        int rest = k, at = 0;
+        for (int p = 0; p < f.np; ++p) {
+            at += rest % f.r[p] * f.m[p];
+            rest /= f.r[p];
+        }
+        pos[(size_t)k] = at;
+    }
+    void *d[2] = {nullptr, nullptr};
+    const size_t b[2] = {sizeof(float2) * tw.size(), sizeof(int) * pos.size()};
+    const void *h[2] = {tw.data(), pos.data()};
+    for (int i = 0; i < 2; ++i) {
+        if (cudaMalloc(&d[i], b[i]) != cudaSuccess) {
+            cudaGetLastError();
+            return FRESCO_ERR_OOM;
+        }
+        allocs.push_back(d[i]);
+        bytes += (int64_t)b[i];
+        if (cudaMemcpy(d[i], h[i], b[i], cudaMemcpyHostToDevice) != cudaSuccess)
+            return FRESCO_ERR_CUDA;
+    }
+    f.tw = (const float2 *)d[0];
+    f.pos = (const int *)d[1];
+    return FRESCO_OK;
+}
+
+// Threads (a multiple of 32, from 64) that leave the fewest idle lanes over the passes of `rows`
+// transforms, preferring more of them where it is close: cost = passes' steps x threads.
+static int fft_threads(const FftDesc &f, int rows) {
+    int best = 64;
+    double best_cost = 1e300;
+    for (int t = 64; t <= kFftThreads; t += 32) {
+        double cost = 0.0;
+        for (int p = 0; p < f.np; ++p) {
+            const int nb = rows * (f.n / f.r[p]);
+            cost += (double)((nb + t - 1) / t) * t * f.r[p];
+        }
+        cost *= 1.0 + 0.25 * 64.0 / t;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = t;
+        }
+    }
+    return best;
+}
+
+void fft_size_rows(FftDesc &f, int64_t rows) {
+    // rows per block: up to sixteen (a column's write is then whole 32-byte sectors from four on)
+    // while kFftBlocks blocks fit an SM and every SM has two
+    f.rows = 1;
+    while (f.rows < 16 && fft_bytes(f, 2 * f.rows) * kFftBlocks <= kFftSmem &&
+           rows / (2 * f.rows) >= 2 * 152)
+        f.rows *= 2;
+    f.threads = fft_threads(f, f.rows);
+}
+
+void fft_size_cols(FftDesc &f) {
+    f.rows = 1;
+    f.threads = fft_threads(f, 1);
+}
+
+static size_t cols_bytes(const FftDesc &f, int buffers) {
+    const int words = f.words;
+    return sizeof(float2) * (size_t)buffers * words + 4 * (size_t)((words + 31) / 32);
+}
+
+cudaError_t fft_allow_smem() {
+    const int b = (int)kFftSmem;
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_fft_rows_fwd, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv_c, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols<true>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols<false>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_b<true>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_b<false>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_spec, attr, b);
+    return e;
+}
+
+bool fft_cols_fit(const FftDesc &f, bool kderiv) {
+    return cols_bytes(f, kderiv ? 1 : 2) <= kFftSmem;
+}
+
+constexpr double kOwnCells = 1.2e6;
+
+fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int count,
+                            bool ensemble) {
+    const int64_t rows = (int64_t)nf[1] * nf[2] * count;
+    // 2D single grids beyond kOwnCells stay on cuFFT, whose larger radices then outweigh its extra
+    // passes over memory; ensembles (many grids, launches per size class) and the 3D rows do not.
+    // Measured, x passes, y passes and mask, cuFFT against these kernels (us): 432^2 46 / 36, 784^2
+    // 53 / 38, 2500^2 95 / 109, 6480^2 448 / 471; ensemble of 128 410 / 318; the 324^3 grid's x
+    // passes with cuFFT's (z, y) transforms 468 / 374
+    if (dim == 2 && !ensemble && (double)nf[0] * nf[1] > kOwnCells) return FRESCO_OK;
+    // (the kernels work on whole rows of nf[0] floats; nf[0] is even)
+    f.fwd = fft_describe(nf[0] / 2, f.x);
+    f.inv = kderiv ? f.fwd : fft_describe(nf[0], f.xc);
+    f.cols = dim == 2 && f.fwd && f.inv && fft_describe(nf[1], f.y) && fft_cols_fit(f.y, kderiv);
+    if (!f.fwd && !f.inv) return FRESCO_OK;
+    if (fft_allow_smem() != cudaSuccess) return FRESCO_ERR_CUDA;
+    fresco_status st = FRESCO_OK;
+    if (f.fwd) {
+        fft_size_rows(f.x, rows);
+        st = fft_tables(f.x, f.allocs, f.bytes);
+    }
+    if (!st && f.inv && !kderiv) {
+        fft_size_rows(f.xc, rows);
+        st = fft_tables(f.xc, f.allocs, f.bytes);
+    }
+    if (!st && f.cols) {
+        fft_size_cols(f.y);
+        st = fft_tables(f.y, f.allocs, f.bytes);
+    }
+    return st;
+}
+
+void fft_set_free(FftSet *f) {
+    if (!f) return;
+    for (void *p : f->allocs) cudaFree(p);
+    delete f;
+}
+
+std::vector<int> rep_columns(const std::vector<int32_t> &rep_n, int dim, int kx) {
+    std::vector<int> first((size_t)kx + 2, 0);
+    const size_t n = rep_n.size() / (size_t)dim;
+    size_t e = 0;
+    for (int k = 0; k <= kx + 1; ++k) {
+        while (e < n && rep_n[e * (size_t)dim] < k) ++e;
+        first[(size_t)k] = (int)e;
+    }
+    return first;
+}
+
+cudaError_t fft_rows_forward(const FftDesc &f, const float *grid, float2 *xt, const float2 *tws,
+                             int64_t rows, int kx, cudaStream_t s, int batch, int64_t grid_stride,
+                             int64_t xt_stride) {
+    const dim3 g((unsigned)((rows + f.rows - 1) / f.rows), 1, (unsigned)batch);
+    k_fft_rows_fwd<<<g, f.threads, fft_bytes(f, f.rows), s>>>(f, grid, xt, tws, rows, kx,
+                                                                grid_stride, xt_stride);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_rows_inverse(const FftDesc &f, const float2 *bt, float *grid, const float2 *tws,
+                             int64_t rows, int kx, cudaStream_t s, int batch, int64_t bt_stride,
+                             int64_t grid_stride) {
+    const dim3 g((unsigned)((rows + f.rows - 1) / f.rows), 1, (unsigned)batch);
+    k_fft_rows_inv<<<g, f.threads, fft_bytes(f, f.rows), s>>>(f, bt, grid, tws, rows, kx,
+                                                                bt_stride, grid_stride);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_rows_inverse_c(const FftDesc &f, const float2 *bt, float2 *g, int64_t rows, int kx,
+                               cudaStream_t s, int batch, int64_t bt_stride, int64_t g_stride) {
+    const dim3 gr((unsigned)((rows + f.rows - 1) / f.rows), 1, (unsigned)batch);
+    k_fft_rows_inv_c<<<gr, f.threads, fft_bytes(f, f.rows), s>>>(f, bt, g, rows, kx, bt_stride,
+                                                                   g_stride);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_cols_mask(const FftDesc &f, const ColsArgs &a, double loss_const, double *loss,
+                          unsigned *done, cudaStream_t s) {
+    const unsigned cols = (unsigned)(a.m.kx + 1);
+    if (a.m.kderiv)
+        k_fft_cols<true><<<cols, f.threads, cols_bytes(f, 1), s>>>(f, a, loss_const, loss, done);
+    else
+        k_fft_cols<false><<<cols, f.threads, cols_bytes(f, 2), s>>>(f, a, loss_const, loss, done);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_cols_mask_b(const FftDesc &f, const ColsBatch &a, int count, bool kderiv,
+                            cudaStream_t s) {
+    const dim3 g((unsigned)(a.kx + 1), (unsigned)count);
+    if (kderiv) k_fft_cols_b<true><<<g, f.threads, cols_bytes(f, 1), s>>>(f, a);
+    else k_fft_cols_b<false><<<g, f.threads, cols_bytes(f, 2), s>>>(f, a);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_cols_spectrum(const FftDesc &f, const float2 *xt, float2 *out, int kx,
+                              cudaStream_t s) {
+    k_fft_cols_spec<<<(unsigned)(kx + 1), f.threads, fft_bytes(f, 1), s>>>(f, xt, out);
+    return cudaGetLastError();
+}
+
+}  // namespace fresco

@@ -1,0 +1,124 @@
+// Transforms of the FP32 fine grids fused with the steps around them (fresco_fft.cu): host side.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <vector>
+
+#include "fresco_internal.h"
+
+namespace fresco {
+
+constexpr int kFftMaxPasses = 8;
+
+// A complex transform of length n = r[0] r[1] ... r[np - 1], in place in shared memory: pass p
+// splits blocks of length m[p] r[p] into r[p] parts of m[p]. pos[k] is the place of frequency k
+// after the forward passes; tw[k] = exp(-2 pi i k / n).
+struct FftDesc {
+    int n = 0, np = 0;
+    int r[kFftMaxPasses] = {}, m[kFftMaxPasses] = {};
+    FastDiv dm[kFftMaxPasses];   // division by m[p]
+    FastDiv db[kFftMaxPasses];   // division by n / r[p], the butterflies of one transform
+    const float2 *tw = nullptr;
+    const int *pos = nullptr;
+    int shift = 31, words = 0;   // padding (fft_place), elements a padded row takes
+    int threads = 0;             // threads per block
+    int rows = 1;                // transforms per block
+};
+
+// padded place of element i (shift 31: no padding): strides that are powers of two would meet in one
+// shared-memory bank
+__host__ __device__ inline int fft_place(const FftDesc &f, int i) { return i + (i >> f.shift); }
+inline size_t fft_bytes(const FftDesc &f, int rows) {
+    return sizeof(float2) * (size_t)rows * f.words;
+}
+// Most threads of a block, and the blocks per SM the registers leave room for. The transforms wait on
+// shared-memory and global loads, so warps in flight count more than fewer passes: with radices up to
+// 20 (100 registers, two or three blocks) the x pass of 6480^2 took 141 .. 197 us and the column
+// kernel 182 .. 361 us, with radices up to 10 in 64 registers 144 and 159 us.
+constexpr int kFftThreads = 256;
+constexpr int kFftBlocks = 4;
+
+// largest length whose one transform fits a block's shared memory
+constexpr size_t kFftSmem = 224 * 1024;
+
+// Whether n factors into the radices used and fits; fills everything but the device tables.
+bool fft_describe(int n, FftDesc &f);
+// Device tables of a described transform (allocations appended to allocs)
+fresco_status fft_tables(FftDesc &f, std::vector<void *> &allocs, int64_t &bytes);
+// Transforms per block and threads for the row kernels; rows: rows of a launch
+void fft_size_rows(FftDesc &f, int64_t rows);
+// Threads for one transform per block
+void fft_size_cols(FftDesc &f);
+
+// Real rows of 2 M floats -> columns k = 0 .. kx of their half spectra, transposed: xt[k][row].
+// f: the transform of length M; tws: exp(-2 pi i k / 2M), k <= M / 2.
+cudaError_t fft_rows_forward(const FftDesc &f, const float *grid, float2 *xt, const float2 *tws,
+                             int64_t rows, int kx, cudaStream_t s, int batch = 1,
+                             int64_t grid_stride = 0, int64_t xt_stride = 0);
+// The inverse: transposed half spectra bt[k][row], k = 0 .. kx, -> real rows.
+cudaError_t fft_rows_inverse(const FftDesc &f, const float2 *bt, float *grid, const float2 *tws,
+                             int64_t rows, int kx, cudaStream_t s, int batch = 1,
+                             int64_t bt_stride = 0, int64_t grid_stride = 0);
+// Transposed columns bt[c][row], c = 0 .. 2 kx + 1 for n_x = c - kx - 1, -> complex rows of length n.
+cudaError_t fft_rows_inverse_c(const FftDesc &f, const float2 *bt, float2 *g, int64_t rows, int kx,
+                               cudaStream_t s, int batch = 1, int64_t bt_stride = 0,
+                               int64_t g_stride = 0);
+
+// 2D column pass: for every column n_x = 0 .. kx, the forward transform along y, the mask (S, loss,
+// gradient coefficients) and the inverse transform, in shared memory.
+struct ColsArgs {
+    MaskGeom m;
+    const float2 *xt;             // [kx + 1][nf1]
+    float2 *bt;                   // kderiv: [kx + 1][nf1]; direct: [2 kx + 2][nf1]
+    const int *rep_n;             // representatives, n_x major
+    const float *rep_s0, *rep_w;
+    const int *rep_first;         // [kx + 2] first representative of every column
+    const float *ip0, *ip1;
+    double *partial;              // [kx + 1] loss partials
+};
+cudaError_t fft_cols_mask(const FftDesc &f, const ColsArgs &a, double loss_const, double *loss,
+                          unsigned *done, cudaStream_t s);
+// the same over every instance of a batch class: block (column, z) works on instance inst[z]
+struct ColsBatch {
+    const BInst *inst;
+    const int *list;              // instances of the class
+    const int *rep_first;         // per instance at rep_off[i]
+    const int64_t *rep_off;
+    const float2 *xt;
+    float2 *bt;
+    const int *rep_n;
+    const float *rep_s0, *rep_w, *ip;
+    double *partial;              // instance i's columns at partial + part_off[i]
+    const int64_t *part_off;
+    int kx;
+};
+cudaError_t fft_cols_mask_b(const FftDesc &f, const ColsBatch &a, int count, bool kderiv,
+                            cudaStream_t s);
+// the column spectra themselves: out[k][row] = forward transform of xt[k] along y, in place allowed
+cudaError_t fft_cols_spectrum(const FftDesc &f, const float2 *xt, float2 *out, int kx,
+                              cudaStream_t s);
+// whether a column (with its scratch) fits a block
+bool fft_cols_fit(const FftDesc &f, bool kderiv);
+// allow the kernels their shared memory (once per process and device)
+cudaError_t fft_allow_smem();
+
+// The transforms of one fine grid: x rows as complex rows of half the length, complex rows of the
+// direct mode's inverse, and 2D columns.
+struct FftSet {
+    FftDesc x, xc, y;
+    bool fwd = false, inv = false, cols = false;   // which steps run here
+    int *rep_first = nullptr;                      // single plans, [kx + 2]
+    std::vector<void *> allocs;
+    int64_t bytes = 0;
+};
+// Chooses and builds the transforms of `count` FP32 grids (of an ensemble, or one of a single plan);
+// steps whose lengths do not fit or that cuFFT runs faster keep cuFFT.
+fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int count,
+                            bool ensemble);
+void fft_set_free(FftSet *f);
+// first[k] = index of the first representative with n_x >= k, k = 0 .. kx + 1 (rep_n is n_x major)
+std::vector<int> rep_columns(const std::vector<int32_t> &rep_n, int dim, int kx);
+
+}  // namespace fresco

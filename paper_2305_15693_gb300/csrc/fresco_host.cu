@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "fresco.h"
+#include "fresco_fft.h"
 #include "fresco_internal.h"
 
 using namespace fresco;
@@ -507,7 +508,7 @@ void release(fresco_plan_s *p) {
                     p->d_block_sums, p->d_grid, p->d_tw, p->d_specT, p->d_bt[0], p->d_bt[1],
                     p->d_hc[0], p->d_hc[1], p->d_r[0],
                     p->d_r[1], p->d_g[0], p->d_g[1], p->d_rep_n, p->d_rep_s0, p->d_rep_w,
-                    p->d_ip[0], p->d_ip[1], p->d_ip[2], p->d_partial, p->d_err,
+                    p->d_ip[0], p->d_ip[1], p->d_ip[2], p->d_partial, p->d_done, p->d_err,
                     p->d_mask_orig, p->d_fft_work, p->d_stage_pts, p->d_stage_grad,
                     p->d_stage_loss};
     for (void *b : bufs)
@@ -522,6 +523,7 @@ void release(fresco_plan_s *p) {
     for (int i = 0; i < 4; ++i)
         if (p->have_fft[i]) cufftDestroy(hs[i]);
     fresco::direct_free(p->direct);
+    fresco::fft_set_free(p->own_fft);
     p->prof.release();
     delete p;
 }
@@ -546,6 +548,8 @@ cufftType c2c_type<float>() { return CUFFT_C2C; }
 template <>
 cufftType c2c_type<double>() { return CUFFT_Z2Z; }
 
+// FP32 plans run the steps whose lengths fit in the library's own kernels (fresco_fft.cu); the rest,
+// and FP64, run on cuFFT as follows.
 // Four cuFFT plans implement the pruned d-dimensional transforms, every one a batch of
 // contiguous transforms (our kernels move the data in between):
 //   forward: each real row of length nf0 as a complex row of length nf0/2, in place on the grid;
@@ -566,13 +570,17 @@ fresco_status make_ffts(fresco_plan_s *p) {
     const long long hcw = p->mgeom.hc_row;
     size_t ws[4] = {0, 0, 0, 0};
     cufftHandle *hs[4] = {&p->fft_rows, &p->fft_cols, &p->ifft_cols, &p->ifft_rows};
+    const fresco::FftSet *own = p->own_fft;
+    const bool need[4] = {!own || !own->fwd, !own || !own->cols, !own || !own->cols,
+                          !own || !own->inv};
     for (int i = 0; i < 4; ++i) {
+        if (!need[i]) continue;
         FR_CUFFT(cufftCreate(hs[i]));
         p->have_fft[i] = true;
         FR_CUFFT(cufftSetAutoAllocation(*hs[i], 0));
     }
     const long long mh = nf0 / 2;   // the real rows run as complex rows of half the length
-    {   // rows, forward, in place on the grid
+    if (need[0]) {   // rows, forward, in place on the grid
         long long n[1] = {mh};
         FR_CUFFT(cufftMakePlanMany64(p->fft_rows, 1, n, nullptr, 1, mh, nullptr, 1, mh,
                                      c2c_type<T>(), rows, &ws[0]));
@@ -587,11 +595,14 @@ fresco_status make_ffts(fresco_plan_s *p) {
     }
     const long long plane = rows;
     // (z,)y transforms over contiguous planes of the transposed spectra
-    FR_CUFFT(cufftMakePlanMany64(p->fft_cols, crank, cn, nullptr, 1, plane, nullptr, 1, plane,
-                                 c2c_type<T>(), kx + 1, &ws[1]));
-    FR_CUFFT(cufftMakePlanMany64(p->ifft_cols, crank, cn, nullptr, 1, plane, nullptr, 1, plane,
-                                 c2c_type<T>(), hcw, &ws[2]));
-    if (p->mgeom.kderiv) {   // rows, inverse, in place on the merged half-length rows
+    if (need[1]) {
+        FR_CUFFT(cufftMakePlanMany64(p->fft_cols, crank, cn, nullptr, 1, plane, nullptr, 1, plane,
+                                     c2c_type<T>(), kx + 1, &ws[1]));
+        FR_CUFFT(cufftMakePlanMany64(p->ifft_cols, crank, cn, nullptr, 1, plane, nullptr, 1, plane,
+                                     c2c_type<T>(), hcw, &ws[2]));
+    }
+    if (!need[3]) {
+    } else if (p->mgeom.kderiv) {   // rows, inverse, in place on the merged half-length rows
         long long n[1] = {mh};
         FR_CUFFT(cufftMakePlanMany64(p->ifft_rows, 1, n, nullptr, 1, mh, nullptr, 1, mh,
                                      c2c_type<T>(), rows, &ws[3]));
@@ -604,6 +615,7 @@ fresco_status make_ffts(fresco_plan_s *p) {
     fresco_status st = dalloc(p, &p->d_fft_work, wmax);
     if (st) return st;
     for (int i = 0; i < 4; ++i) {
+        if (!need[i]) continue;
         FR_CUFFT(cufftSetWorkArea(*hs[i], p->d_fft_work));
         FR_CUFFT(cufftSetStream(*hs[i], p->stream));
     }
@@ -779,9 +791,24 @@ fresco_status build_plan(fresco_plan_s *p, const Params &P, const Folded &F) {
     if ((st = dalloc(p, &p->d_ring, sizeof(T) * (size_t)(g.n_tiles * p->ring_slot)))) return st;
     if ((st = dalloc(p, &p->d_cnt, sizeof(int) * (size_t)g.n_bins))) return st;
     if ((st = dalloc(p, &p->d_off, sizeof(int) * (size_t)(g.n_bins + 1)))) return st;
-    if ((st = dalloc(p, &p->d_block_sums, sizeof(int) * (size_t)((g.n_bins + 1023) / 1024 + 1))))
-        return st;
+    if ((st = dalloc(p, &p->d_block_sums, sizeof(int) * (size_t)kBinFinishBlocks))) return st;
+    if ((p->bin_blocks = Launch<T>::bin_finish_blocks(g)) < 1) return FRESCO_ERR_CUDA;
 
+    if (sizeof(T) == 4) {
+        p->own_fft = new (std::nothrow) fresco::FftSet();
+        if (!p->own_fft) return FRESCO_ERR_OOM;
+        fresco::FftSet &f = *p->own_fft;
+        if ((st = fresco::fft_set_build(f, P.nf, dim, m.kderiv != 0, 1, false))) return st;
+        if (f.cols) {
+            const std::vector<int> first = fresco::rep_columns(F.n, dim, m.kx);
+            if ((st = dalloc(p, &f.rep_first, sizeof(int) * first.size()))) return st;
+            f.allocs.push_back(f.rep_first);
+            FR_CUDA(cudaMemcpy(f.rep_first, first.data(), sizeof(int) * first.size(),
+                               cudaMemcpyHostToDevice));
+        }
+        p->device_bytes += f.bytes;
+    }
+    const bool own_cols = p->own_fft && p->own_fft->cols, own_inv = p->own_fft && p->own_fft->inv;
     if ((st = dalloc(p, &p->d_grid, sizeof(T) * (size_t)cells))) return st;
     {   // tau_k = exp(-2 pi i k / nf0), k = 0..nf0/4, for the real-row split and merge
         const int mh = g.nf[0] / 2;
@@ -803,19 +830,27 @@ fresco_status build_plan(fresco_plan_s *p, const Params &P, const Folded &F) {
     // (the kderiv mode's inverse runs in place in R, whose rows then hold the real field)
     const size_t g_bytes = m.kderiv ? 0 : sizeof(C2) * (size_t)cells;
     for (int q = 0; q < p->n_pipes; ++q) {
-        if ((st = dalloc(p, &p->d_hc[q], sizeof(C2) * (size_t)(rows * m.hc_row)))) return st;
-        if ((st = dalloc(p, &p->d_bt[q], sizeof(C2) * (size_t)(rows * m.hc_row)))) return st;
-        if ((st = dalloc(p, &p->d_r[q], sizeof(C2) * r_elems))) return st;
+        // (own columns write the transformed spectrum directly, own inverse rows their result)
+        const size_t spec = sizeof(C2) * (size_t)(rows * m.hc_row);
+        if (!own_cols && (st = dalloc(p, &p->d_hc[q], spec))) return st;
+        if ((st = dalloc(p, &p->d_bt[q], spec))) return st;
+        const bool need_r = m.kderiv || !own_inv;
+        if (need_r && (st = dalloc(p, &p->d_r[q], sizeof(C2) * r_elems))) return st;
         if (g_bytes && (st = dalloc(p, &p->d_g[q], g_bytes))) return st;
-        FR_CUDA(cudaMemsetAsync(p->d_hc[q], 0, sizeof(C2) * (size_t)(rows * m.hc_row), p->stream));
-        FR_CUDA(cudaMemsetAsync(p->d_r[q], 0, sizeof(C2) * r_elems, p->stream));
+        if (p->d_hc[q]) FR_CUDA(cudaMemsetAsync(p->d_hc[q], 0, spec, p->stream));
+        if (own_cols) FR_CUDA(cudaMemsetAsync(p->d_bt[q], 0, spec, p->stream));
+        if (need_r) FR_CUDA(cudaMemsetAsync(p->d_r[q], 0, sizeof(C2) * r_elems, p->stream));
     }
     const int64_t nrep = m.n_rep;
     if ((st = dalloc(p, &p->d_rep_n, sizeof(int) * (size_t)(nrep * dim)))) return st;
     if ((st = dalloc(p, &p->d_rep_s0, sizeof(T) * (size_t)nrep))) return st;
     if ((st = dalloc(p, &p->d_rep_w, sizeof(T) * (size_t)nrep))) return st;
-    p->n_mask_blocks = (int)std::max<int64_t>(1, std::min<int64_t>((nrep + 255) / 256, 152 * 8));
+    p->n_mask_blocks = own_cols
+                           ? m.kx + 1
+                           : (int)std::max<int64_t>(1, std::min<int64_t>((nrep + 255) / 256, 152 * 8));
     if ((st = dalloc(p, &p->d_partial, sizeof(double) * (size_t)p->n_mask_blocks))) return st;
+    if ((st = dalloc(p, &p->d_done, sizeof(unsigned)))) return st;
+    FR_CUDA(cudaMemsetAsync(p->d_done, 0, sizeof(unsigned), p->stream));
     if ((st = dalloc(p, &p->d_err, sizeof(int)))) return st;
     FR_CUDA(cudaMemsetAsync(p->d_err, 0, sizeof(int), p->stream));
 
@@ -855,10 +890,10 @@ template <>
 const EsPoly<double> &poly_of<double>(const fresco_plan_s *p) { return p->poly64; }
 
 // Host points into the device staging buffer, overlapped with the binning: the copy runs in
-// chunks on a second stream and the plan's stream bins each chunk as soon as it has landed (the
-// direct form places it, the compact form counts it). The slots within a tile come from atomics
-// in any case and the fixed-point spread does not depend on them, so the result is the same as
-// binning all points at once. The caller zeroes the counts (compact) or cursors (direct).
+// chunks on a second stream and the plan's stream places each chunk as soon as it has landed (plans
+// with the direct form). The slots within a tile come from atomics in any case and the fixed-point
+// spread does not depend on them, so the result is the same as binning all points at once. The
+// caller zeroes the cursors.
 template <typename T>
 fresco_status stage_and_bin(fresco_plan_s *p, const T *h_pts, T *d_pts) {
     const Geom &g = p->geom;
@@ -870,9 +905,7 @@ fresco_status stage_and_bin(fresco_plan_s *p, const T *h_pts, T *d_pts) {
         if (!e) FR_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     FR_CUDA(cudaEventRecord(p->copy_ev[kHostChunks], p->stream));
     FR_CUDA(cudaStreamWaitEvent(p->copy_stream, p->copy_ev[kHostChunks], 0));
-    // chunks start at multiples of the cursors per tile, so a point's bin (which depends on its
-    // caller index modulo g.sub) is the same whether it is counted in its chunk or placed later
-    const int64_t per = ((n + chunks - 1) / chunks + g.sub - 1) / g.sub * g.sub;
+    const int64_t per = (n + chunks - 1) / chunks;
     for (int c = 0; c < chunks; ++c) {
         const int64_t j0 = c * per, cnt = std::min(per, n - j0);
         if (cnt <= 0) break;
@@ -880,13 +913,11 @@ fresco_status stage_and_bin(fresco_plan_s *p, const T *h_pts, T *d_pts) {
                                 cudaMemcpyHostToDevice, p->copy_stream));
         FR_CUDA(cudaEventRecord(p->copy_ev[c], p->copy_stream));
         FR_CUDA(cudaStreamWaitEvent(p->stream, p->copy_ev[c], 0));
+        if (!g.tcap) continue;   // (the compact form bins all points at once)
         Geom gc = g;
         gc.n_points = cnt;
-        if (g.tcap)
-            FR_CUDA(Launch<T>::place_direct(gc, d_pts + j0 * d, j0, p->d_tcur, p->d_sorted,
-                                            p->d_perm, p->d_err, p->stream));
-        else
-            FR_CUDA(Launch<T>::count(gc, d_pts + j0 * d, p->d_cnt, p->d_err, p->stream));
+        FR_CUDA(Launch<T>::place_direct(gc, d_pts + j0 * d, j0, p->d_tcur, p->d_sorted, p->d_perm,
+                                        p->d_err, p->stream));
         p->launches += 1;
     }
     return FRESCO_OK;
@@ -900,6 +931,7 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
     const Geom &g = p->geom;
     const MaskGeom &m = p->mgeom;
     cudaStream_t s = p->stream;
+    const fresco::FftSet *own = sizeof(T) == 4 ? p->own_fft : nullptr;
     if (p->direct) {
         if (h_pts)
             FR_CUDA(cudaMemcpyAsync(const_cast<T *>(pts), h_pts,
@@ -920,14 +952,10 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
     {
         StageScope sc(p->prof, p->stream, ST_SORT);
         int nl = 0;
-        // the direct form (one pass), then the compact form: always in a plan without the direct
-        // form, else only if a tile overflowed (its kernels read the overflow word as a guard)
-        const int *guard = nullptr;
-        if (g.tcap) {
+        // the direct form (one pass); then the tiles' record ranges, after an overflow (or in a plan
+        // without the direct form) with the compact form
+        if (g.tcap)
             FR_CUDA(cudaMemsetAsync(p->d_tcur, 0, sizeof(int) * (size_t)(g.n_tiles + 1), s));
-            guard = p->d_tcur + g.n_tiles;
-        }
-        FR_CUDA(cudaMemsetAsync(p->d_cnt, 0, sizeof(int) * (size_t)g.n_bins, s));
         if (h_pts) {
             fresco_status st = stage_and_bin<T>(p, h_pts, const_cast<T *>(pts));
             if (st) return st;
@@ -936,16 +964,10 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
                                             s));
             nl += 1;
         }
-        if (!h_pts || g.tcap) {
-            FR_CUDA(Launch<T>::count(g, pts, p->d_cnt, p->d_err, s, guard));
-            nl += 1;
-        }
-        // the counts become the placement cursors (a copy of the tile offsets)
-        FR_CUDA(Launch<T>::scan(p->d_cnt, p->d_off, p->d_block_sums, g.n_bins, s, &nl, p->d_cnt,
-                                guard));
-        FR_CUDA(Launch<T>::place(g, pts, p->d_cnt, p->d_sorted, p->d_perm, s, guard));
-        FR_CUDA(Launch<T>::tile_ranges(g, g.tcap ? p->d_tcur : nullptr, p->d_off, p->d_tr, s));
-        nl += 2;
+        FR_CUDA(Launch<T>::bin_finish(g, pts, g.tcap ? p->d_tcur : nullptr, p->d_cnt, p->d_off,
+                                      p->d_block_sums, p->d_sorted, p->d_perm, p->d_tr, p->d_err,
+                                      p->bin_blocks, s));
+        nl += 1;
         p->launches += nl;
     }
     {
@@ -958,32 +980,47 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
     {
         StageScope sc(p->prof, p->stream, ST_FFT_FWD);
         const int64_t rows = m.plane;
-        if (sizeof(T) == 4)
-            FR_CUFFT(cufftExecC2C(p->fft_rows, (cufftComplex *)p->d_grid,
-                                  (cufftComplex *)p->d_grid, CUFFT_FORWARD));
-        else
-            FR_CUFFT(cufftExecZ2Z(p->fft_rows, (cufftDoubleComplex *)p->d_grid,
-                                  (cufftDoubleComplex *)p->d_grid, CUFFT_FORWARD));
-        FR_CUDA(Launch<T>::rfft_split(p->d_grid, p->d_specT, p->d_tw, rows, g.nf[0] / 2, m.kx, s));
         p->launches += 1;
-        if (sizeof(T) == 4)
+        if (own && own->fwd) {
+            FR_CUDA(fresco::fft_rows_forward(own->x, (const float *)p->d_grid, (float2 *)p->d_specT,
+                                             (const float2 *)p->d_tw, rows, m.kx, s));
+        } else {
+            if (sizeof(T) == 4)
+                FR_CUFFT(cufftExecC2C(p->fft_rows, (cufftComplex *)p->d_grid,
+                                      (cufftComplex *)p->d_grid, CUFFT_FORWARD));
+            else
+                FR_CUFFT(cufftExecZ2Z(p->fft_rows, (cufftDoubleComplex *)p->d_grid,
+                                      (cufftDoubleComplex *)p->d_grid, CUFFT_FORWARD));
+            FR_CUDA(Launch<T>::rfft_split(p->d_grid, p->d_specT, p->d_tw, rows, g.nf[0] / 2, m.kx,
+                                          s));
+        }
+        if (own && own->cols) {
+        } else if (sizeof(T) == 4) {
             FR_CUFFT(cufftExecC2C(p->fft_cols, (cufftComplex *)p->d_specT,
                                   (cufftComplex *)p->d_specT, CUFFT_FORWARD));
-        else
+        } else {
             FR_CUFFT(cufftExecZ2Z(p->fft_cols, (cufftDoubleComplex *)p->d_specT,
                                   (cufftDoubleComplex *)p->d_specT, CUFFT_FORWARD));
+        }
+    }
+    if (own && own->cols) {
+        // the y pass, the mask with its loss and the y pass back, column by column
+        StageScope sc(p->prof, p->stream, ST_MASK);
+        fresco::ColsArgs a{m, (const float2 *)p->d_specT, (float2 *)p->d_bt[0], p->d_rep_n,
+                           (const float *)p->d_rep_s0, (const float *)p->d_rep_w, own->rep_first,
+                           (const float *)p->d_ip[0], (const float *)p->d_ip[1], p->d_partial};
+        FR_CUDA(fresco::fft_cols_mask(own->y, a, p->info.loss_const, loss, p->d_done, s));
+        p->launches += 1;
+        p->spec_ready = false;
+        p->forward_done = true;
+        return FRESCO_OK;
     }
     {
         StageScope sc(p->prof, p->stream, ST_MASK);
         FR_CUDA(Launch<T>::mask(m, p->d_rep_n, (const T *)p->d_rep_s0, (const T *)p->d_rep_w,
                                 p->d_specT, (const T *)p->d_ip[0], (const T *)p->d_ip[1],
                                 (const T *)p->d_ip[2], p->d_hc[0], p->d_hc[1], p->d_partial,
-                                p->n_mask_blocks, s));
-        p->launches += 1;
-    }
-    {
-        StageScope sc(p->prof, p->stream, ST_LOSS);
-        FR_CUDA(Launch<T>::finalize(p->d_partial, p->n_mask_blocks, p->info.loss_const, loss, s));
+                                p->n_mask_blocks, p->d_done, p->info.loss_const, loss, s));
         p->launches += 1;
     }
     (void)sizeof(C2);
@@ -996,6 +1033,7 @@ fresco_status backward_impl(fresco_plan_s *p, const double *grad_out, T *grad) {
     const Geom &g = p->geom;
     const MaskGeom &m = p->mgeom;
     cudaStream_t s = p->stream;
+    const fresco::FftSet *own = sizeof(T) == 4 ? p->own_fft : nullptr;
     if (p->direct) {
         StageScope sc(p->prof, s, ST_INTERP);
         FR_CUDA(fresco::direct_grad<T>(p->direct, grad_out, grad, s));
@@ -1005,21 +1043,29 @@ fresco_status backward_impl(fresco_plan_s *p, const double *grad_out, T *grad) {
     if (m.kderiv) {
         {
             StageScope sc(p->prof, p->stream, ST_FFT_INV);
-            if (sizeof(T) == 4)
+            if (own && own->cols) {
+            } else if (sizeof(T) == 4) {
                 FR_CUFFT(cufftExecC2C(p->ifft_cols, (cufftComplex *)p->d_hc[0],
                                       (cufftComplex *)p->d_bt[0], CUFFT_INVERSE));
-            else
+            } else {
                 FR_CUFFT(cufftExecZ2Z(p->ifft_cols, (cufftDoubleComplex *)p->d_hc[0],
                                       (cufftDoubleComplex *)p->d_bt[0], CUFFT_INVERSE));
-            FR_CUDA(Launch<T>::rfft_merge(p->d_bt[0], p->d_r[0], p->d_tw, m.plane, g.nf[0] / 2,
-                                          m.kx, s));
+            }
             p->launches += 1;
-            if (sizeof(T) == 4)
-                FR_CUFFT(cufftExecC2C(p->ifft_rows, (cufftComplex *)p->d_r[0],
-                                      (cufftComplex *)p->d_r[0], CUFFT_INVERSE));
-            else
-                FR_CUFFT(cufftExecZ2Z(p->ifft_rows, (cufftDoubleComplex *)p->d_r[0],
-                                      (cufftDoubleComplex *)p->d_r[0], CUFFT_INVERSE));
+            if (own && own->inv) {
+                FR_CUDA(fresco::fft_rows_inverse(own->x, (const float2 *)p->d_bt[0],
+                                                 (float *)p->d_r[0], (const float2 *)p->d_tw,
+                                                 m.plane, m.kx, s));
+            } else {
+                FR_CUDA(Launch<T>::rfft_merge(p->d_bt[0], p->d_r[0], p->d_tw, m.plane, g.nf[0] / 2,
+                                              m.kx, s));
+                if (sizeof(T) == 4)
+                    FR_CUFFT(cufftExecC2C(p->ifft_rows, (cufftComplex *)p->d_r[0],
+                                          (cufftComplex *)p->d_r[0], CUFFT_INVERSE));
+                else
+                    FR_CUFFT(cufftExecZ2Z(p->ifft_rows, (cufftDoubleComplex *)p->d_r[0],
+                                          (cufftDoubleComplex *)p->d_r[0], CUFFT_INVERSE));
+            }
         }
         StageScope sc(p->prof, p->stream, ST_INTERP);
         FR_CUDA(Launch<T>::interp_kd(g, poly_of<T>(p), p->d_sorted, p->d_perm, p->d_tr,
@@ -1031,14 +1077,21 @@ fresco_status backward_impl(fresco_plan_s *p, const double *grad_out, T *grad) {
     {
         StageScope sc(p->prof, p->stream, ST_FFT_INV);
         for (int q = 0; q < p->n_pipes; ++q) {
-            if (sizeof(T) == 4)
+            if (own && own->cols) {
+            } else if (sizeof(T) == 4) {
                 FR_CUFFT(cufftExecC2C(p->ifft_cols, (cufftComplex *)p->d_hc[q],
                                       (cufftComplex *)p->d_bt[q], CUFFT_INVERSE));
-            else
+            } else {
                 FR_CUFFT(cufftExecZ2Z(p->ifft_cols, (cufftDoubleComplex *)p->d_hc[q],
                                       (cufftDoubleComplex *)p->d_bt[q], CUFFT_INVERSE));
-            FR_CUDA(Launch<T>::rows_to_cols(p->d_bt[q], p->d_r[q], m.plane, g.nf[0], m.kx, s));
+            }
             p->launches += 1;
+            if (own && own->inv) {
+                FR_CUDA(fresco::fft_rows_inverse_c(own->xc, (const float2 *)p->d_bt[q],
+                                                   (float2 *)p->d_g[q], m.plane, m.kx, s));
+                continue;
+            }
+            FR_CUDA(Launch<T>::rows_to_cols(p->d_bt[q], p->d_r[q], m.plane, g.nf[0], m.kx, s));
             if (sizeof(T) == 4)
                 FR_CUFFT(cufftExecC2C(p->ifft_rows, (cufftComplex *)p->d_r[q],
                                       (cufftComplex *)p->d_g[q], CUFFT_INVERSE));
@@ -1159,17 +1212,24 @@ fresco_status fresco::point_side_build(PointSide &ps, int dim, const int nf[3], 
     g.n_bins = g.n_tiles * g.sub;
     g.n_points = n_points;
     g.beta = beta;
+    g.tcap = direct_tile_capacity(g);
     set_tile_divisors(g);
     ps.precision = precision;
     const int64_t cells = (int64_t)g.nf[0] * g.nf[1] * g.nf[2];
     const int pw = es == 4 ? 4 : (dim == 3 ? 4 : 2);
     ps.ring_slot = es == 8 ? Launch<double>::ring_slot(g) : Launch<float>::ring_slot(g);
-    bool ok = ps_alloc(ps, &ps.sorted, es * (size_t)n_points * pw) &&
-              (es == 4 || ps_alloc(ps, (void **)&ps.perm, sizeof(int) * (size_t)n_points)) &&
+    const int64_t slots = std::max<int64_t>(n_points, (int64_t)g.tcap * g.n_tiles);
+    ps.bin_blocks =
+        es == 8 ? Launch<double>::bin_finish_blocks(g) : Launch<float>::bin_finish_blocks(g);
+    if (ps.bin_blocks < 1) return FRESCO_ERR_CUDA;
+    bool ok = ps_alloc(ps, &ps.sorted, es * (size_t)slots * pw) &&
+              (es == 4 || ps_alloc(ps, (void **)&ps.perm, sizeof(int) * (size_t)slots)) &&
+              (!g.tcap ||
+               ps_alloc(ps, (void **)&ps.tcur, sizeof(int) * (size_t)(g.n_tiles + 1))) &&
               ps_alloc(ps, (void **)&ps.cnt, sizeof(int) * (size_t)g.n_bins) &&
               ps_alloc(ps, (void **)&ps.off, sizeof(int) * (size_t)(g.n_bins + 1)) &&
               ps_alloc(ps, (void **)&ps.tr, sizeof(int2) * (size_t)g.n_tiles) &&
-              ps_alloc(ps, (void **)&ps.bsum, sizeof(int) * (size_t)((g.n_bins + 1023) / 1024 + 1)) &&
+              ps_alloc(ps, (void **)&ps.bsum, sizeof(int) * (size_t)kBinFinishBlocks) &&
               ps_alloc(ps, (void **)&ps.err, sizeof(int)) &&
               ps_alloc(ps, &ps.grid, es * (size_t)cells) &&
               ps_alloc(ps, &ps.ring, es * (size_t)(g.n_tiles * ps.ring_slot));
@@ -1185,13 +1245,14 @@ template <typename T>
 fresco_status fresco::point_side_spread(PointSide &ps, const T *pts, cudaStream_t s,
                                         int64_t *launches) {
     const Geom &g = ps.g;
-    FR_CUDA(cudaMemsetAsync(ps.cnt, 0, sizeof(int) * (size_t)g.n_bins, s));
-    FR_CUDA(Launch<T>::count(g, pts, ps.cnt, ps.err, s));
     int nl = 1;
-    FR_CUDA(Launch<T>::scan(ps.cnt, ps.off, ps.bsum, g.n_bins, s, &nl, ps.cnt));
-    FR_CUDA(Launch<T>::place(g, pts, ps.cnt, ps.sorted, ps.perm, s));
-    FR_CUDA(Launch<T>::tile_ranges(g, nullptr, ps.off, ps.tr, s));
-    nl += 2;
+    if (g.tcap) {
+        FR_CUDA(cudaMemsetAsync(ps.tcur, 0, sizeof(int) * (size_t)(g.n_tiles + 1), s));
+        FR_CUDA(Launch<T>::place_direct(g, pts, 0, ps.tcur, ps.sorted, ps.perm, ps.err, s));
+        nl += 1;
+    }
+    FR_CUDA(Launch<T>::bin_finish(g, pts, ps.tcur, ps.cnt, ps.off, ps.bsum, ps.sorted, ps.perm,
+                                  ps.tr, ps.err, ps.bin_blocks, s));
     const EsPoly<T> &ep = *reinterpret_cast<const EsPoly<T> *>(sizeof(T) == 4 ? (const void *)&ps.p32
                                                                               : (const void *)&ps.p64);
     FR_CUDA(Launch<T>::spread_own(g, ep, ps.sorted, ps.tr, (T *)ps.grid, (T *)ps.ring,
@@ -1395,6 +1456,13 @@ fresco_status fresco_get_rho_S(fresco_plan_t p, void *d_rho, void *d_S) {
                 ? fresco::direct_rho_s<double>(p->direct, (double *)d_rho, (double *)d_S, p->stream)
                 : fresco::direct_rho_s<float>(p->direct, (float *)d_rho, (float *)d_S, p->stream));
     }
+    if (p->own_fft && p->own_fft->cols && !p->spec_ready) {
+        // the column kernel keeps its spectra on chip: transform the columns here, once per forward
+        FR_CUDA(fresco::fft_cols_spectrum(p->own_fft->y, (const float2 *)p->d_specT,
+                                          (float2 *)p->d_specT, p->mgeom.kx, p->stream));
+        p->spec_ready = true;
+        p->launches += 1;
+    }
     if (!p->d_mask_orig) {
         fresco_status st = dalloc(p, &p->d_mask_orig, sizeof(int) * p->h_mask.size());
         if (st) return st;
@@ -1502,9 +1570,11 @@ void batch_free(fresco_batch_s *b) {
     else cudaDeviceSynchronize();
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->graph) cudaGraphDestroy(b->graph);
-    for (auto &c : b->cls)
+    for (auto &c : b->cls) {
         for (int i = 0; i < 4; ++i)
             if (c.have[i]) cufftDestroy(c.h[i]);
+        fresco::fft_set_free(c.own);
+    }
     for (void *p : b->allocs) cudaFree(p);
     b->prof.release();
     delete b;
@@ -1572,6 +1642,21 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
         reo += nrep;
         I.loss_const = F[i].loss_const;
     }
+    // FP32 ensembles whose every size class fits run the library's own transforms; an instance's loss
+    // partials are then one per column of its class
+    b->own_fft = sizeof(T) == 4;
+    for (auto &K : b->cls) {
+        if (!b->own_fft) break;
+        K.own = new (std::nothrow) fresco::FftSet();
+        if (!K.own) return FRESCO_ERR_OOM;
+        const int nf[3] = {K.nf[0], K.nf[1], 1};
+        const fresco_status st = fresco::fft_set_build(*K.own, nf, 2, b->kderiv != 0, K.count, true);
+        if (st) return st;
+        b->own_fft = K.own->cols;
+    }
+    if (b->own_fft)
+        for (int i = 0; i < n; ++i)
+            b->mblk_first[i + 1] = b->mblk_first[i] + b->cls[cls_of[i]].kx + 1;
     b->n_points = b->pt_first[n];
     b->n_bins = bo;
     b->n_rep = reo;
@@ -1669,8 +1754,9 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
               balloc(b, &b->grid, sizeof(T) * b->cells) &&
               balloc(b, &b->tw, sizeof(C2) * b->n_tw) &&
               balloc(b, &b->specT, sizeof(C2) * b->n_specT) &&
-              balloc(b, &b->hc, sizeof(C2) * b->n_hc) && balloc(b, &b->bt, sizeof(C2) * b->n_hc) &&
-              (b->kderiv || balloc(b, &b->r, sizeof(C2) * b->n_r)) &&
+              (b->own_fft || balloc(b, &b->hc, sizeof(C2) * b->n_hc)) &&
+              balloc(b, &b->bt, sizeof(C2) * b->n_hc) &&
+              (b->kderiv || b->own_fft || balloc(b, &b->r, sizeof(C2) * b->n_r)) &&
               (b->kderiv || balloc(b, &b->g, sizeof(C2) * b->cells)) &&
               balloc(b, (void **)&b->rep_n, sizeof(int) * b->n_rep * dim) &&
               balloc(b, &b->rep_s0, sizeof(T) * b->n_rep) &&
@@ -1704,7 +1790,32 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
                            cudaMemcpyHostToDevice));
         FR_CUDA(cudaMemcpy(b->d_mblk_first, b->mblk_first.data(), sizeof(int64_t) * (n + 1),
                            cudaMemcpyHostToDevice));
-        FR_CUDA(cudaMemset(b->hc, 0, sizeof(C2) * b->n_hc));
+        if (b->hc) FR_CUDA(cudaMemset(b->hc, 0, sizeof(C2) * b->n_hc));
+        if (b->own_fft) {
+            FR_CUDA(cudaMemset(b->bt, 0, sizeof(C2) * b->n_hc));
+            std::vector<int> list, first;
+            std::vector<int64_t> off((size_t)n, 0);
+            for (size_t c = 0; c < b->cls.size(); ++c) {
+                b->cls[c].list0 = (int)list.size();
+                for (int i = 0; i < n; ++i)
+                    if (cls_of[i] == (int)c) list.push_back(i);
+            }
+            for (int i = 0; i < n; ++i) {
+                off[(size_t)i] = (int64_t)first.size();
+                const std::vector<int> f = fresco::rep_columns(F[i].n, dim, b->cls[cls_of[i]].kx);
+                first.insert(first.end(), f.begin(), f.end());
+            }
+            if (!balloc(b, (void **)&b->cls_list, sizeof(int) * list.size()) ||
+                !balloc(b, (void **)&b->rep_first, sizeof(int) * first.size()) ||
+                !balloc(b, (void **)&b->rep_off, sizeof(int64_t) * off.size()))
+                return FRESCO_ERR_OOM;
+            FR_CUDA(cudaMemcpy(b->cls_list, list.data(), sizeof(int) * list.size(),
+                               cudaMemcpyHostToDevice));
+            FR_CUDA(cudaMemcpy(b->rep_first, first.data(), sizeof(int) * first.size(),
+                               cudaMemcpyHostToDevice));
+            FR_CUDA(cudaMemcpy(b->rep_off, off.data(), sizeof(int64_t) * off.size(),
+                               cudaMemcpyHostToDevice));
+        }
         if (b->r) FR_CUDA(cudaMemset(b->r, 0, sizeof(C2) * b->n_r));
         std::vector<C2> tw((size_t)b->n_tw);
         for (auto &K : b->cls)
@@ -1746,6 +1857,10 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
     // ---- cuFFT plans per class (all transforms of a class in one batch)
     size_t wmax = 0;
     for (auto &K : b->cls) {
+        if (b->own_fft) {
+            b->device_bytes += K.own->bytes;
+            continue;
+        }
         size_t ws = 0;
         for (int i = 0; i < 4; ++i) {
             FR_CUFFT(cufftCreate(&K.h[i]));
@@ -1774,7 +1889,7 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
     }
     if (!balloc(b, &b->work, wmax)) return FRESCO_ERR_OOM;
     for (auto &K : b->cls)
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 4 && !b->own_fft; ++i) {
             FR_CUFFT(cufftSetWorkArea(K.h[i], b->work));
             FR_CUFFT(cufftSetStream(K.h[i], b->stream));
         }
@@ -1814,6 +1929,13 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
             const int64_t plane = K.nf[1];
             const int mh = K.nf[0] / 2;
             C2 *A = (C2 *)((T *)b->grid + K.go0), *AT = (C2 *)b->specT + K.ato0;
+            if (b->own_fft) {
+                FR_CUDA(fresco::fft_rows_forward(K.own->x, (const float *)A, (float2 *)AT,
+                                                 (const float2 *)b->tw + K.two0, plane, K.kx, s,
+                                                 K.count, 2 * plane * mh, plane * (K.kx + 1)));
+                b->launches += 1;
+                continue;
+            }
             if (sizeof(T) == 4)
                 FR_CUFFT(cufftExecC2C(K.h[0], (cufftComplex *)A, (cufftComplex *)A,
                                       CUFFT_FORWARD));
@@ -1833,9 +1955,20 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
     }
     {
         StageScope sc(b->prof, s, ST_MASK);
-        FR_CUDA(Launch<T>::mask_b(t, b->rep_n, (const T *)b->rep_s0, (const T *)b->rep_w,
-                                  b->specT, (const T *)b->ip, b->hc, nullptr, b->partial, s));
-        b->launches += 1;
+        if (b->own_fft) {
+            for (auto &K : b->cls) {   // the y pass, the mask and the y pass back, column by column
+                fresco::ColsBatch a{b->d_inst, b->cls_list + K.list0, b->rep_first, b->rep_off,
+                                    (const float2 *)b->specT, (float2 *)b->bt, b->rep_n,
+                                    (const float *)b->rep_s0, (const float *)b->rep_w,
+                                    (const float *)b->ip, b->partial, b->d_mblk_first, K.kx};
+                FR_CUDA(fresco::fft_cols_mask_b(K.own->y, a, K.count, b->kderiv != 0, s));
+                b->launches += 1;
+            }
+        } else {
+            FR_CUDA(Launch<T>::mask_b(t, b->rep_n, (const T *)b->rep_s0, (const T *)b->rep_w,
+                                      b->specT, (const T *)b->ip, b->hc, nullptr, b->partial, s));
+            b->launches += 1;
+        }
     }
     {
         StageScope sc(b->prof, s, ST_LOSS);
@@ -1851,6 +1984,13 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
                 const int mh = K.nf[0] / 2;
                 C2 *H = (C2 *)b->hc + K.hco0, *BT = (C2 *)b->bt + K.hco0;
                 C2 *Z = (C2 *)((T *)b->grid + K.go0);
+                if (b->own_fft) {
+                    FR_CUDA(fresco::fft_rows_inverse(
+                        K.own->x, (const float2 *)BT, (float *)Z, (const float2 *)b->tw + K.two0,
+                        plane, K.kx, s, K.count, plane * ((int64_t)K.kx + 1), 2 * plane * mh));
+                    b->launches += 1;
+                    continue;
+                }
                 if (sizeof(T) == 4)
                     FR_CUFFT(cufftExecC2C(K.h[2], (cufftComplex *)H, (cufftComplex *)BT,
                                           CUFFT_INVERSE));
@@ -1880,6 +2020,13 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
             const int64_t plane = K.nf[1];
             C2 *H = (C2 *)b->hc + K.hco0, *BT = (C2 *)b->bt + K.hco0, *R = (C2 *)b->r + K.ro0;
             C2 *G = (C2 *)b->g + K.ro0;
+            if (b->own_fft) {
+                FR_CUDA(fresco::fft_rows_inverse_c(
+                    K.own->xc, (const float2 *)BT, (float2 *)G, plane, K.kx, s, K.count,
+                    plane * (2 * (int64_t)K.kx + 2), (int64_t)K.nf[0] * plane));
+                b->launches += 1;
+                continue;
+            }
             if (sizeof(T) == 4)
                 FR_CUFFT(cufftExecC2C(K.h[2], (cufftComplex *)H, (cufftComplex *)BT,
                                       CUFFT_INVERSE));

@@ -20,6 +20,7 @@ constexpr int kTileCursors = 4;   // placement cursors per tile of a single plan
 constexpr int kZSegmentMax = 16;  // 3D single plans: most tiles per z-column segment (Geom.zseg)
 constexpr int kColMaxPlanes = 64; // column spread: tiles with tmax_z + w above this spread one by one
 constexpr int kDirectPointsPerThread = 8;   // points in flight per thread of k_place_direct
+constexpr int kBinFinishBlocks = 1024;      // most blocks of k_bin_finish
 // fresco_loss_grad_host copies the points in up to kHostChunks pieces of at least
 // kHostChunkBytes, binning each piece while the next one is in flight
 constexpr int kHostChunks = 8;
@@ -110,6 +111,11 @@ __host__ __device__ inline int tile_of_cell(int c, int q, int r, float inv) {
     while (b > 0 && tile_start(b, q, r) > c) --b;
     while (tile_start(b + 1, q, r) <= c) ++b;
     return b;
+}
+
+// Whether the 2D rings fold in one gathering launch (k_halo_gather, which has the reason).
+inline bool fold_gathers(const Geom &g) {
+    return g.dim == 2 && g.tq[0] >= g.width && g.tq[1] >= g.width && g.n_tiles <= 152 * 8;
 }
 
 // Geometry of the mask and the spectra.
@@ -215,26 +221,21 @@ struct StageScope {
 // return the cudaError_t of the launch. Element layouts are documented in fresco_kernels.cuh.
 template <typename T>
 struct Launch {
-    // exclusive prefix sum of cnt into off[0..n] (off[n] = total); when cur is not null it
-    // receives a copy of off[0..n) (the placement cursors of k_place)
-    // (with a guard, not null: the passes do nothing unless *guard != 0)
+    // exclusive prefix sum of cnt into off[0..n] (off[n] = total)
     static cudaError_t scan(const int *cnt, int *off, int *block_sums, int64_t n, cudaStream_t s,
-                            int *launches, int *cur = nullptr, const int *guard = nullptr);
-    // single plans (tiles without border sub-bins), compact form: points per bin, then placement
-    // by cursor (guard as for scan)
-    static cudaError_t count(const Geom &g, const T *points, int *cnt, int *err, cudaStream_t s,
-                             const int *guard = nullptr);
-    static cudaError_t place(const Geom &g, const T *points, int *cur, void *sorted, int *perm,
-                             cudaStream_t s, const int *guard = nullptr);
+                            int *launches);
     // direct form: g.n_points points starting at caller index j0 (points points at that point)
     // into tile slots of capacity g.tcap; tcur [n_tiles + 1] zero before the first chunk, its
     // last entry the overflow word
     static cudaError_t place_direct(const Geom &g, const T *points, int64_t j0, int *tcur,
                                     void *sorted, int *perm, int *err, cudaStream_t s);
-    // tr[t] = record range of tile t from the direct form (tcur) unless it overflowed or tcur is
-    // null, else from the compact offsets off
-    static cudaError_t tile_ranges(const Geom &g, const int *tcur, const int *off, int2 *tr,
-                                   cudaStream_t s);
+    // tr[t] = record range of tile t from the direct form (tcur); if a tile overflowed, or tcur is
+    // null, the points are first binned in the compact form (cnt, off, bsum: its work arrays, bsum
+    // of kBinFinishBlocks entries). A cooperative launch of `blocks` blocks, bin_finish_blocks(g)
+    static cudaError_t bin_finish(const Geom &g, const T *points, const int *tcur, int *cnt,
+                                  int *off, int *bsum, void *sorted, int *perm, int2 *tr, int *err,
+                                  int blocks, cudaStream_t s);
+    static int bin_finish_blocks(const Geom &g);
     // own-points spread into the grid plus per-tile rings, then the ring sums into the grid
     static cudaError_t spread_own(const Geom &g, const EsPoly<T> &ep, const void *sorted,
                                   const int2 *tr, T *grid, T *ring, int64_t ring_slot,
@@ -244,9 +245,8 @@ struct Launch {
 
     static cudaError_t mask(const MaskGeom &m, const int *rep_n, const T *rep_s0, const T *rep_w,
                             const void *spec, const T *ip0, const T *ip1, const T *ip2,
-                            void *hc0, void *hc1, double *partial, int n_blocks, cudaStream_t s);
-    static cudaError_t finalize(const double *partial, int n_blocks, double loss_const,
-                                double *loss, cudaStream_t s);
+                            void *hc0, void *hc1, double *partial, int n_blocks, unsigned *done,
+                            double loss_const, double *loss, cudaStream_t s);
     static cudaError_t interp(const Geom &g, const EsPoly<T> &ep, const void *sorted,
                               const int *perm, const int2 *tr, const void *g0, const void *g1,
                               const double *grad_out, T *grad, cudaStream_t s);
@@ -314,7 +314,9 @@ struct PointSide {
     int precision = FRESCO_F32;
     void *sorted = nullptr;
     int *perm = nullptr, *cnt = nullptr, *off = nullptr, *bsum = nullptr, *err = nullptr;
-    int2 *tr = nullptr;   // record range of every tile (compact binning only: Geom.tcap = 0)
+    int *tcur = nullptr;  // direct-form cursors, then the overflow word (null: Geom.tcap = 0)
+    int bin_blocks = 1;
+    int2 *tr = nullptr;   // record range of every tile
     void *grid = nullptr, *ring = nullptr;
     int64_t ring_slot = 0;
     int64_t device_bytes = 0;
@@ -340,6 +342,7 @@ void es_poly_table(int w, double beta, EsPoly<double> &out);
 // Direct sums for small plans (fresco_direct.cu). direct_wanted: the plan's options leave the choice
 // to the library; direct_build leaves *out null where the problem is large enough for the NUFFT.
 struct DirectPlan;
+struct FftSet;   // fresco_fft.h
 bool direct_wanted(int64_t n_points, const fresco_opts &o, int precision, double tol);
 fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const double *box,
                            int precision, const int32_t *mask, int64_t n_k,
@@ -421,7 +424,8 @@ struct fresco_plan_s {
     int *d_tcur = nullptr;           // [n_tiles + 1] direct-form cursors, then the overflow word
     int2 *d_tr = nullptr;            // [n_tiles] record range of every tile
     CUtensorMap tmap{};              // geom.tma: the interpolated real field as a TMA tensor
-    int *d_block_sums = nullptr;     // scan scratch
+    int *d_block_sums = nullptr;     // [kBinFinishBlocks] scan scratch
+    int bin_blocks = 1;              // blocks of k_bin_finish
     void *d_grid = nullptr;          // real fine grid (spread output)
     void *d_tw = nullptr;            // exp(-2 pi i k / nf0), k = 0..nf0/4 (real-row split/merge)
     void *d_specT = nullptr;         // its columns x = 0..kx transposed: [kx+1][plane]
@@ -434,6 +438,7 @@ struct fresco_plan_s {
     void *d_rep_w = nullptr;         // [n_rep] folded W'
     void *d_ip[3] = {nullptr, nullptr, nullptr};  // 1 / Psi_a(nu), nu = 0..k_max[a]
     double *d_partial = nullptr;     // per-block loss partial sums
+    unsigned *d_done = nullptr;      // blocks of the mask kernel that have finished
     int *d_err = nullptr;            // device error word
     int *d_mask_orig = nullptr;      // lazily uploaded mask (fresco_get_rho_S)
     void *d_fft_work = nullptr;
@@ -456,6 +461,8 @@ struct fresco_plan_s {
     cufftHandle ifft_rows = 0;       // C2C inverse along x, all rows (kderiv: nf0/2, in place)
     bool have_fft[4] = {false, false, false, false};
 
+    fresco::FftSet *own_fft = nullptr;      // FP32 plans: the library's own transforms
+    bool spec_ready = false;                // d_specT holds the transformed columns (own_fft->cols)
     fresco::DirectPlan *direct = nullptr;   // small problems: direct sums, none of the above
     fresco::StageProfile prof;
     int64_t launches = 0;
@@ -471,6 +478,8 @@ struct fresco_batch_s {
         int64_t go0 = 0, ato0 = 0, hco0 = 0, ro0 = 0, two0 = 0;
         cufftHandle h[4] = {0, 0, 0, 0};   // rows fwd, cols fwd, cols inv, rows inv
         bool have[4] = {false, false, false, false};
+        fresco::FftSet *own = nullptr;     // FP32: the library's own transforms instead
+        int list0 = 0;                     // first entry of the class in cls_list
     };
     int dim = 0;
     int precision = FRESCO_F32;
@@ -508,4 +517,8 @@ struct fresco_batch_s {
     fresco::StageProfile prof;
     int kderiv = 0;                  // gradient mode FRESCO_GRAD_KDERIV
     int64_t n_r = 0;                 // complex elements of the row-order backward buffer
+    bool own_fft = false;            // every class runs the library's own transforms
+    int *cls_list = nullptr;         // instances, class by class
+    int *rep_first = nullptr;        // per instance, first representative of every column
+    int64_t *rep_off = nullptr;      // per instance, its part of rep_first
 };

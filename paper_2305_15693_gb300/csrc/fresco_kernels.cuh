@@ -229,13 +229,11 @@ __device__ __forceinline__ int strip_part(int rel, int wd, int w, int strips) {
     return 1;
 }
 
-// K1b: exclusive prefix sum of the tile counts, in three passes over blocks of 1024. With a guard
-// (not null) the passes do nothing unless *guard != 0.
+// K1b: exclusive prefix sum of the bin counts (ensembles and pair terms), in three passes over
+// blocks of 1024.
 static __global__ void __launch_bounds__(1024) k_scan_blocks(const int *__restrict__ cnt,
                                                       int *__restrict__ off,
-                                                      int *__restrict__ bsum, int64_t n,
-                                                      const int *__restrict__ guard) {
-    if (guard && !*guard) return;
+                                                      int *__restrict__ bsum, int64_t n) {
     __shared__ int warp_tot[32];
     int64_t i = (int64_t)blockIdx.x * 1024 + threadIdx.x;
     int v = (i < n) ? cnt[i] : 0;
@@ -264,9 +262,7 @@ static __global__ void __launch_bounds__(1024) k_scan_blocks(const int *__restri
 }
 
 static __global__ void __launch_bounds__(1024) k_scan_sums(int *__restrict__ bsum, int64_t nb,
-                                                    int *__restrict__ off_end,
-                                                    const int *__restrict__ guard) {
-    if (guard && !*guard) return;
+                                                    int *__restrict__ off_end) {
     __shared__ int warp_tot[32];
     __shared__ int carry;
     if (threadIdx.x == 0) carry = 0;
@@ -303,16 +299,9 @@ static __global__ void __launch_bounds__(1024) k_scan_sums(int *__restrict__ bsu
 }
 
 static __global__ void __launch_bounds__(1024) k_scan_add(int *__restrict__ off,
-                                                   const int *__restrict__ bsum, int64_t n,
-                                                   int *__restrict__ cur,
-                                                   const int *__restrict__ guard) {
-    if (guard && !*guard) return;
+                                                   const int *__restrict__ bsum, int64_t n) {
     int64_t i = (int64_t)blockIdx.x * 1024 + threadIdx.x;
-    if (i < n) {
-        const int v = off[i] + bsum[blockIdx.x];
-        off[i] = v;
-        if (cur) cur[i] = v;
-    }
+    if (i < n) off[i] += bsum[blockIdx.x];
 }
 
 // Largest i with first[i] <= v (first is ascending, first[0] = 0).
@@ -864,12 +853,30 @@ __global__ void __launch_bounds__(256) k_mask(MaskGeom m, const int *__restrict_
                                               const T *__restrict__ ip2,
                                               typename PT<T>::C *__restrict__ hc0,
                                               typename PT<T>::C *__restrict__ hc1,
-                                              double *__restrict__ partial) {
+                                              double *__restrict__ partial,
+                                              unsigned *__restrict__ done, double loss_const,
+                                              double *__restrict__ loss) {
+    __shared__ bool s_last;
     const double lsum = mask_range<T, D>(m, rep_n, rep_s0, rep_w, spec, ip0, ip1, ip2, hc0, hc1,
                                          (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
                                          (int64_t)gridDim.x * blockDim.x);
     const double b = block_sum(lsum);
-    if (threadIdx.x == 0) partial[blockIdx.x] = b;
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = b;
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // the block that finishes last adds the partial sums in a fixed order, plus the folding constant
+    double v = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(partial + i);
+    const double t = block_sum(v);
+    if (threadIdx.x == 0) {
+        *loss = t + loss_const;
+        *done = 0;
+    }
 }
 
 // Batched mask: blocks [I.mb0, I.mb1) work on instance I only, so every partial belongs to one
@@ -908,21 +915,6 @@ static __global__ void __launch_bounds__(256) k_finalize_b(const BInst *__restri
         v += partial[k];
     const double s = block_sum(v);
     if (threadIdx.x == 0) losses[i] = s + inst[i].loss_const;
-}
-
-// K5: second-stage loss sum in a fixed order, plus the folding constant.
-static __global__ void __launch_bounds__(512) k_finalize(const double *__restrict__ partial, int nb,
-                                                  double loss_const, double *__restrict__ loss) {
-    __shared__ double sm[512];
-    double v = 0.0;
-    for (int i = threadIdx.x; i < nb; i += 512) v += partial[i];
-    sm[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 256; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sm[threadIdx.x] += sm[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *loss = sm[0] + loss_const;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1828,32 +1820,40 @@ inline int grid_for(int64_t n, int threads, int cap) {
 
 template <typename T>
 cudaError_t Launch<T>::scan(const int *cnt, int *off, int *block_sums, int64_t n, cudaStream_t s,
-                            int *launches, int *cur, const int *guard) {
+                            int *launches) {
     const int64_t nb = (n + 1023) / 1024;
-    k_scan_blocks<<<(unsigned)nb, 1024, 0, s>>>(cnt, off, block_sums, n, guard);
-    k_scan_sums<<<1, 1024, 0, s>>>(block_sums, nb, off + n, guard);
-    k_scan_add<<<(unsigned)nb, 1024, 0, s>>>(off, block_sums, n, cur, guard);
+    k_scan_blocks<<<(unsigned)nb, 1024, 0, s>>>(cnt, off, block_sums, n);
+    k_scan_sums<<<1, 1024, 0, s>>>(block_sums, nb, off + n);
+    k_scan_add<<<(unsigned)nb, 1024, 0, s>>>(off, block_sums, n);
     *launches += 3;
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t Launch<T>::count(const Geom &g, const T *points, int *cnt, int *err, cudaStream_t s,
-                             const int *guard) {
-    const int grid = grid_for((g.n_points + 3) / 4, 256, 152 * 16);
-    if (g.dim == 2) k_count<T, 2><<<grid, 256, 0, s>>>(g, points, cnt, err, guard);
-    else k_count<T, 3><<<grid, 256, 0, s>>>(g, points, cnt, err, guard);
-    return cudaGetLastError();
+int Launch<T>::bin_finish_blocks(const Geom &g) {
+    // all blocks must be resident together (grid barriers); more than the points need are no use
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const cudaError_t e =
+        g.dim == 2
+            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_finish<T, 2>, 256, 0)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bin_finish<T, 3>, 256, 0);
+    if (e != cudaSuccess) return 0;
+    return grid_for((std::max(g.n_points / 4, g.n_tiles) + 255) / 256 * 256, 256,
+                    std::min(kBinFinishBlocks, sms * per));
 }
 
 template <typename T>
-cudaError_t Launch<T>::place(const Geom &g, const T *points, int *cur, void *sorted, int *perm,
-                             cudaStream_t s, const int *guard) {
+cudaError_t Launch<T>::bin_finish(const Geom &g, const T *points, const int *tcur, int *cnt,
+                                  int *off, int *bsum, void *sorted, int *perm, int2 *tr, int *err,
+                                  int blocks, cudaStream_t s) {
     using U = typename PT<T>::U;
-    const int grid = grid_for((g.n_points + 3) / 4, 256, 152 * 16);
-    if (g.dim == 2) k_place<T, 2><<<grid, 256, 0, s>>>(g, points, cur, (U *)sorted, perm, guard);
-    else k_place<T, 3><<<grid, 256, 0, s>>>(g, points, cur, (U *)sorted, perm, guard);
-    return cudaGetLastError();
+    Geom gg = g;
+    U *so = (U *)sorted;
+    void *args[] = {&gg, &points, &tcur, &cnt, &off, &bsum, &so, &perm, &tr, &err};
+    const void *kern = g.dim == 2 ? (const void *)k_bin_finish<T, 2> : (const void *)k_bin_finish<T, 3>;
+    return cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3(256), args, 0, s);
 }
 
 template <typename T>
@@ -1866,13 +1866,6 @@ cudaError_t Launch<T>::place_direct(const Geom &g, const T *points, int64_t j0, 
         k_place_direct<T, 2><<<grid, 256, 0, s>>>(g, points, j0, tcur, (U *)sorted, perm, err);
     else
         k_place_direct<T, 3><<<grid, 256, 0, s>>>(g, points, j0, tcur, (U *)sorted, perm, err);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t Launch<T>::tile_ranges(const Geom &g, const int *tcur, const int *off, int2 *tr,
-                                   cudaStream_t s) {
-    k_tile_ranges<<<grid_for(g.n_tiles, 256, 152 * 16), 256, 0, s>>>(g, tcur, off, tr);
     return cudaGetLastError();
 }
 
@@ -1943,6 +1936,12 @@ cudaError_t WOps<T, W, D>::spread_own(const Geom &g, const EsPoly<T> &ep, const 
     kern<<<nt, 256, smem, s>>>(g, ep, (const U *)sorted, tr, grid, ring, ring_slot);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    if constexpr (D == 2) {
+        if (fold_gathers(g)) {
+            k_halo_gather<T, W><<<nt, 256, 0, s>>>(g, ring, ring_slot, grid);
+            return cudaGetLastError();
+        }
+    }
     // one launch per axis when every tile along it is at least W wide, else two (low, high)
     if (g.tq[0] >= W) {
         k_halo_fold<T, W, D, 0, 3, 0><<<nt, 256, 0, s>>>(g, ring, ring_slot, grid);
@@ -2086,7 +2085,9 @@ cudaError_t Launch<T>::spread_own(const Geom &g, const EsPoly<T> &ep, const void
                                   const int2 *tr, T *grid, T *ring, int64_t ring_slot,
                                   cudaStream_t s, int *launches) {
     *launches += 1;   // (the column spread's folds: the same count, z first)
-    for (int a = 0; a < g.dim; ++a) *launches += g.tq[a] >= g.width ? 1 : 2;
+    if (fold_gathers(g)) *launches += 1;
+    else
+        for (int a = 0; a < g.dim; ++a) *launches += g.tq[a] >= g.width ? 1 : 2;
     if (g.dim == 2) {
         FRESCO_WIDTH_SWITCH(g.width, return (WOps<T, WW, 2>::spread_own(g, ep, sorted, tr, grid,
                                                                           ring, ring_slot, s)));
@@ -2128,21 +2129,17 @@ cudaError_t Launch<T>::interp_kd(const Geom &g, const EsPoly<T> &ep, const void 
 template <typename T>
 cudaError_t Launch<T>::mask(const MaskGeom &m, const int *rep_n, const T *rep_s0, const T *rep_w,
                             const void *spec, const T *ip0, const T *ip1, const T *ip2, void *hc0,
-                            void *hc1, double *partial, int n_blocks, cudaStream_t s) {
+                            void *hc1, double *partial, int n_blocks, unsigned *done,
+                            double loss_const, double *loss, cudaStream_t s) {
     using C = typename PT<T>::C;
     if (m.dim == 2)
         k_mask<T, 2><<<n_blocks, 256, 0, s>>>(m, rep_n, rep_s0, rep_w, (const C *)spec, ip0, ip1,
-                                               ip2, (C *)hc0, (C *)hc1, partial);
+                                               ip2, (C *)hc0, (C *)hc1, partial, done, loss_const,
+                                               loss);
     else
         k_mask<T, 3><<<n_blocks, 256, 0, s>>>(m, rep_n, rep_s0, rep_w, (const C *)spec, ip0, ip1,
-                                               ip2, (C *)hc0, (C *)hc1, partial);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t Launch<T>::finalize(const double *partial, int n_blocks, double loss_const,
-                                double *loss, cudaStream_t s) {
-    k_finalize<<<1, 512, 0, s>>>(partial, n_blocks, loss_const, loss);
+                                               ip2, (C *)hc0, (C *)hc1, partial, done, loss_const,
+                                               loss);
     return cudaGetLastError();
 }
 

@@ -5,18 +5,16 @@
 //   k_place_direct  computes each point's tile and record and takes its slot from the tile's
 //                   cursor, pos = atomicAdd(&tcur[t], 1), at record t * tcap + pos;
 // the tile's points are then records [t tcap, t tcap + tcur[t]). A point whose tile is full sets
-// the overflow word tcur[n_tiles]; the compact form below then runs (its kernels do nothing
-// unless the overflow word is set), so any input is binned correctly and uniform inputs pay for
-// one pass only. The compact form, two passes with no per-point key or rank arrays:
-//   k_count  counts the points of every bin (global atomics whose result is unused);
-//   (exclusive scan of the counts into off[], and a copy of off[] into the cursor array cur[])
-//   k_place  recomputes each point's bin and record and takes its sorted position from the
-//            bin's cursor, pos = atomicAdd(&cur[bin], 1).
+// the overflow word tcur[n_tiles]; the compact form then runs inside the next kernel, so any input
+// is binned correctly and uniform inputs pay for one pass only:
+//   k_bin_finish    writes the record range of every tile, tr[t] = (first, end); after an overflow
+//                   it first counts the points of every bin, scans the counts into off[] and the
+//                   cursors, and places every point at its bin's next place, pos =
+//                   atomicAdd(&cur[bin], 1) (no per-point key or rank arrays).
 // In the compact form a tile owns Geom.sub consecutive bins, bin = tile * sub + (caller index mod
 // sub): the points of a tile stay contiguous (off[t sub] .. off[(t + 1) sub]), and each cursor
 // takes 1/sub of the tile's atomics, which keeps the returning atomics from queueing on few
-// addresses. k_tile_ranges writes the record range of every tile, tr[t] = (first, end), from
-// whichever form ran; the spread and interpolation kernels read only tr.
+// addresses. The spread and interpolation kernels read only tr.
 // The order of the points inside a tile depends on the order the atomics run in. Nothing
 // downstream depends on it: the fixed-point spread sums integers (order independent), the
 // interpolation writes each point's gradient through its caller index.
@@ -33,6 +31,8 @@
 // (E_x cells), rows through the tile store only their W halo cells (HL below the tile in x, then
 // W - HL above). ring_index maps an extended-region cell outside the tile to its position.
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include <utility>
 
@@ -96,12 +96,10 @@ __device__ __forceinline__ bool warp_has_runs(int bin, bool in) {
     return __any_sync(0xffffffffu, in && (threadIdx.x & 31) > 0 && prev == bin);
 }
 
-// guard (k_count, k_place): when not null, the kernel does nothing unless *guard != 0
+// Counts of every bin (compact form).
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_count(Geom g, const T *__restrict__ pts,
-                                               int *__restrict__ cnt, int *__restrict__ err,
-                                               const int *__restrict__ guard) {
-    if (guard && !*guard) return;
+__device__ __forceinline__ void count_points(const Geom &g, const T *__restrict__ pts,
+                                             int *__restrict__ cnt, int *__restrict__ err) {
     constexpr int IL = 4;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * IL;
     bool ok = true;
@@ -137,13 +135,12 @@ __global__ void __launch_bounds__(256) k_count(Geom g, const T *__restrict__ pts
     if (!ok) atomicOr(err, 1);
 }
 
+// Every point into its bin's next place (compact form; cur: the bins' offsets, advanced).
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_place(Geom g, const T *__restrict__ pts,
-                                               int *__restrict__ cur,
-                                               typename PT<T>::U *__restrict__ sorted,
-                                               int *__restrict__ perm,
-                                               const int *__restrict__ guard) {
-    if (guard && !*guard) return;
+__device__ __forceinline__ void place_points(const Geom &g, const T *__restrict__ pts,
+                                             int *__restrict__ cur,
+                                             typename PT<T>::U *__restrict__ sorted,
+                                             int *__restrict__ perm) {
     using U = typename PT<T>::U;
     constexpr int IL = 4;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x * IL;
@@ -189,6 +186,91 @@ __global__ void __launch_bounds__(256) k_place(Geom g, const T *__restrict__ pts
             if (j < g.n_points) store_record<T, D>(sorted, perm, pos[k], u[k], (int)j);
         }
     }
+}
+
+// Exclusive scan of a block's chunk of the bin counts: returns the chunk's total to every thread.
+__device__ __forceinline__ int block_total(int v) {
+    __shared__ int s_tot[8];
+    __syncthreads();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) s_tot[threadIdx.x >> 5] = v;
+    __syncthreads();
+    int t = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += s_tot[w];
+    return t;
+}
+
+// Completes the binning in one launch: the record range of every tile from the direct form, or,
+// when a tile overflowed (or the plan has no direct form, tcur null), the whole compact form: zero
+// the counts, count, scan, place, with grid barriers in between (a cooperative launch). The
+// separate kernels of the compact form, each returning at once after reading the overflow word,
+// cost an evaluation six launches: 20 us of the 46 us that binning 1e5 points took.
+template <typename T, int D>
+__global__ void __launch_bounds__(256) k_bin_finish(Geom g, const T *__restrict__ pts,
+                                                    const int *__restrict__ tcur,
+                                                    int *__restrict__ cnt, int *__restrict__ off,
+                                                    int *__restrict__ bsum,
+                                                    typename PT<T>::U *__restrict__ sorted,
+                                                    int *__restrict__ perm,
+                                                    int2 *__restrict__ tr, int *__restrict__ err) {
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t nt = (int64_t)gridDim.x * blockDim.x;
+    if (tcur && !tcur[g.n_tiles]) {
+        for (int64_t t = tid; t < g.n_tiles; t += nt) {
+            const int b = (int)(t * g.tcap);
+            tr[t] = make_int2(b, b + tcur[t]);
+        }
+        return;
+    }
+    cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    for (int64_t i = tid; i < g.n_bins; i += nt) cnt[i] = 0;
+    grid.sync();
+    count_points<T, D>(g, pts, cnt, err);
+    grid.sync();
+    // block b scans bins [b0, b1)
+    const int64_t per = (g.n_bins + gridDim.x - 1) / gridDim.x;
+    const int64_t b0 = min((int64_t)blockIdx.x * per, g.n_bins), b1 = min(b0 + per, g.n_bins);
+    int v = 0;
+    for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) v += __ldcg(cnt + i);
+    v = block_total(v);
+    if (threadIdx.x == 0) bsum[blockIdx.x] = v;
+    grid.sync();
+    v = 0;
+    for (int i = threadIdx.x; i < (int)blockIdx.x; i += blockDim.x) v += __ldcg(bsum + i);
+    int run = block_total(v);
+    __shared__ int s_warp[8];
+    for (int64_t i0 = b0; i0 < b1; i0 += blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        const int c = i < b1 ? __ldcg(cnt + i) : 0;
+        int x = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        __syncthreads();
+        if (lane == 31) s_warp[wid] = x;
+        __syncthreads();
+        int before = run, all = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < wid) before += s_warp[w];
+            all += s_warp[w];
+        }
+        if (i < b1) {
+            off[i] = before + x - c;
+            cnt[i] = before + x - c;   // the bin's placement cursor
+        }
+        run += all;
+    }
+    if (b1 == g.n_bins && b0 < b1 && threadIdx.x == 0) off[g.n_bins] = run;
+    grid.sync();
+    for (int64_t t = tid; t < g.n_tiles; t += nt)
+        tr[t] = make_int2(__ldcg(off + t * g.sub), __ldcg(off + (t + 1) * g.sub));
+    place_points<T, D>(g, pts, cnt, sorted, perm);
 }
 
 // One pass of the direct form: points j0 .. j0 + g.n_points - 1 of the caller's array (pts points
@@ -253,23 +335,6 @@ __global__ void __launch_bounds__(256) k_place_direct(Geom g, const T *__restric
     }
     if (!ok) atomicOr(err, 1);
     if (over) atomicOr(&tcur[g.n_tiles], 1);
-}
-
-// Record range of every tile: the direct form's (t tcap, t tcap + tcur[t]) unless its overflow
-// word is set (or the plan has no direct form, tcur null), else the compact form's offsets.
-static __global__ void __launch_bounds__(256) k_tile_ranges(Geom g, const int *__restrict__ tcur,
-                                                            const int *__restrict__ off,
-                                                            int2 *__restrict__ tr) {
-    const bool direct = tcur && !tcur[g.n_tiles];
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < g.n_tiles;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        if (direct) {
-            const int b = (int)(t * g.tcap);
-            tr[t] = make_int2(b, b + tcur[t]);
-        } else {
-            tr[t] = make_int2(off[t * g.sub], off[(t + 1) * g.sub]);
-        }
-    }
 }
 
 // Shared-memory accesses of the window loops, written as PTX on 32-bit shared-space addresses
@@ -1134,6 +1199,82 @@ __global__ void __launch_bounds__(256) k_halo_fold(Geom g, T *ring, int64_t ring
 #pragma unroll
         for (int k = 0; k < IL; ++k)
             if (dst[k]) *dst[k] = d[k] + v[k];
+    }
+}
+
+// The 2D fold in one launch: every cell of a tile's border bands gathers what the rings of the
+// neighbouring tiles hold for it (a side neighbour's halo, in the corners two sides' and the
+// diagonal's), in the order in which the passes above would have added them. Needs tiles at least
+// W wide on both axes, so that a cell has one neighbour per axis to gather from. Every ring cell is
+// read once and no ring is written, where the passes read and write the corners' rings again: one
+// launch instead of two. Its reads are the more scattered ones, so it is taken up to eight tiles
+// per SM, about one wave of blocks (fold_gathers). Measured, spread and fold, passes against gathering (us): 784
+// tiles 23.6 / 21.6, 2304 tiles 60.4 / 64.2, 6400 tiles 246 / 251.
+template <typename T, int W>
+__global__ void __launch_bounds__(256) k_halo_gather(Geom g, const T *__restrict__ ring,
+                                                     int64_t ring_slot, T *__restrict__ grid) {
+    constexpr int HL = W / 2, HR = W - HL;
+    const int64_t t = blockIdx.x;
+    int s[3], w[3], tc[3];
+    tile_extent(g, t, W, s, w, tc);
+    // neighbours' tile columns (rows) and widths: 0 below, 1 this tile, 2 above
+    int nx[3], ny[3], wx[3], wy[3];
+    nx[1] = tc[0];
+    ny[1] = tc[1];
+    nx[0] = tc[0] == 0 ? g.nb[0] - 1 : tc[0] - 1;
+    nx[2] = tc[0] == g.nb[0] - 1 ? 0 : tc[0] + 1;
+    ny[0] = tc[1] == 0 ? g.nb[1] - 1 : tc[1] - 1;
+    ny[2] = tc[1] == g.nb[1] - 1 ? 0 : tc[1] + 1;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        wx[i] = tile_start(nx[i] + 1, g.tq[0], g.tr[0]) - tile_start(nx[i], g.tq[0], g.tr[0]);
+        wy[i] = tile_start(ny[i] + 1, g.tq[1], g.tr[1]) - tile_start(ny[i], g.tq[1], g.tr[1]);
+    }
+    const FastDiv f0 = tile_div<0, false>(g, w[0]);
+    const int full = W * w[0], count = full + W * (w[1] - W);
+    constexpr int IL = 4;
+    for (int i0 = threadIdx.x; i0 < count; i0 += IL * blockDim.x) {
+        T v[IL], d[IL];
+        int64_t at[IL];
+#pragma unroll
+        for (int k = 0; k < IL; ++k) {
+            const int i = i0 + k * blockDim.x;
+            at[k] = -1;
+            v[k] = d[k] = T(0);
+            if (i >= count) continue;
+            int x, y;
+            if (i < full) {   // the W border rows, whole
+                const int r = f0.div(i);
+                x = i - r * w[0];
+                y = r < HR ? r : w[1] - W + r;
+            } else {          // the W border cells of the rows between
+                const int j = i - full, r = j / W, c = j - r * W;
+                y = HR + r;
+                x = c < HR ? c : w[0] - W + c;
+            }
+            // the neighbour along each axis that reaches the cell, and the cell in its region
+            const int ax = x < HR ? 0 : (x >= w[0] - HL ? 2 : 1);
+            const int ay = y < HR ? 0 : (y >= w[1] - HL ? 2 : 1);
+            const int ex = ax == 0 ? HL + wx[0] + x : (ax == 2 ? x - w[0] + HL : HL + x);
+            const int ey = ay == 0 ? HL + wy[0] + y : (ay == 2 ? y - w[1] + HL : HL + y);
+            auto from = [&](int bx, int by, int fx, int fy) -> T {
+                return ring[((int64_t)ny[by] * g.nb[0] + nx[bx]) * ring_slot +
+                            ring_index<W, 2>(fx, fy, 0, wx[bx], wy[by], 1)];
+            };
+            T sx = T(0), sy = T(0);
+            if (ax != 1) sx = from(ax, 1, ex, HL + y);
+            if (ay != 1) sy = from(1, ay, HL + x, ey);
+            if (ax != 1 && ay != 1) sy += from(ax, ay, ex, ey);
+            v[k] = sx;
+            d[k] = sy;
+            at[k] = (int64_t)(s[1] + y) * g.nf[0] + s[0] + x;
+        }
+        T o[IL];
+#pragma unroll
+        for (int k = 0; k < IL; ++k) o[k] = at[k] >= 0 ? grid[at[k]] : T(0);
+#pragma unroll
+        for (int k = 0; k < IL; ++k)
+            if (at[k] >= 0) grid[at[k]] = (o[k] + v[k]) + d[k];
     }
 }
 
