@@ -35,10 +35,12 @@
 #include <vector>
 
 #include "fresco.h"
+#include "fresco_fft.cuh"
 #include "fresco_kernels.cuh"
 #include "fresco_uwnu_tiles.h"
 
 using namespace fresco;
+using namespace fresco::fft_detail;
 
 namespace fresco {
 FRESCO_EXTERN_WIDTH_OPS(float)
@@ -363,12 +365,30 @@ __global__ void __launch_bounds__(256) k_un_spread(UGrid g, UTiles tl, EsPoly<T>
                                                    const int *__restrict__ tcell,
                                                    const T *__restrict__ tfrac,
                                                    const CxT<T> *__restrict__ coef,
-                                                   CxT<T> *__restrict__ U) {
+                                                   CxT<T> *__restrict__ U,
+                                                   const double *__restrict__ part, int n_part,
+                                                   double *__restrict__ scal,
+                                                   double *__restrict__ loss) {
     using F = SpreadFixed<T>;
     using I = typename F::I;
     __shared__ I sh[2 * kUTileCells];   // real parts, then imaginary parts at + kUTileCells
     __shared__ T s_max[8];
-    for (int64_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    // with part given, one block more than the tiles' adds the interpolation's partial sums (the
+    // loss and F) in a fixed order
+    const int nb = gridDim.x - (part ? 1 : 0);
+    if ((int)blockIdx.x == nb) {
+        for (int k = 0; k < 2; ++k) {
+            double v = 0.0;
+            for (int i = threadIdx.x; i < n_part; i += blockDim.x) v += part[(int64_t)k * n_part + i];
+            const double s = ublock_sum(v);
+            if (threadIdx.x == 0) {
+                scal[1 + k] = s;
+                if (k == 0) *loss = s;
+            }
+        }
+        return;
+    }
+    for (int64_t t = blockIdx.x; t < n_tiles; t += nb) {
         const int tx = (int)(t % tl.nt[0]);
         const int ty = (int)((t / tl.nt[0]) % tl.nt[1]);
         const int tz = (int)(t / ((int64_t)tl.nt[0] * tl.nt[1]));
@@ -464,6 +484,202 @@ __global__ void __launch_bounds__(256) k_un_grad(UGrid g, int64_t cells, const T
     }
 }
 
+// ---- real grids: half-plane transforms -----------------------------------------------------------
+// The weights (or the points' grid) are real, so the type-2 field F[l] = sum_m (c_m / Psi) exp(-2 pi
+// i m l / n_f) is Hermitian and half of it holds everything: a constraint at x' = nu / M (modulo 1)
+// in the upper half along x is replaced by the one at -x' (rho conjugated, the same S and the same
+// term of the gradient), after which every kernel support lies in l_x = -w .. n_f/2 + w. In 2D FP32
+// plans U then holds these rows only, transposed: [n_f/2 + 2 w + 1][n_fy], y contiguous, row e for
+// l_x = e - w, and the transforms go in four kernels that read and write each of their arrays once:
+//   k_ug_rows_fwd  the pixel rows, deconvolved and zero-filled on the way in, along x; the half
+//                  spectrum out, transposed: only the M_y rows that are not zero;
+//   k_ug_cols_fwd  a column of it, zero-filled along y, into its row of U (and the rows of the
+//                  margins that are its conjugates);
+//   k_ug_cols_inv  a row of U with the margins' conjugates, along y back, the M_y rows needed;
+//   k_ug_rows_inv  those, along x back, the M_x pixels needed, with the gradient's last step.
+// Against a zeroed complex grid, a fill and a complex transform of the whole grid each way that is
+// less than a quarter of the traffic and no clearing. Measured on GB300 (us, before and after): 1024^2
+// weights, 10^6 constraints: onto U 75 / 48, interpolation 82 / 43, spread 77 / 69, back 56 / 38;
+// 1620^2 points' grid, 10^6 wavevectors: 162 / 72, 154 / 85, 104 / 82, 146 / 75.
+struct RealGrid {
+    int mx, my;     // pixels
+    int nfx, nfy;   // fine grid
+    int w;
+    int centred;    // pixel m sits at m - floor(M / 2) (weights), else at m or m - M past the middle
+};
+__device__ __forceinline__ bool ug_pixel(int f, int nf, int M, int centred, int &m, int &t) {
+    t = f < nf / 2 ? f : f - nf;
+    m = centred ? t + M / 2 : (t < 0 ? t + M : t);
+    return t >= -(M / 2) && t < M - M / 2;
+}
+// fine position of pixel m along an axis
+__device__ __forceinline__ int ug_centre(int m, int M, int centred) {
+    return centred ? m - M / 2 : (m < M / 2 ? m : m - M);
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_ug_rows_fwd(const __grid_constant__ FftDesc f, RealGrid g, const float *__restrict__ c,
+                  const float *__restrict__ ip0, const float *__restrict__ ip1,
+                  const float2 *__restrict__ tws, float2 *__restrict__ xt) {
+    extern __shared__ __align__(128) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const int M = f.n, pitch = f.words;
+    const int r0 = blockIdx.x * f.rows, nr = min(f.rows, g.my - r0);
+    fft_forward(f, nr, s, pitch, [&](int row, int i) {
+        const int m1 = r0 + row;
+        const int t1 = ug_centre(m1, g.my, g.centred);
+        const float ipy = __ldg(ip1 + (t1 < 0 ? -t1 : t1));
+        float v[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            int m, t;
+            v[h] = 0.f;
+            if (ug_pixel(2 * i + h, g.nfx, g.mx, g.centred, m, t))
+                v[h] = c[(int64_t)m1 * g.mx + m] * (__ldg(ip0 + (t < 0 ? -t : t)) * ipy);
+        }
+        return float2{v[0], v[1]};
+    });
+    // columns 0 .. M of the half spectrum (as k_fft_rows_fwd)
+    const int half = M / 2, shift = __popc(f.rows - 1);
+    for (int t = threadIdx.x; t < (half + 1) << shift; t += blockDim.x) {
+        const int row = t & (f.rows - 1), k = t >> shift;
+        if (row >= nr) continue;
+        const int km = M - k;
+        const float2 a = s[row * pitch + fft_place(f, __ldg(f.pos + k))];
+        const float2 b = s[row * pitch + fft_place(f, __ldg(f.pos + (k == 0 ? 0 : km)))];
+        const float2 w = __ldg(tws + k);
+        const float ex = 0.5f * (a.x + b.x), ey = 0.5f * (a.y - b.y);
+        const float ox = 0.5f * (a.y + b.y), oy = -0.5f * (a.x - b.x);
+        const float px = w.x * ox - w.y * oy, py = w.x * oy + w.y * ox;
+        float2 *o = xt + r0 + row;
+        o[(int64_t)k * g.my] = {ex + px, ey + py};
+        if (km > half) o[(int64_t)km * g.my] = {ex - px, -(ey - py)};
+    }
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_ug_cols_fwd(const __grid_constant__ FftDesc f, RealGrid g, const float2 *__restrict__ xt,
+                  float2 *__restrict__ U) {
+    extern __shared__ __align__(128) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const int k = blockIdx.x, n = f.n, hx = g.nfx / 2;
+    const float2 *in = xt + (int64_t)k * g.my;
+    fft_forward(f, 1, s, 0, [&](int, int i) {
+        int m, t;
+        float2 v = {0.f, 0.f};
+        if (ug_pixel(i, n, g.my, g.centred, m, t)) v = in[m];
+        return v;
+    });
+    float2 *row = U + (int64_t)(k + g.w) * n;
+    float2 *lo = k >= 1 && k <= g.w ? U + (int64_t)(g.w - k) * n : nullptr;
+    const int j = hx - k;
+    float2 *hi = j >= 1 && j <= g.w ? U + (int64_t)(g.w + hx + j) * n : nullptr;
+    for (int l = threadIdx.x; l < n; l += blockDim.x) {
+        const float2 v = s[fft_place(f, __ldg(f.pos + l))];
+        row[l] = v;
+        const int lm = l ? n - l : 0;
+        if (lo) lo[lm] = {v.x, -v.y};
+        if (hi) hi[lm] = {v.x, -v.y};
+    }
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_ug_cols_inv(const __grid_constant__ FftDesc f, RealGrid g, const float2 *__restrict__ U,
+                  float2 *__restrict__ bt) {
+    extern __shared__ __align__(128) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const int k = blockIdx.x, n = f.n, hx = g.nfx / 2;
+    // X = (V[k] + conj V[-k]) / 2; V[-k] has a row in U next to either end only
+    const float2 *row = U + (int64_t)(k + g.w) * n;
+    const int e = k <= g.w ? g.w - k : (hx - k <= g.w ? g.w + g.nfx - k : -1);
+    const float2 *neg = e >= 0 ? U + (int64_t)e * n : nullptr;
+    for (int l = threadIdx.x; l < n; l += blockDim.x) {
+        float2 v = row[l];
+        if (neg) {
+            const float2 u = neg[l ? n - l : 0];
+            v = {v.x + u.x, v.y - u.y};
+        }
+        s[fft_place(f, __ldg(f.pos + l))] = {0.5f * v.y, 0.5f * v.x};
+    }
+    __syncthreads();
+    float2 *out = bt + (int64_t)k * g.my;
+    fft_adjoint(f, 1, s, 0, [&](int, int i, float2 v) {
+        int m, t;
+        if (ug_pixel(i, n, g.my, g.centred, m, t)) out[m] = {v.y, v.x};
+    });
+}
+
+// out = field / Psi (minus (4 F / rho0) c where c is given: the weight gradient)
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_ug_rows_inv(const __grid_constant__ FftDesc f, RealGrid g, const float2 *__restrict__ bt,
+                  const float *__restrict__ ip0, const float *__restrict__ ip1,
+                  const float2 *__restrict__ tws, const float *__restrict__ c,
+                  const double *__restrict__ scal, float *__restrict__ out) {
+    extern __shared__ __align__(128) unsigned char sm_raw[];
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    const int M = f.n, pitch = f.words;
+    const int r0 = blockIdx.x * f.rows, nr = min(f.rows, g.my - r0);
+    const int half = M / 2, shift = __popc(f.rows - 1);
+    const float coef = c ? (float)(4.0 * scal[2] / scal[0]) : 0.f;
+    for (int t = threadIdx.x; t < (half + 1) << shift; t += blockDim.x) {
+        const int row = t & (f.rows - 1), k = t >> shift;
+        if (row >= nr) continue;
+        const int km = M - k;
+        const float2 a = bt[(int64_t)k * g.my + r0 + row], b = bt[(int64_t)km * g.my + r0 + row];
+        const float2 w = __ldg(tws + k);
+        const float px = a.x + b.x, py = a.y - b.y;
+        const float dx = a.x - b.x, dy = a.y + b.y;
+        const float qx = dx * w.x + dy * w.y, qy = dy * w.x - dx * w.y;
+        s[row * pitch + fft_place(f, __ldg(f.pos + k))] = {py + qx, px - qy};
+        if (km > half && km < M)
+            s[row * pitch + fft_place(f, __ldg(f.pos + km))] = {-py + qx, px + qy};
+    }
+    __syncthreads();
+    fft_adjoint(f, nr, s, pitch, [&](int row, int i, float2 v) {
+        const int m1 = r0 + row;
+        const int t1 = ug_centre(m1, g.my, g.centred);
+        const float ipy = __ldg(ip1 + (t1 < 0 ? -t1 : t1));
+        const float x[2] = {v.y, v.x};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            int m, t;
+            if (!ug_pixel(2 * i + h, g.nfx, g.mx, g.centred, m, t)) continue;
+            const int64_t p = (int64_t)m1 * g.mx + m;
+            const float ip = __ldg(ip0 + (t < 0 ? -t : t)) * ipy;
+            out[p] = c ? x[h] * ip - coef * c[p] : x[h] * ip;
+        }
+    });
+}
+
+// rho0 = sum c^2 in one launch: the block that finishes last adds the partial sums in a fixed order
+template <typename T>
+__global__ void __launch_bounds__(256) k_un_rho0(const T *__restrict__ c, int64_t n,
+                                                 double *__restrict__ part,
+                                                 unsigned *__restrict__ done,
+                                                 double *__restrict__ out) {
+    __shared__ bool s_last;
+    DotAcc<T> acc;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        acc.add(c[i], c[i]);
+    const double b = ublock_sum(acc.value());
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = b;
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double v = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(part + i);
+    const double s = ublock_sum(v);
+    if (threadIdx.x == 0) {
+        *out = s;
+        *done = 0;
+    }
+}
+
 fresco_status un_status(cudaError_t e) {
     if (e == cudaSuccess) return FRESCO_OK;
     if (e == cudaErrorMemoryAllocation) return FRESCO_ERR_OOM;
@@ -506,6 +722,15 @@ struct fresco_uwnu_s {
     int *ent = nullptr;                          // [n_ent] constraint slots, tile by tile
     int *kcov = nullptr;                         // [n_tiles] most supports covering one cell
     double *part = nullptr, *scal = nullptr;     // scal: rho0 (or N), loss, F sum
+    // real grids (2D FP32): U is the half plane [n_f/2 + 2 w + 1][n_fy] of the RealGrid form; ug is
+    // its geometry for the constraint-side kernels (axis 0 is y)
+    bool real = false;
+    RealGrid rg{};
+    UGrid ug{};
+    fresco::FftDesc fx, fy;
+    void *xt = nullptr;                          // [n_f/2 + 1][M_y] between the x and y passes
+    void *tws = nullptr;                         // exp(-2 pi i k / n_fx), k <= n_fx / 4
+    unsigned *done = nullptr;
     cufftHandle fft = 0;
     bool have_fft = false;
     bool evaluated = false;
@@ -532,7 +757,7 @@ cudaError_t launch_un_interp(const fresco_uwnu_s *u, const EsPoly<T> &ep, cudaSt
     const auto *U = (const CxT<T> *)u->U;
     if (u->g.dim == 2)
         k_un_interp_win<T, W><<<u->nb, 256, 0, s>>>(
-            u->g, u->tl, ep, u->n_tiles, u->hoff, u->tcell, (const T *)u->tfrac, U,
+            u->ug, u->tl, ep, u->n_tiles, u->hoff, u->tcell, (const T *)u->tfrac, U,
             (const T *)u->s0, (const T *)u->wq, u->scal, (const T *)u->dq, u->perm,
             (CxT<T> *)u->coef, (T *)u->S, u->part);
     else
@@ -543,17 +768,22 @@ cudaError_t launch_un_interp(const fresco_uwnu_s *u, const EsPoly<T> &ep, cudaSt
     return cudaGetLastError();
 }
 
+// loss, when given: the spread also adds the interpolation's partial sums and writes the loss there
 template <typename T, int W>
-cudaError_t launch_un_spread(const fresco_uwnu_s *u, const EsPoly<T> &ep, cudaStream_t s) {
-    const unsigned nb = (unsigned)std::min<int64_t>(u->n_tiles, 152 * 64);
+cudaError_t launch_un_spread(const fresco_uwnu_s *u, const EsPoly<T> &ep, double *loss,
+                             cudaStream_t s) {
+    const unsigned nb = (unsigned)std::min<int64_t>(u->n_tiles, 152 * 64) + (loss ? 1 : 0);
+    const double *part = loss ? u->part : nullptr;
     if (u->g.dim == 2)
-        k_un_spread<T, W, 2><<<nb, 256, 0, s>>>(u->g, u->tl, ep, u->n_tiles, u->toff, u->ent,
+        k_un_spread<T, W, 2><<<nb, 256, 0, s>>>(u->ug, u->tl, ep, u->n_tiles, u->toff, u->ent,
                                                 u->kcov, u->tcell, (const T *)u->tfrac,
-                                                (const CxT<T> *)u->coef, (CxT<T> *)u->U);
+                                                (const CxT<T> *)u->coef, (CxT<T> *)u->U, part,
+                                                u->nb, u->scal, loss);
     else
-        k_un_spread<T, W, 3><<<nb, 256, 0, s>>>(u->g, u->tl, ep, u->n_tiles, u->toff, u->ent,
+        k_un_spread<T, W, 3><<<nb, 256, 0, s>>>(u->ug, u->tl, ep, u->n_tiles, u->toff, u->ent,
                                                 u->kcov, u->tcell, (const T *)u->tfrac,
-                                                (const CxT<T> *)u->coef, (CxT<T> *)u->U);
+                                                (const CxT<T> *)u->coef, (CxT<T> *)u->U, part,
+                                                u->nb, u->scal, loss);
     return cudaGetLastError();
 }
 
@@ -572,9 +802,9 @@ cudaError_t un_interp(const fresco_uwnu_s *u, cudaStream_t s) {
 
 // the strengths onto every tile of U (one launch)
 template <typename T>
-cudaError_t un_spread(const fresco_uwnu_s *u, cudaStream_t s) {
+cudaError_t un_spread(const fresco_uwnu_s *u, cudaStream_t s, double *loss = nullptr) {
     const EsPoly<T> &ep = un_poly<T>(u);
-    FRESCO_WIDTH_SWITCH(u->width, return (launch_un_spread<T, WW>(u, ep, s)));
+    FRESCO_WIDTH_SWITCH(u->width, return (launch_un_spread<T, WW>(u, ep, loss, s)));
 }
 
 bool un_alloc(fresco_uwnu_s *u, void **p, size_t bytes) {
@@ -600,15 +830,28 @@ void un_free(fresco_uwnu_s *u) {
 // Builds the constraint side of a plan: the deconvolution tables, the kernel polynomials, the
 // constraints' fine cells and positions (from FP64), their tile order and the tiles' lists, and
 // the FFT plan. dq (point plans; may be null): a factor per constraint in the caller's order.
+// centred: where pixel m of the grid sits (RealGrid).
 template <typename T>
 fresco_status un_build(fresco_uwnu_s *u, const double *nu, const double *S0, const double *W,
-                       const double *dq) {
+                       const double *dq, int centred) {
     using C2 = CxT<T>;
     const UGrid &g = u->g;
     const int dim = g.dim;
     const int64_t nk = u->n_k;
     const int w = u->width;
-    u->tl = utiles_for(dim, g.nf);
+    // real grids (2D FP32) whose transforms fit the shared memory of the library's own kernels; the
+    // margins of the half plane must not overlap
+    u->real = dim == 2 && sizeof(T) == 4 && g.nf[0] >= 4 * w + 2 &&
+              fresco::fft_describe(g.nf[0] / 2, u->fx) && fresco::fft_describe(g.nf[1], u->fy);
+    u->ug = g;
+    if (u->real) {
+        u->rg = RealGrid{g.M[0], g.M[1], g.nf[0], g.nf[1], w, centred};
+        u->ug.nf[0] = g.nf[1];
+        u->ug.nf[1] = g.nf[0] / 2 + 2 * w + 1;
+        u->fine = (int64_t)u->ug.nf[0] * u->ug.nf[1];
+    }
+    const int *tnf = u->ug.nf;   // the constraint side's grid
+    u->tl = utiles_for(dim, tnf);
     const UTiles &tl = u->tl;
     u->n_tiles = (int64_t)tl.nt[0] * tl.nt[1] * tl.nt[2];
     if (dim == 2)   // the window interpolation: a block per home tile (up to kUWinBlocks)
@@ -619,7 +862,25 @@ fresco_status un_build(fresco_uwnu_s *u, const double *nu, const double *S0, con
     // fine cell and fraction of every target x = -nu / M (modulo 1), in the caller's order
     std::vector<int> cell((size_t)(nk * dim));
     std::vector<double> frac((size_t)(nk * dim));
-    for (int64_t q = 0; q < nk; ++q)
+    for (int64_t q = 0; q < nk; ++q) {
+        if (u->real) {
+            // at +nu / M (the forward transform), folded to l_x <= n_f / 2; axis 0 is y, and the
+            // rows of U start at l_x = -w
+            double t[2];
+            for (int a = 0; a < 2; ++a) {
+                const double x = nu[q * 2 + a] / (double)g.M[a];
+                t[a] = (x - std::floor(x)) * (double)g.nf[a];
+            }
+            if (t[0] > 0.5 * (double)g.nf[0])
+                for (int a = 0; a < 2; ++a) t[a] = (double)g.nf[a] - t[a];
+            for (int a = 0; a < 2; ++a) {
+                const double c = std::floor(t[a]);
+                const int64_t ci = a == 0 ? (int64_t)c + w : (int64_t)c % g.nf[1];
+                cell[(size_t)(q * 2 + 1 - a)] = (int)ci;
+                frac[(size_t)(q * 2 + 1 - a)] = t[a] - c;
+            }
+            continue;
+        }
         for (int a = 0; a < dim; ++a) {
             const double x = -nu[q * dim + a] / (double)g.M[a];
             const double t = (x - std::floor(x)) * (double)g.nf[a];
@@ -629,9 +890,10 @@ fresco_status un_build(fresco_uwnu_s *u, const double *nu, const double *S0, con
             cell[(size_t)(q * dim + a)] = (int)ci;
             frac[(size_t)(q * dim + a)] = t - c;
         }
+    }
     // tile order, the tiles' lists and their cover counts (fresco_uwnu_tiles.h)
     UTilePlan tp;
-    if (!build_utile_plan<T>(dim, g.nf, w, tl, cell.data(), frac.data(), nk, tp))
+    if (!build_utile_plan<T>(dim, tnf, w, tl, cell.data(), frac.data(), nk, tp))
         return FRESCO_ERR_UNSUPPORTED;
     u->n_ent = tp.n_ent;
     const std::vector<int> &perm = tp.perm;
@@ -690,6 +952,34 @@ fresco_status un_build(fresco_uwnu_s *u, const double *nu, const double *S0, con
     UN_CUDA(cudaMemcpy(u->toff, toff.data(), sizeof(int64_t) * toff.size(), cudaMemcpyHostToDevice));
     UN_CUDA(cudaMemcpy(u->ent, ent.data(), sizeof(int) * ent.size(), cudaMemcpyHostToDevice));
     UN_CUDA(cudaMemcpy(u->kcov, kcov.data(), sizeof(int) * kcov.size(), cudaMemcpyHostToDevice));
+    if (u->real) {
+        const size_t half = (size_t)g.nf[0] / 2 + 1;
+        if (!un_alloc(u, &u->xt, sizeof(C2) * half * (size_t)g.M[1]) ||
+            !un_alloc(u, &u->tws, sizeof(C2) * (size_t)(g.nf[0] / 4 + 1)) ||
+            !un_alloc(u, (void **)&u->done, sizeof(unsigned)))
+            return FRESCO_ERR_OOM;
+        UN_CUDA(cudaMemset(u->done, 0, sizeof(unsigned)));
+        std::vector<C2> tw((size_t)g.nf[0] / 4 + 1);
+        for (int k = 0; k <= g.nf[0] / 4; ++k) {
+            const double a = 2.0 * kPiU * (double)k / (double)g.nf[0];
+            tw[(size_t)k].x = (T)std::cos(a);
+            tw[(size_t)k].y = (T)-std::sin(a);
+        }
+        UN_CUDA(cudaMemcpy(u->tws, tw.data(), sizeof(C2) * tw.size(), cudaMemcpyHostToDevice));
+        int64_t bytes = 0;
+        fresco::fft_size_rows(u->fx, g.M[1]);
+        fresco::fft_size_cols(u->fy);
+        fresco_status st = fresco::fft_tables(u->fx, u->allocs, bytes);
+        if (!st) st = fresco::fft_tables(u->fy, u->allocs, bytes);
+        if (st) return st;
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        UN_CUDA(cudaFuncSetAttribute(k_ug_rows_fwd, attr, (int)fresco::kFftSmem));
+        UN_CUDA(cudaFuncSetAttribute(k_ug_cols_fwd, attr, (int)fresco::kFftSmem));
+        UN_CUDA(cudaFuncSetAttribute(k_ug_cols_inv, attr, (int)fresco::kFftSmem));
+        UN_CUDA(cudaFuncSetAttribute(k_ug_rows_inv, attr, (int)fresco::kFftSmem));
+        UN_CUDA(cudaDeviceSynchronize());
+        return FRESCO_OK;
+    }
     const cufftType type = sizeof(T) == 4 ? CUFFT_C2C : CUFFT_Z2Z;
     if (dim == 2) UN_CUFFT(cufftPlan2d(&u->fft, g.nf[1], g.nf[0], type));
     else UN_CUFFT(cufftPlan3d(&u->fft, g.nf[2], g.nf[1], g.nf[0], type));
@@ -708,8 +998,67 @@ fresco_status un_fft(fresco_uwnu_s *u, int dir) {
     return FRESCO_OK;
 }
 
+// The half-plane transforms of a real grid c (pixels) and back (c, when given, adds the weight
+// gradient's second term)
+fresco_status ug_forward(const fresco_uwnu_s *u, const float *c, cudaStream_t s) {
+    const RealGrid &g = u->rg;
+    k_ug_rows_fwd<<<(unsigned)((g.my + u->fx.rows - 1) / u->fx.rows), u->fx.threads,
+                    fresco::fft_bytes(u->fx, u->fx.rows), s>>>(
+        u->fx, g, c, (const float *)u->ip[0], (const float *)u->ip[1], (const float2 *)u->tws,
+        (float2 *)u->xt);
+    k_ug_cols_fwd<<<(unsigned)(g.nfx / 2 + 1), u->fy.threads, fresco::fft_bytes(u->fy, 1), s>>>(
+        u->fy, g, (const float2 *)u->xt, (float2 *)u->U);
+    return un_status(cudaGetLastError());
+}
+fresco_status ug_inverse(const fresco_uwnu_s *u, const float *c, float *out, cudaStream_t s) {
+    const RealGrid &g = u->rg;
+    k_ug_cols_inv<<<(unsigned)(g.nfx / 2 + 1), u->fy.threads, fresco::fft_bytes(u->fy, 1), s>>>(
+        u->fy, g, (const float2 *)u->U, (float2 *)u->xt);
+    k_ug_rows_inv<<<(unsigned)((g.my + u->fx.rows - 1) / u->fx.rows), u->fx.threads,
+                    fresco::fft_bytes(u->fx, u->fx.rows), s>>>(
+        u->fx, g, (const float2 *)u->xt, (const float *)u->ip[0], (const float *)u->ip[1],
+        (const float2 *)u->tws, c, u->scal, out);
+    return un_status(cudaGetLastError());
+}
+
+// un_eval of a real-grid plan: seven launches, the loss's last sum among the spread's blocks (or
+// five, the sum on its own, when only the loss is wanted).
+fresco_status un_eval_real(fresco_uwnu_s *u, const float *c, double *loss, float *grad) {
+    cudaStream_t s = u->stream;
+    fresco_status st;
+    {
+        fresco::StageScope sc(u->prof, s, UST_TYPE2);
+        const unsigned nb = (unsigned)std::min<int64_t>((u->cells + 1023) / 1024, kUBlocks);
+        k_un_rho0<float><<<nb, 256, 0, s>>>(c, u->cells, u->part, u->done, u->scal);
+        if ((st = ug_forward(u, c, s))) return st;
+    }
+    {
+        fresco::StageScope sc(u->prof, s, UST_INTERP);
+        UN_CUDA(un_interp<float>(u, s));
+        if (!grad) {
+            k_un_sum<<<1, 256, 0, s>>>(u->part, u->nb, 2, u->scal + 1);
+            UN_CUDA(cudaMemcpyAsync(loss, u->scal + 1, sizeof(double), cudaMemcpyDeviceToDevice, s));
+        }
+    }
+    u->launches += 4 + (grad ? 0 : 1);
+    u->evaluated = true;
+    if (!grad) return un_status(cudaGetLastError());
+    {
+        fresco::StageScope sc(u->prof, s, UST_SPREAD);
+        UN_CUDA(un_spread<float>(u, s, loss));
+    }
+    {
+        fresco::StageScope sc(u->prof, s, UST_TYPE1);
+        if ((st = ug_inverse(u, c, grad, s))) return st;
+    }
+    u->launches += 3;
+    return un_status(cudaGetLastError());
+}
+
 template <typename T>
 fresco_status un_eval(fresco_uwnu_s *u, const T *c, double *loss, T *grad) {
+    if constexpr (sizeof(T) == 4)
+        if (u->real) return un_eval_real(u, c, loss, grad);
     using C2 = CxT<T>;
     const UGrid &g = u->g;
     cudaStream_t s = u->stream;
@@ -801,8 +1150,8 @@ fresco_status fresco_uwnu_plan(fresco_uwnu_t *out, int dim, const int64_t *grid,
     u->n_k = n_k;
     u->nb = (int)std::max<int64_t>(1, std::min<int64_t>((n_k + 255) / 256, kUBlocks));
     u->stream = (cudaStream_t)stream;
-    const fresco_status st = o.precision == FRESCO_F64 ? un_build<double>(u, nu, S0, W, nullptr)
-                                                       : un_build<float>(u, nu, S0, W, nullptr);
+    const fresco_status st = o.precision == FRESCO_F64 ? un_build<double>(u, nu, S0, W, nullptr, 1)
+                                                       : un_build<float>(u, nu, S0, W, nullptr, 1);
     if (st) {
         un_free(u);
         return st;
@@ -946,7 +1295,7 @@ __global__ void __launch_bounds__(256) k_nu_bounds(const T *__restrict__ pts, in
          j += (int64_t)gridDim.x * blockDim.x)
         for (int a = 0; a < dim; ++a) {
             const double r = (double)pts[j * dim + a];
-            out |= r < -half[a] || r > half[a];   // NaN passes here: k_count flags it
+            out |= r < -half[a] || r > half[a];   // NaN passes here: the binning flags it
         }
     if (out) atomicOr(err, 2);
 }
@@ -993,7 +1342,7 @@ fresco_status nu_build(fresco_nuwnu_s *p, const double *kvec, const double *S0, 
         fresco::kernel_ft_at(u->width, u->beta, theta.data(), n_k, psi.data());
         for (int64_t q = 0; q < n_k; ++q) dq[(size_t)q] /= psi[(size_t)q];
     }
-    fresco_status st = un_build<T>(u, nu.data(), S0, W, dq.data());
+    fresco_status st = un_build<T>(u, nu.data(), S0, W, dq.data(), 0);
     if (st) return st;
     const double norm = (double)p->n_points;   // S = |rho|^2 / N
     UN_CUDA(cudaMemcpy(u->scal, &norm, sizeof(double), cudaMemcpyHostToDevice));
@@ -1032,11 +1381,15 @@ fresco_status nu_eval(fresco_nuwnu_s *p, const T *pts, double *loss, T *grad) {
     }
     {   // type 2 of the spread grid: onto U, inverse FFT
         fresco::StageScope sc(u->prof, s, UST_TYPE2);
-        UN_CUDA(cudaMemsetAsync(u->U, 0, sizeof(C2) * (size_t)u->fine, s));
-        k_nu_fill<T><<<pb, 256, 0, s>>>(g, p->cells, (const T *)p->ps.grid, ip0, ip1, ip2,
-                                        (C2 *)u->U);
-        st = un_fft<T>(u, CUFFT_INVERSE);
-        if (st) return st;
+        if (u->real) {
+            if ((st = ug_forward(u, (const float *)p->ps.grid, s))) return st;
+        } else {
+            UN_CUDA(cudaMemsetAsync(u->U, 0, sizeof(C2) * (size_t)u->fine, s));
+            k_nu_fill<T><<<pb, 256, 0, s>>>(g, p->cells, (const T *)p->ps.grid, ip0, ip1, ip2,
+                                            (C2 *)u->U);
+            st = un_fft<T>(u, CUFFT_INVERSE);
+            if (st) return st;
+        }
     }
     {   // at the wavevectors: S, the loss and the type-1 strengths
         fresco::StageScope sc(u->prof, s, UST_INTERP);
@@ -1044,7 +1397,7 @@ fresco_status nu_eval(fresco_nuwnu_s *p, const T *pts, double *loss, T *grad) {
         k_un_sum<<<1, 256, 0, s>>>(u->part, u->nb, 1, u->scal + 1);
         UN_CUDA(cudaMemcpyAsync(loss, u->scal + 1, sizeof(double), cudaMemcpyDeviceToDevice, s));
     }
-    p->launches += 4;
+    p->launches += 4 + (u->real ? 1 : 0);
     u->evaluated = true;
     if (!grad) return un_status(cudaGetLastError());
     {   // type 1 of the strengths onto U
@@ -1053,10 +1406,14 @@ fresco_status nu_eval(fresco_nuwnu_s *p, const T *pts, double *loss, T *grad) {
     }
     {   // forward FFT, the field on the points' grid
         fresco::StageScope sc(u->prof, s, UST_TYPE1);
-        st = un_fft<T>(u, CUFFT_FORWARD);
-        if (st) return st;
-        k_nu_field<T><<<pb, 256, 0, s>>>(g, p->cells, ip0, ip1, ip2, (const C2 *)u->U,
-                                         (T *)p->ps.grid);
+        if (u->real) {
+            if ((st = ug_inverse(u, nullptr, (float *)p->ps.grid, s))) return st;
+        } else {
+            st = un_fft<T>(u, CUFFT_FORWARD);
+            if (st) return st;
+            k_nu_field<T><<<pb, 256, 0, s>>>(g, p->cells, ip0, ip1, ip2, (const C2 *)u->U,
+                                             (T *)p->ps.grid);
+        }
     }
     {   // the kernel-derivative interpolation at the points
         fresco::StageScope sc(u->prof, s, UST_POINT_INTERP);
@@ -1066,7 +1423,7 @@ fresco_status nu_eval(fresco_nuwnu_s *p, const T *pts, double *loss, T *grad) {
         UN_CUDA(Launch<T>::interp_kd(p->ps.g, ep, p->ps.sorted, p->ps.perm, p->ps.tr,
                                      (const T *)p->ps.grid, nullptr, dscale, grad, s));
     }
-    p->launches += 3;
+    p->launches += 3 + (u->real ? 1 : 0);
     return un_status(cudaGetLastError());
 }
 
