@@ -61,12 +61,14 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_fwd(const 
     }
 }
 
-__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_inv(const __grid_constant__ FftDesc f,
-                                                      const float2 *__restrict__ bt,
-                                                      float *__restrict__ grid,
-                                                      const float2 *__restrict__ tws, int64_t rows,
-                                                      int kx, int64_t bt_stride,
-                                                      int64_t grid_stride) {
+// WEIGHTS: the result less (4 F / rho0) c, c the weights on the same grid and scal[0] = rho0, scal[3]
+// = F (the weight gradient's second term)
+template <bool WEIGHTS>
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_rows_inv(const __grid_constant__ FftDesc f, const float2 *__restrict__ bt,
+                   float *__restrict__ grid, const float2 *__restrict__ tws, int64_t rows, int kx,
+                   int64_t bt_stride, int64_t grid_stride, const float *__restrict__ c,
+                   const double *__restrict__ scal) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     float2 *s = reinterpret_cast<float2 *>(sm_raw);
     const int M = f.n, pitch = f.words;
@@ -91,8 +93,17 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_inv(const 
         if (km > half && km < M) s[row * pitch + fft_place(f, __ldg(f.pos + km))] = {-py + qx, px + qy};
     }
     __syncthreads();
-    fft_adjoint(f, nr, s, pitch,
-                [&](int row, int i, float2 v) { out[(int64_t)row * M + i] = {v.y, v.x}; });
+    if constexpr (WEIGHTS) {
+        const float coef = (float)(4.0 * scal[3] / scal[0]);
+        const float2 *cr = reinterpret_cast<const float2 *>(c) + r0 * M;
+        fft_adjoint(f, nr, s, pitch, [&](int row, int i, float2 v) {
+            const float2 w = cr[(int64_t)row * M + i];
+            out[(int64_t)row * M + i] = {v.y - coef * w.x, v.x - coef * w.y};
+        });
+    } else {
+        fft_adjoint(f, nr, s, pitch,
+                    [&](int row, int i, float2 v) { out[(int64_t)row * M + i] = {v.y, v.x}; });
+    }
 }
 
 __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_inv_c(const __grid_constant__ FftDesc f,
@@ -247,6 +258,87 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols_b(const __
                                    a.ip + I.ipo[0], a.ip + I.ipo[1]);
     const double b = block_sum(l);
     if (threadIdx.x == 0) a.partial[a.part_off[i] + k] = b;
+}
+
+// The columns of the weights-on-a-grid form (exact transforms, no kernel): S = |rho|^2 / rho0, the
+// loss and F = sum W S (S - S0), and (E / 2) rho, E = 4 W (S - S0) / rho0, back along y. Both sums
+// keep float pairs (products and sums with their errors) as the point form's loss does. scal[0] =
+// rho0 on entry; the last block leaves the loss (and its constant) in scal[2] and *loss, F in scal[3].
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_cols_w(const __grid_constant__ FftDesc f, const __grid_constant__ ColsArgs a,
+                 double loss_const, double *__restrict__ scal, double *__restrict__ loss,
+                 unsigned *__restrict__ done) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ bool s_last;
+    const int n = f.n, words = f.words, nbit = (words + 31) / 32, k = blockIdx.x;
+    float2 *s = reinterpret_cast<float2 *>(sm_raw);
+    unsigned *bits = reinterpret_cast<unsigned *>(s + words);
+    const int e0 = a.rep_first[k], e1 = a.rep_first[k + 1];
+    double bl = 0.0, bf = 0.0;
+    if (e0 != e1) {   // (a column without representatives stays zero from plan time)
+        for (int i = threadIdx.x; i < nbit; i += blockDim.x) bits[i] = 0;
+        const float2 *in = a.xt + (int64_t)k * n;
+        fft_forward(f, 1, s, 0, [&](int, int i) { return in[i]; });
+        const double inv_rho0 = 1.0 / scal[0];
+        const float inv = (float)inv_rho0;
+        float lh = 0.f, ll = 0.f, fh = 0.f, fl = 0.f;
+        for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+            const int ny = a.rep_n[2 * e + 1];
+            const int p = fft_place(f, __ldg(f.pos + (ny < 0 ? ny + n : ny)));
+            const float2 F = s[p];
+            const float S = (F.x * F.x + F.y * F.y) * inv, w = a.rep_w[e];
+            float dh, dl, sh, se;
+            two_sum(S, -a.rep_s0[e], dh, dl);
+            const float pr = dh * dh, pl = fmaf(2.f * dh, dl, fmaf(dh, dh, -pr));
+            const float th = w * pr, tl = fmaf(w, pl, fmaf(w, pr, -th));
+            two_sum(lh, th, sh, se);
+            lh = sh;
+            ll += se + tl;
+            const float ws = w * S, wse = fmaf(w, S, -ws);
+            const float uh = ws * dh, ul = fmaf(ws, dl, fmaf(wse, dh, fmaf(ws, dh, -uh)));
+            two_sum(fh, uh, sh, se);
+            fh = sh;
+            fl += se + ul;
+            const float h = (float)(2.0 * (double)w * ((double)dh + (double)dl) * inv_rho0);
+            s[p] = {h * F.y, h * F.x};   // parts exchanged for the inverse
+            atomicOr(&bits[p >> 5], 1u << (p & 31));
+            if (k == 0) {
+                const int p2 = fft_place(f, __ldg(f.pos + (ny > 0 ? n - ny : -ny)));
+                s[p2] = {-h * F.y, h * F.x};
+                atomicOr(&bits[p2 >> 5], 1u << (p2 & 31));
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < words; i += blockDim.x)
+            if (!(bits[i >> 5] >> (i & 31) & 1)) s[i] = {0.f, 0.f};
+        __syncthreads();
+        float2 *out = a.bt + (int64_t)k * n;
+        fft_adjoint(f, 1, s, 0, [&](int, int i, float2 v) { out[i] = {v.y, v.x}; });
+        bl = block_sum((double)lh + (double)ll);
+        bf = block_sum((double)fh + (double)fl);
+    }
+    if (threadIdx.x == 0) {
+        a.partial[k] = bl;
+        a.partial[gridDim.x + k] = bf;
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double v = 0.0, u = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
+        v += __ldcg(a.partial + i);
+        u += __ldcg(a.partial + gridDim.x + i);
+    }
+    v = block_sum(v);
+    u = block_sum(u);
+    if (threadIdx.x == 0) {
+        scal[2] = v + loss_const;
+        scal[3] = u;
+        *loss = v + loss_const;
+        *done = 0;
+    }
 }
 
 __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols_spec(const __grid_constant__ FftDesc f,
@@ -434,7 +526,9 @@ cudaError_t fft_allow_smem() {
     const int b = (int)kFftSmem;
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(k_fft_rows_fwd, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv<false>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv<true>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_w, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv_c, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols<true>, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols<false>, attr, b);
@@ -451,14 +545,14 @@ bool fft_cols_fit(const FftDesc &f, bool kderiv) {
 constexpr double kOwnCells = 1.2e6;
 
 fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int count,
-                            bool ensemble) {
+                            bool always) {
     const int64_t rows = (int64_t)nf[1] * nf[2] * count;
     // 2D single grids beyond kOwnCells stay on cuFFT, whose larger radices then outweigh its extra
     // passes over memory; ensembles (many grids, launches per size class) and the 3D rows do not.
     // Measured, x passes, y passes and mask, cuFFT against these kernels (us): 432^2 46 / 36, 784^2
     // 53 / 38, 2500^2 95 / 109, 6480^2 448 / 471; ensemble of 128 410 / 318; the 324^3 grid's x
     // passes with cuFFT's (z, y) transforms 468 / 374
-    if (dim == 2 && !ensemble && (double)nf[0] * nf[1] > kOwnCells) return FRESCO_OK;
+    if (dim == 2 && !always && (double)nf[0] * nf[1] > kOwnCells) return FRESCO_OK;
     // (the kernels work on whole rows of nf[0] floats; nf[0] is even)
     f.fwd = fft_describe(nf[0] / 2, f.x);
     f.inv = kderiv ? f.fwd : fft_describe(nf[0], f.xc);
@@ -511,8 +605,23 @@ cudaError_t fft_rows_inverse(const FftDesc &f, const float2 *bt, float *grid, co
                              int64_t rows, int kx, cudaStream_t s, int batch, int64_t bt_stride,
                              int64_t grid_stride) {
     const dim3 g((unsigned)((rows + f.rows - 1) / f.rows), 1, (unsigned)batch);
-    k_fft_rows_inv<<<g, f.threads, fft_bytes(f, f.rows), s>>>(f, bt, grid, tws, rows, kx,
-                                                                bt_stride, grid_stride);
+    k_fft_rows_inv<false><<<g, f.threads, fft_bytes(f, f.rows), s>>>(
+        f, bt, grid, tws, rows, kx, bt_stride, grid_stride, nullptr, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_rows_inverse_w(const FftDesc &f, const float2 *bt, float *grad, const float2 *tws,
+                               int64_t rows, int kx, const float *c, const double *scal,
+                               cudaStream_t s) {
+    k_fft_rows_inv<true><<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads,
+                           fft_bytes(f, f.rows), s>>>(f, bt, grad, tws, rows, kx, 0, 0, c, scal);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_cols_weights(const FftDesc &f, const ColsArgs &a, double loss_const, double *scal,
+                             double *loss, unsigned *done, cudaStream_t s) {
+    k_fft_cols_w<<<(unsigned)(a.m.kx + 1), f.threads, cols_bytes(f, 1), s>>>(f, a, loss_const, scal,
+                                                                             loss, done);
     return cudaGetLastError();
 }
 

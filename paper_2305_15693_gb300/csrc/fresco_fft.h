@@ -96,6 +96,14 @@ struct ColsBatch {
 };
 cudaError_t fft_cols_mask_b(const FftDesc &f, const ColsBatch &a, int count, bool kderiv,
                             cudaStream_t s);
+// The weights-on-a-grid form of the two kernels (fresco_uwu_*): the columns with that form's mask
+// (a.partial [2 (kx + 1)]; scal: rho0 in, loss and F out at 2 and 3), and the rows back less (4 F /
+// rho0) c.
+cudaError_t fft_cols_weights(const FftDesc &f, const ColsArgs &a, double loss_const, double *scal,
+                             double *loss, unsigned *done, cudaStream_t s);
+cudaError_t fft_rows_inverse_w(const FftDesc &f, const float2 *bt, float *grad, const float2 *tws,
+                               int64_t rows, int kx, const float *c, const double *scal,
+                               cudaStream_t s);
 // the column spectra themselves: out[k][row] = forward transform of xt[k] along y, in place allowed
 cudaError_t fft_cols_spectrum(const FftDesc &f, const float2 *xt, float2 *out, int kx,
                               cudaStream_t s);
@@ -113,10 +121,10 @@ struct FftSet {
     std::vector<void *> allocs;
     int64_t bytes = 0;
 };
-// Chooses and builds the transforms of `count` FP32 grids (of an ensemble, or one of a single plan);
-// steps whose lengths do not fit or that cuFFT runs faster keep cuFFT.
+// Chooses and builds the transforms of `count` FP32 grids; steps whose lengths do not fit keep cuFFT,
+// and, unless `always`, all of a 2D grid on which cuFFT's are the faster ones.
 fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int count,
-                            bool ensemble);
+                            bool always);
 void fft_set_free(FftSet *f);
 // first[k] = index of the first representative with n_x >= k, k = 0 .. kx + 1 (rep_n is n_x major)
 std::vector<int> rep_columns(const std::vector<int32_t> &rep_n, int dim, int kx);

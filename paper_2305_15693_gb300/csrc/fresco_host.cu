@@ -995,25 +995,23 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
                                           s));
         }
         if (own && own->cols) {
-        } else if (sizeof(T) == 4) {
+            // the y pass, the mask with its loss and the y pass back, column by column
+            fresco::ColsArgs a{m, (const float2 *)p->d_specT, (float2 *)p->d_bt[0], p->d_rep_n,
+                               (const float *)p->d_rep_s0, (const float *)p->d_rep_w,
+                               own->rep_first, (const float *)p->d_ip[0],
+                               (const float *)p->d_ip[1], p->d_partial};
+            FR_CUDA(fresco::fft_cols_mask(own->y, a, p->info.loss_const, loss, p->d_done, s));
+            p->launches += 1;
+            p->spec_ready = false;
+            p->forward_done = true;
+            return FRESCO_OK;
+        }
+        if (sizeof(T) == 4)
             FR_CUFFT(cufftExecC2C(p->fft_cols, (cufftComplex *)p->d_specT,
                                   (cufftComplex *)p->d_specT, CUFFT_FORWARD));
-        } else {
+        else
             FR_CUFFT(cufftExecZ2Z(p->fft_cols, (cufftDoubleComplex *)p->d_specT,
                                   (cufftDoubleComplex *)p->d_specT, CUFFT_FORWARD));
-        }
-    }
-    if (own && own->cols) {
-        // the y pass, the mask with its loss and the y pass back, column by column
-        StageScope sc(p->prof, p->stream, ST_MASK);
-        fresco::ColsArgs a{m, (const float2 *)p->d_specT, (float2 *)p->d_bt[0], p->d_rep_n,
-                           (const float *)p->d_rep_s0, (const float *)p->d_rep_w, own->rep_first,
-                           (const float *)p->d_ip[0], (const float *)p->d_ip[1], p->d_partial};
-        FR_CUDA(fresco::fft_cols_mask(own->y, a, p->info.loss_const, loss, p->d_done, s));
-        p->launches += 1;
-        p->spec_ready = false;
-        p->forward_done = true;
-        return FRESCO_OK;
     }
     {
         StageScope sc(p->prof, p->stream, ST_MASK);
@@ -1933,7 +1931,13 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
                 FR_CUDA(fresco::fft_rows_forward(K.own->x, (const float *)A, (float2 *)AT,
                                                  (const float2 *)b->tw + K.two0, plane, K.kx, s,
                                                  K.count, 2 * plane * mh, plane * (K.kx + 1)));
-                b->launches += 1;
+                // the y pass, the mask and the y pass back, column by column
+                fresco::ColsBatch a{b->d_inst, b->cls_list + K.list0, b->rep_first, b->rep_off,
+                                    (const float2 *)b->specT, (float2 *)b->bt, b->rep_n,
+                                    (const float *)b->rep_s0, (const float *)b->rep_w,
+                                    (const float *)b->ip, b->partial, b->d_mblk_first, K.kx};
+                FR_CUDA(fresco::fft_cols_mask_b(K.own->y, a, K.count, b->kderiv != 0, s));
+                b->launches += 2;
                 continue;
             }
             if (sizeof(T) == 4)
@@ -1953,22 +1957,11 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
             b->launches += 1;
         }
     }
-    {
+    if (!b->own_fft) {
         StageScope sc(b->prof, s, ST_MASK);
-        if (b->own_fft) {
-            for (auto &K : b->cls) {   // the y pass, the mask and the y pass back, column by column
-                fresco::ColsBatch a{b->d_inst, b->cls_list + K.list0, b->rep_first, b->rep_off,
-                                    (const float2 *)b->specT, (float2 *)b->bt, b->rep_n,
-                                    (const float *)b->rep_s0, (const float *)b->rep_w,
-                                    (const float *)b->ip, b->partial, b->d_mblk_first, K.kx};
-                FR_CUDA(fresco::fft_cols_mask_b(K.own->y, a, K.count, b->kderiv != 0, s));
-                b->launches += 1;
-            }
-        } else {
-            FR_CUDA(Launch<T>::mask_b(t, b->rep_n, (const T *)b->rep_s0, (const T *)b->rep_w,
-                                      b->specT, (const T *)b->ip, b->hc, nullptr, b->partial, s));
-            b->launches += 1;
-        }
+        FR_CUDA(Launch<T>::mask_b(t, b->rep_n, (const T *)b->rep_s0, (const T *)b->rep_w, b->specT,
+                                  (const T *)b->ip, b->hc, nullptr, b->partial, s));
+        b->launches += 1;
     }
     {
         StageScope sc(b->prof, s, ST_LOSS);
@@ -2237,15 +2230,33 @@ __device__ __forceinline__ double uwu_block_sum(double v) {
     return b;
 }
 
+// *out = sum c^2; the block that finishes last adds the partial sums in a fixed order
 template <typename T>
 __global__ void __launch_bounds__(256) k_uwu_sumsq(const T *__restrict__ c, int64_t n,
-                                                   double *__restrict__ part) {
-    double acc = 0.0;
+                                                   double *__restrict__ part,
+                                                   unsigned *__restrict__ done,
+                                                   double *__restrict__ out) {
+    __shared__ bool s_last;
+    fresco::DotAcc<T> acc;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        acc = fma((double)c[i], (double)c[i], acc);
-    const double b = uwu_block_sum(acc);
-    if (threadIdx.x == 0) part[blockIdx.x] = b;
+        acc.add(c[i], c[i]);
+    const double b = uwu_block_sum(acc.value());
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = b;
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double v = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) v += __ldcg(part + i);
+    const double s = uwu_block_sum(v);
+    if (threadIdx.x == 0) {
+        *out = s;
+        *done = 0;
+    }
 }
 
 // out[k] = sum of part[k * nb .. (k + 1) * nb) (+ add[k]) for k < n_out; fixed order
@@ -2326,7 +2337,10 @@ struct fresco_uwu_s {
     int *rep_n = nullptr;
     void *rep_s0 = nullptr, *rep_w = nullptr;
     void *spec = nullptr, *specT = nullptr, *hs = nullptr, *bt = nullptr, *r = nullptr, *h = nullptr;
-    double *part = nullptr, *scal = nullptr;   // scal[0] = rho0, scal[1] = F sum
+    double *part = nullptr, *scal = nullptr;   // scal[0] = rho0, [2] = loss, [3] = F sum
+    unsigned *done = nullptr;
+    fresco::FftSet *own = nullptr;             // 2D FP32 grids on the library's own transforms
+    void *tws = nullptr;                       // exp(-2 pi i k / M_0), k <= M_0 / 4
     void *work = nullptr;
     cufftHandle fft[4] = {0, 0, 0, 0};        // rows R2C, cols fwd, cols inv, rows C2R
     bool have[4] = {false, false, false, false};
@@ -2350,6 +2364,7 @@ void uwu_free(fresco_uwu_s *u) {
     else cudaDeviceSynchronize();
     for (int i = 0; i < 4; ++i)
         if (u->have[i]) cufftDestroy(u->fft[i]);
+    fresco::fft_set_free(u->own);
     for (void *p : u->allocs) cudaFree(p);
     delete u;
 }
@@ -2364,15 +2379,30 @@ fresco_status uwu_build(fresco_uwu_s *u, const Folded &F) {
     u->n_rep = (int64_t)F.s0.size();
     u->n_mask_blocks = std::max<int64_t>(1, std::min<int64_t>((u->n_rep + 255) / 256, kUwuBlocks));
     const size_t specT_n = (size_t)(u->kx + 1) * (size_t)u->plane;
+    if (sizeof(T) == 4 && dim == 2) {
+        u->own = new (std::nothrow) fresco::FftSet();
+        if (!u->own) return FRESCO_ERR_OOM;
+        const fresco_status st = fresco::fft_set_build(*u->own, u->M, 2, true, 1, true);
+        if (st) return st;
+        if (!u->own->cols) {
+            fresco::fft_set_free(u->own);
+            u->own = nullptr;
+        }
+    }
+    const bool lib = !u->own;   // the buffers of the cuFFT form
     bool ok = ualloc(u, (void **)&u->rep_n, sizeof(int) * F.n.size()) &&
               ualloc(u, &u->rep_s0, sizeof(T) * (size_t)u->n_rep) &&
               ualloc(u, &u->rep_w, sizeof(T) * (size_t)u->n_rep) &&
-              ualloc(u, &u->spec, sizeof(C2) * (size_t)(u->plane * u->half)) &&
-              ualloc(u, &u->specT, sizeof(C2) * specT_n) && ualloc(u, &u->hs, sizeof(C2) * specT_n) &&
+              (!lib || ualloc(u, &u->spec, sizeof(C2) * (size_t)(u->plane * u->half))) &&
+              ualloc(u, &u->specT, sizeof(C2) * specT_n) &&
+              (!lib || ualloc(u, &u->hs, sizeof(C2) * specT_n)) &&
               ualloc(u, &u->bt, sizeof(C2) * specT_n) &&
-              ualloc(u, &u->r, sizeof(C2) * (size_t)(u->plane * u->half)) &&
-              ualloc(u, &u->h, sizeof(T) * (size_t)u->cells) &&
-              ualloc(u, (void **)&u->part, sizeof(double) * (size_t)std::max<int64_t>(2 * u->n_mask_blocks, kUwuBlocks)) &&
+              (!lib || ualloc(u, &u->r, sizeof(C2) * (size_t)(u->plane * u->half))) &&
+              (!lib || ualloc(u, &u->h, sizeof(T) * (size_t)u->cells)) &&
+              ualloc(u, (void **)&u->part,
+                     sizeof(double) * (size_t)std::max<int64_t>(
+                                          {2 * u->n_mask_blocks, kUwuBlocks, 2 * (u->kx + 1)})) &&
+              ualloc(u, (void **)&u->done, sizeof(unsigned)) &&
               ualloc(u, (void **)&u->scal, sizeof(double) * 4);
     if (!ok) return FRESCO_ERR_OOM;
     std::vector<T> s0(F.s0.size()), w(F.w.size());
@@ -2383,6 +2413,25 @@ fresco_status uwu_build(fresco_uwu_s *u, const Folded &F) {
     FR_CUDA(cudaMemcpy(u->rep_n, F.n.data(), sizeof(int) * F.n.size(), cudaMemcpyHostToDevice));
     FR_CUDA(cudaMemcpy(u->rep_s0, s0.data(), sizeof(T) * s0.size(), cudaMemcpyHostToDevice));
     FR_CUDA(cudaMemcpy(u->rep_w, w.data(), sizeof(T) * w.size(), cudaMemcpyHostToDevice));
+    FR_CUDA(cudaMemset(u->done, 0, sizeof(unsigned)));
+    if (u->own) {
+        const std::vector<int> first = fresco::rep_columns(F.n, dim, u->kx);
+        std::vector<C2> tw((size_t)u->M[0] / 4 + 1);
+        for (size_t k = 0; k < tw.size(); ++k) {
+            const double a = 2.0 * M_PI * (double)k / (double)u->M[0];
+            tw[k].x = (T)std::cos(a);
+            tw[k].y = (T)-std::sin(a);
+        }
+        if (!ualloc(u, (void **)&u->own->rep_first, sizeof(int) * first.size()) ||
+            !ualloc(u, &u->tws, sizeof(C2) * tw.size()))
+            return FRESCO_ERR_OOM;
+        FR_CUDA(cudaMemcpy(u->own->rep_first, first.data(), sizeof(int) * first.size(),
+                           cudaMemcpyHostToDevice));
+        FR_CUDA(cudaMemcpy(u->tws, tw.data(), sizeof(C2) * tw.size(), cudaMemcpyHostToDevice));
+        FR_CUDA(cudaMemset(u->bt, 0, sizeof(C2) * specT_n));   // columns without a mask entry
+        FR_CUDA(cudaDeviceSynchronize());
+        return FRESCO_OK;
+    }
     // entries outside the mask stay zero from here on
     FR_CUDA(cudaMemset(u->hs, 0, sizeof(C2) * specT_n));
     FR_CUDA(cudaMemset(u->r, 0, sizeof(C2) * (size_t)(u->plane * u->half)));
@@ -2420,8 +2469,29 @@ fresco_status uwu_eval(fresco_uwu_s *u, const T *c, double *loss, T *grad) {
     using C2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
     cudaStream_t s = u->stream;
     // rho0 = sum c^2
-    k_uwu_sumsq<T><<<kUwuBlocks, 256, 0, s>>>(c, u->cells, u->part);
-    k_uwu_sum<<<1, 256, 0, s>>>(u->part, kUwuBlocks, 1, 0.0, u->scal);
+    k_uwu_sumsq<T><<<(unsigned)std::min<int64_t>((u->cells + 1023) / 1024, kUwuBlocks), 256, 0, s>>>(
+        c, u->cells, u->part, u->done, u->scal);
+    if (u->own) {
+        // four launches: rho0, x forward, y forward with the mask and y back, x back with the second
+        // term. 1536 x 1500 weights, K = 460: 135 -> 72 us
+        fresco::ColsArgs a{};
+        a.m.kx = u->kx;
+        a.xt = (const float2 *)u->specT;
+        a.bt = (float2 *)u->bt;
+        a.rep_n = u->rep_n;
+        a.rep_s0 = (const float *)u->rep_s0;
+        a.rep_w = (const float *)u->rep_w;
+        a.rep_first = u->own->rep_first;
+        a.partial = u->part;
+        FR_CUDA(fresco::fft_rows_forward(u->own->x, (const float *)c, (float2 *)u->specT,
+                                         (const float2 *)u->tws, u->plane, u->kx, s));
+        FR_CUDA(fresco::fft_cols_weights(u->own->y, a, u->loss_const, u->scal, loss, u->done, s));
+        if (grad)
+            FR_CUDA(fresco::fft_rows_inverse_w(u->own->x, (const float2 *)u->bt, (float *)grad,
+                                               (const float2 *)u->tws, u->plane, u->kx,
+                                               (const float *)c, u->scal, s));
+        return cuda_status(cudaGetLastError());
+    }
     // forward transform, columns n_x = 0..kx transposed
     if (sizeof(T) == 4)
         FR_CUFFT(cufftExecR2C(u->fft[0], (cufftReal *)c, (cufftComplex *)u->spec));

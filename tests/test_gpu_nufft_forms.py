@@ -136,3 +136,30 @@ def test_half_plane_weights_at_edge_frequencies(shape):
     assert abs(loss.item() - want_l) <= 1e-5 * abs(want_l)
     assert rel_l2(grad.double().cpu().numpy().reshape(-1), want_g) <= 1e-4
 
+
+@pytest.mark.parametrize("shape,K", [((4, 4), 1), ((64, 22), 9), ((26, 36), 11), ((12, 100), 5),
+                                     ((200, 18), 8), ((90, 84), 40), ((2, 2), 0)])
+def test_uniform_weights_on_own_and_library_transforms(shape, K):
+    """Grids whose lengths factor into the library's radices and grids that keep cuFFT (11, 13), a
+    one-sided mask with repeated rows among them; (2, 2) is refused, as its axes are too short."""
+    import torch
+    from paper_2305_15693_gb300 import fresco
+    g = inputs.rng(shape[0] + 7 * shape[1])
+    if K == 0:
+        with pytest.raises(fresco.FrescoError):
+            fresco.Uwu(shape, np.array([[0, 1]], dtype=np.int32), [0.0], [1.0], "f32")
+        return
+    mask = inputs.ball_mask(K, 2)
+    mask = np.vstack([mask[inputs.half_space(mask)], -mask[:3]])
+    c = g.standard_normal(int(np.prod(shape))).astype(np.float32)
+    S0, W = 0.3 * g.random(len(mask)), 0.2 + g.random(len(mask))
+    want_l, want_g, _, _ = oracle.weight_loss_grad(oracle.grid_points(shape), c.astype(np.float64),
+                                                   mask, S0, W)
+    with fresco.Uwu(shape, mask, S0, W, "f32") as u:
+        x = torch.from_numpy(c.reshape(shape[::-1])).cuda()
+        l0, _ = u.loss_grad(x, want_grad=False)
+        loss, grad = u.loss_grad(x)
+        torch.cuda.synchronize()
+    assert l0.item() == loss.item()
+    assert abs(loss.item() - want_l) <= 1e-5 * abs(want_l)
+    assert rel_l2(grad.double().cpu().numpy().reshape(-1), want_g) <= 1e-4
