@@ -10,8 +10,7 @@
 //   dL/dr_j = -sum_n k Im[A_j[n] (sum_m D+ B_j[m] + D- conj B_j[m])],
 // where the sums over m with and without the factors n_y, n_z share their loads. Three launches:
 //   k_direct_rho   one block per chunk of points: phases (kept for the gradient), then the sums of
-//                  its points for every quad of four n at one column; blocks (and thread groups
-//                  inside a block) leave partial sums;
+//                  its points for every quad of four n at one column; blocks leave partial sums;
 //   k_direct_mask  adds the partial sums in a fixed order, forms S, the loss (FP64) and D; the last
 //                  block to finish adds the loss partials in a fixed order;
 //   k_direct_grad  threads over (point, n), the block's points' B in shared memory.
@@ -150,13 +149,15 @@ __global__ void __launch_bounds__(kRhoThreads) k_direct_rho(DirectGeom g, const 
     }
     const int gt = blockDim.x / g.groups, grp = threadIdx.x / gt;
     const int64_t cells = 4 * (int64_t)g.n_quad;
-    T *out = part + (int64_t)(blockIdx.x * g.groups + grp) * 4 * cells;
-    for (int q = threadIdx.x - grp * gt; q < g.n_quad; q += gt) {
-        const int2 qm = quads[q];
+    T *out = part + (int64_t)blockIdx.x * 4 * cells;
+    // (several groups: a group has a thread for every quad, so the loop runs once)
+    for (int q = threadIdx.x - grp * gt; q < g.n_quad || g.groups > 1; q += gt) {
         T rr[4] = {}, ii[4] = {}, ri[4] = {}, ir[4] = {};
+        const bool in = q < g.n_quad;
+        const int2 qm = in ? quads[q] : make_int2(0, 0);
         const C *a = sa + 4 * qm.x, *b = sb + qm.y;
 #pragma unroll 4
-        for (int j = grp; j < n; j += g.groups) {
+        for (int j = in ? grp : n; j < n; j += g.groups) {
             const C v = b[j * g.n_col];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -167,6 +168,31 @@ __global__ void __launch_bounds__(kRhoThreads) k_direct_rho(DirectGeom g, const 
                 ir[k] = fma(u.y, v.x, ir[k]);
             }
         }
+        if (g.groups > 1) {
+            // the groups' sums through shared memory, added in order by the first one
+            __syncthreads();
+            T *red = reinterpret_cast<T *>(sm_raw);
+            if (grp && in)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    T *o = red + (size_t)((grp - 1) * 16 + 4 * k) * gt + q;
+                    o[0] = rr[k];
+                    o[gt] = ii[k];
+                    o[2 * gt] = ri[k];
+                    o[3 * gt] = ir[k];
+                }
+            __syncthreads();
+            if (grp || !in) return;
+            for (int h = 0; h < g.groups - 1; ++h)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const T *o = red + (size_t)(h * 16 + 4 * k) * gt + q;
+                    rr[k] += o[0];
+                    ii[k] += o[gt];
+                    ri[k] += o[2 * gt];
+                    ir[k] += o[3 * gt];
+                }
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             out[4 * (int64_t)q + k] = rr[k];
@@ -174,16 +200,17 @@ __global__ void __launch_bounds__(kRhoThreads) k_direct_rho(DirectGeom g, const 
             out[2 * cells + 4 * (int64_t)q + k] = ri[k];
             out[3 * cells + 4 * (int64_t)q + k] = ir[k];
         }
+        if (g.groups > 1) return;
     }
 }
 
 // kMaskCells cells per block: 32 threads per cell take every 32nd partial sum, then one warp per
-// cell adds their results. (32 cells per block of 1024 threads put all of a small problem on a
-// dozen SMs, whose FP64 pipes then took 40 us.)
+// cell adds their results. Few cells per block spread a small problem over the SMs: 1024 FP64 points
+// took 40 us with 32 cells a block, 15 with 8 and 18 with 4.
 constexpr int kMaskCells = 8;
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_direct_mask(DirectGeom g, int n_part,
+__global__ void __launch_bounds__(32 * kMaskCells) k_direct_mask(DirectGeom g, int n_part,
                                                      const T *__restrict__ part,
                                                      const T *__restrict__ cell_s0,
                                                      const T *__restrict__ cell_w,
@@ -221,33 +248,31 @@ __global__ void __launch_bounds__(256) k_direct_mask(DirectGeom g, int n_part,
         for (int k = 0; k < 4; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
     }
     const int64_t c = (int64_t)blockIdx.x * kMaskCells + wid;
-    if (lane == 0) {
+    if (lane < 2) {   // lane 0 the wavevector at +m, lane 1 the one at -m
         double l = 0.0;
+        C d{T(0), T(0)};
         if (c < cells) {
             const T inv_n = (T)g.inv_n;
-            C d[2];
-#pragma unroll
-            for (int sgn = 0; sgn < 2; ++sgn) {
-                C r;
-                r.x = sgn ? v[0] + v[1] : v[0] - v[1];
-                r.y = sgn ? v[2] - v[3] : -(v[2] + v[3]);
-                rho[2 * c + sgn] = r;
-                const T w = cell_w[2 * c + sgn], s0 = cell_s0[2 * c + sgn];
-                d[sgn] = C{T(0), T(0)};
-                if (w > T(0)) {
-                    const T S = (r.x * r.x + r.y * r.y) * inv_n;
-                    const double dv = (double)S - (double)s0;
-                    l = fma((double)w * dv, dv, l);
-                    const T e = T(4) * w * (T)dv * inv_n;
-                    d[sgn] = C{e * r.x, e * r.y};
-                }
+            C r;
+            r.x = lane ? v[0] + v[1] : v[0] - v[1];
+            r.y = lane ? v[2] - v[3] : -(v[2] + v[3]);
+            rho[2 * c + lane] = r;
+            const T w = cell_w[2 * c + lane], s0 = cell_s0[2 * c + lane];
+            if (w > T(0)) {
+                const T S = (r.x * r.x + r.y * r.y) * inv_n;
+                const double dv = (double)S - (double)s0;
+                l = (double)w * dv * dv;
+                const T e = T(4) * w * (T)dv * inv_n;
+                d = C{e * r.x, e * r.y};
             }
-            dco[4 * c] = d[0].x + d[1].x;
-            dco[4 * c + 1] = d[0].y + d[1].y;
-            dco[4 * c + 2] = d[0].x - d[1].x;
-            dco[4 * c + 3] = d[0].y - d[1].y;
         }
-        sl[wid] = l;
+        const T ox = __shfl_xor_sync(3u, d.x, 1), oy = __shfl_xor_sync(3u, d.y, 1);
+        l += __shfl_xor_sync(3u, l, 1);
+        if (c < cells) {   // D+ + D-, then D+ - D-
+            dco[4 * c + 2 * lane] = lane ? ox - d.x : d.x + ox;
+            dco[4 * c + 2 * lane + 1] = lane ? oy - d.y : d.y + oy;
+        }
+        if (lane == 0) sl[wid] = l;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -418,6 +443,13 @@ void size_chunks(DirectGeom &g) {
         g.groups *= 2;
 }
 
+// dynamic shared memory of k_direct_rho: the phases, or the groups' sums after them
+template <typename T>
+size_t direct_rho_bytes(const DirectGeom &g) {
+    const size_t red = (size_t)(g.groups - 1) * 16 * (kRhoThreads / g.groups) * sizeof(T);
+    return std::max(direct_rho_smem<T>(g, g.chunk), red);
+}
+
 }  // namespace
 
 struct DirectPlan {
@@ -464,7 +496,7 @@ static fresco_status build_t(DirectPlan *d, const std::vector<int2> &cols,
     DirectGeom &g = d->g;
     size_chunks<T>(g);
     const size_t cells = 4 * (size_t)g.n_quad;
-    const size_t n_part = (size_t)g.n_blk * g.groups;
+    const size_t n_part = (size_t)g.n_blk;
     d->n_mask_blk = (int)((cells + kMaskCells - 1) / kMaskCells);
     auto A = [&](void **p, size_t b) {
         if (cudaMalloc(p, std::max<size_t>(b, 16)) != cudaSuccess) {
@@ -629,7 +661,7 @@ fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const do
 template <typename T>
 cudaError_t direct_rho(DirectPlan *d, const T *pts, int *err, cudaStream_t s) {
     const DirectGeom &g = d->g;
-    const size_t smem = direct_rho_smem<T>(g, g.chunk);
+    const size_t smem = direct_rho_bytes<T>(g);
     const auto kern = g.dim == 2 ? k_direct_rho<T, 2> : k_direct_rho<T, 3>;
     kern<<<g.n_blk, kRhoThreads, smem, s>>>(g, pts, d->cols, d->quads, (Cx<T> *)d->tab, (T *)d->part, err);
     return cudaGetLastError();
@@ -639,7 +671,7 @@ template <typename T>
 cudaError_t direct_mask(DirectPlan *d, double *loss, cudaStream_t s) {
     const DirectGeom &g = d->g;
     k_direct_mask<T><<<d->n_mask_blk, 32 * kMaskCells, 0, s>>>(
-        g, g.n_blk * g.groups, (const T *)d->part, (const T *)d->cell_s0, (const T *)d->cell_w,
+        g, g.n_blk, (const T *)d->part, (const T *)d->cell_s0, (const T *)d->cell_w,
         (Cx<T> *)d->rho, (T *)d->dco, d->lpart, d->done, loss);
     return cudaGetLastError();
 }
