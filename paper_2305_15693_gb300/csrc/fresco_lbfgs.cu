@@ -183,25 +183,35 @@ __global__ void __cluster_dims__(kTlBlocks, 1, 1) __launch_bounds__(kTlThreads)
                const double *__restrict__ rho) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    __shared__ double slot[2][2];
+    constexpr int NW = kTlThreads / 32;
+    __shared__ double slot[2][NW];
     __shared__ double alpha[kMaxHistory];
     const int64_t i0 = (int64_t)blockIdx.x * kTlThreads + threadIdx.x;
     constexpr int64_t ST = kTlBlocks * kTlThreads;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int phase = 0;
-    // sums (or maxima) over the cluster of one value per thread, the same in every thread
-    auto total = [&](double v0, bool is_max) -> double {
-        double v[1] = {v0};
-        block_reduce<1, kTlThreads>(v, is_max);
-        if (threadIdx.x == 0) slot[phase][0] = v[0];
-        cl.sync();
-        double r = 0.0;
+    // sums (or maxima) over the cluster of one value per thread, the same in every thread: every warp
+    // leaves its own, and after one cluster barrier every warp adds all of them in the same tree
+    // (block sums first and their exchange after took 2.2 us a product at 2048 FP64 elements)
+    auto total = [&](double v, bool is_max) -> double {
 #pragma unroll
-        for (int b = 0; b < kTlBlocks; ++b) {
-            const double u = *cl.map_shared_rank(&slot[phase][0], b);
-            r = is_max ? fmax(r, u) : r + u;
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v, o);
+            v = is_max ? fmax(v, u) : v + u;
+        }
+        if (lane == 0) slot[phase][wid] = v;
+        cl.sync();
+        static_assert(kTlBlocks * NW == 64, "two values per lane");
+        const double a = *cl.map_shared_rank(&slot[phase][lane & (NW - 1)], lane / NW);
+        const double b = *cl.map_shared_rank(&slot[phase][lane & (NW - 1)], lane / NW + 32 / NW);
+        v = is_max ? fmax(a, b) : a + b;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v, o);
+            v = is_max ? fmax(v, u) : v + u;
         }
         phase ^= 1;   // the other buffer next: a block writes this one again only after the next
-        return r;     // exchange, which every block reaches after this read
+        return v;     // exchange, which every block reaches after this read
     };
     auto dot = [&](const T (&v)[E], const T *__restrict__ b) -> double {
         fresco::DotAcc<T> acc;
