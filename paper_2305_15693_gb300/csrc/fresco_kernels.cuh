@@ -1861,11 +1861,11 @@ cudaError_t Launch<T>::place_direct(const Geom &g, const T *points, int64_t j0, 
                                     void *sorted, int *perm, int *err, cudaStream_t s) {
     using U = typename PT<T>::U;
     constexpr int IL = kDirectPointsPerThread;
-    const int grid = grid_for((g.n_points + IL - 1) / IL, 256, 152 * 16);
-    if (g.dim == 2)
-        k_place_direct<T, 2><<<grid, 256, 0, s>>>(g, points, j0, tcur, (U *)sorted, perm, err);
-    else
-        k_place_direct<T, 3><<<grid, 256, 0, s>>>(g, points, j0, tcur, (U *)sorted, perm, err);
+    const bool many = g.n_points >= (int64_t)152 * 2 * 256 * IL;
+    const int grid = grid_for(many ? (g.n_points + IL - 1) / IL : g.n_points, 256, 152 * 16);
+    const auto kern = g.dim == 2 ? (many ? k_place_direct<T, 2, IL> : k_place_direct<T, 2, 1>)
+                                 : (many ? k_place_direct<T, 3, IL> : k_place_direct<T, 3, 1>);
+    kern<<<grid, 256, 0, s>>>(g, points, j0, tcur, (U *)sorted, perm, err);
     return cudaGetLastError();
 }
 
