@@ -29,20 +29,16 @@ using namespace fft_detail;
 
 namespace {
 
-__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_fwd(const __grid_constant__ FftDesc f,
-                                                      const float *__restrict__ grid,
-                                                      float2 *__restrict__ xt,
-                                                      const float2 *__restrict__ tws, int64_t rows,
-                                                      int kx, int64_t grid_stride,
-                                                      int64_t xt_stride) {
+// Rows r0 .. of one grid, f.rows of them, in each of the next three; rows: the grid's.
+__device__ __forceinline__ void rows_fwd(const FftDesc &f, const float *__restrict__ grid,
+                                         float2 *__restrict__ xt, const float2 *__restrict__ tws,
+                                         int64_t rows, int64_t r0, int kx) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     float2 *s = reinterpret_cast<float2 *>(sm_raw);
     const int M = f.n, pitch = f.words;
-    const int64_t r0 = (int64_t)blockIdx.x * f.rows;
     const int nr = (int)min((int64_t)f.rows, rows - r0);
-    const float2 *in =
-        reinterpret_cast<const float2 *>(grid + (int64_t)blockIdx.z * grid_stride) + r0 * M;
-    xt += (int64_t)blockIdx.z * xt_stride + r0;
+    const float2 *in = reinterpret_cast<const float2 *>(grid) + r0 * M;
+    xt += r0;
     fft_forward(f, nr, s, pitch, [&](int row, int i) { return in[(int64_t)row * M + i]; });
     // X[k] = E + tau_k O and X[M - k] = conj(E - tau_k O) from Z[k], Z[M - k] (as k_rfft_split_cols)
     const int half = M / 2, shift = __popc(f.rows - 1);   // f.rows is a power of two
@@ -64,18 +60,17 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_fwd(const 
 // WEIGHTS: the result less (4 F / rho0) c, c the weights on the same grid and scal[0] = rho0, scal[3]
 // = F (the weight gradient's second term)
 template <bool WEIGHTS>
-__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
-    k_fft_rows_inv(const __grid_constant__ FftDesc f, const float2 *__restrict__ bt,
-                   float *__restrict__ grid, const float2 *__restrict__ tws, int64_t rows, int kx,
-                   int64_t bt_stride, int64_t grid_stride, const float *__restrict__ c,
-                   const double *__restrict__ scal) {
+__device__ __forceinline__ void rows_inv(const FftDesc &f, const float2 *__restrict__ bt,
+                                         float *__restrict__ grid, const float2 *__restrict__ tws,
+                                         int64_t rows, int64_t r0, int kx,
+                                         const float *__restrict__ c,
+                                         const double *__restrict__ scal) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     float2 *s = reinterpret_cast<float2 *>(sm_raw);
     const int M = f.n, pitch = f.words;
-    const int64_t r0 = (int64_t)blockIdx.x * f.rows;
     const int nr = (int)min((int64_t)f.rows, rows - r0);
-    bt += (int64_t)blockIdx.z * bt_stride + r0;
-    float2 *out = reinterpret_cast<float2 *>(grid + (int64_t)blockIdx.z * grid_stride) + r0 * M;
+    bt += r0;
+    float2 *out = reinterpret_cast<float2 *>(grid) + r0 * M;
     // Z[k] = P + i Q, Z[M - k] = conj P + i conj Q (as k_rfft_merge_rows), parts exchanged
     const int half = M / 2, shift = __popc(f.rows - 1);
     for (int t = threadIdx.x; t < (half + 1) << shift; t += blockDim.x) {
@@ -106,18 +101,15 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
     }
 }
 
-__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_inv_c(const __grid_constant__ FftDesc f,
-                                                        const float2 *__restrict__ bt,
-                                                        float2 *__restrict__ g, int64_t rows,
-                                                        int kx, int64_t bt_stride,
-                                                        int64_t g_stride) {
+__device__ __forceinline__ void rows_inv_c(const FftDesc &f, const float2 *__restrict__ bt,
+                                           float2 *__restrict__ g, int64_t rows, int64_t r0,
+                                           int kx) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     float2 *s = reinterpret_cast<float2 *>(sm_raw);
     const int n = f.n, pitch = f.words;
-    const int64_t r0 = (int64_t)blockIdx.x * f.rows;
     const int nr = (int)min((int64_t)f.rows, rows - r0);
-    bt += (int64_t)blockIdx.z * bt_stride + r0;
-    g += (int64_t)blockIdx.z * g_stride + r0 * n;
+    bt += r0;
+    g += r0 * n;
     const int shift = __popc(f.rows - 1), ncol = 2 * kx + 2;
     for (int t = threadIdx.x; t < n << shift; t += blockDim.x) {
         const int row = t & (f.rows - 1), x = t >> shift;
@@ -131,6 +123,67 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_rows_inv_c(cons
     __syncthreads();
     fft_adjoint(f, nr, s, pitch,
                 [&](int row, int i, float2 v) { g[(int64_t)row * n + i] = {v.y, v.x}; });
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_rows_fwd(const __grid_constant__ FftDesc f, const float *__restrict__ grid,
+                   float2 *__restrict__ xt, const float2 *__restrict__ tws, int64_t rows, int kx) {
+    rows_fwd(f, grid, xt, tws, rows, (int64_t)blockIdx.x * f.rows, kx);
+}
+
+template <bool WEIGHTS>
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_rows_inv(const __grid_constant__ FftDesc f, const float2 *__restrict__ bt,
+                   float *__restrict__ grid, const float2 *__restrict__ tws, int64_t rows, int kx,
+                   const float *__restrict__ c, const double *__restrict__ scal) {
+    rows_inv<WEIGHTS>(f, bt, grid, tws, rows, (int64_t)blockIdx.x * f.rows, kx, c, scal);
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_rows_inv_c(const __grid_constant__ FftDesc f, const float2 *__restrict__ bt,
+                     float2 *__restrict__ g, int64_t rows, int kx) {
+    rows_inv_c(f, bt, g, rows, (int64_t)blockIdx.x * f.rows, kx);
+}
+
+// The size classes of an ensemble in one launch: a class's blocks alone leave most SMs idle and each
+// launch waits for the last of the one before. An ensemble of 128 in nine classes: 27 launches of 4
+// to 36 us, 323 us in all, now three of 52, 65 and 57.
+__device__ __forceinline__ int class_of(const FftClassSet &q, int &block) {
+    int i = 0;
+    while (i + 1 < q.n && (int)blockIdx.x >= q.first[i + 1]) ++i;
+    block = (int)blockIdx.x - q.first[i];
+    return i;
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_rows_fwd_b(const __grid_constant__ FftClassSet q, const float *__restrict__ grid,
+                     float2 *__restrict__ xt, const float2 *__restrict__ tws) {
+    int b;
+    const FftClass &c = q.c[class_of(q, b)];
+    const int z = b / c.blocks;
+    rows_fwd(c.f, grid + c.in0 + z * c.in_stride, xt + c.out0 + z * c.out_stride, tws + c.tw0,
+             c.rows, (int64_t)(b - z * c.blocks) * c.f.rows, c.kx);
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_rows_inv_b(const __grid_constant__ FftClassSet q, const float2 *__restrict__ bt,
+                     float *__restrict__ grid, const float2 *__restrict__ tws) {
+    int b;
+    const FftClass &c = q.c[class_of(q, b)];
+    const int z = b / c.blocks;
+    rows_inv<false>(c.f, bt + c.in0 + z * c.in_stride, grid + c.out0 + z * c.out_stride,
+                    tws + c.tw0, c.rows, (int64_t)(b - z * c.blocks) * c.f.rows, c.kx, nullptr,
+                    nullptr);
+}
+
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_rows_inv_cb(const __grid_constant__ FftClassSet q, const float2 *__restrict__ bt,
+                      float2 *__restrict__ g) {
+    int b;
+    const FftClass &c = q.c[class_of(q, b)];
+    const int z = b / c.blocks;
+    rows_inv_c(c.f, bt + c.in0 + z * c.in_stride, g + c.out0 + z * c.out_stride, c.rows,
+               (int64_t)(b - z * c.blocks) * c.f.rows, c.kx);
 }
 
 // One column of the 2D problem (see k_mask for the mask's arithmetic; the thread's loss terms are an
@@ -215,10 +268,9 @@ __device__ __forceinline__ double cols_column(const FftDesc &f, const MaskGeom &
 }
 
 template <bool KD>
-__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols(const __grid_constant__ FftDesc f,
-                                                  const __grid_constant__ ColsArgs a,
-                                                  double loss_const, double *__restrict__ loss,
-                                                  unsigned *__restrict__ done) {
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_cols(const __grid_constant__ FftDesc f, const __grid_constant__ ColsArgs a,
+               double loss_const, double *__restrict__ loss, unsigned *__restrict__ done) {
     __shared__ bool s_last;
     const int k = blockIdx.x, e0 = a.rep_first[k], e1 = a.rep_first[k + 1];
     // (a column without representatives stays zero from plan time)
@@ -245,15 +297,17 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols(const __gr
 }
 
 template <bool KD>
-__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols_b(const __grid_constant__ FftDesc f,
-                                                    const __grid_constant__ ColsBatch a) {
-    const int i = a.list[blockIdx.y], k = blockIdx.x;
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_cols_b(const __grid_constant__ FftClassSet q, const __grid_constant__ ColsBatch a) {
+    int b0;
+    const FftClass &c = q.c[class_of(q, b0)];
+    const int z = b0 / c.blocks, i = a.list[c.list0 + z], k = b0 - z * c.blocks;
     const BInst &I = a.inst[i];
     const int *first = a.rep_first + a.rep_off[i];
     const int e0 = first[k], e1 = first[k + 1];
     const double l =
         e0 == e1 ? 0.0
-                 : cols_column<KD>(f, I.m, k, a.xt + I.ato + (int64_t)k * f.n, a.bt + I.hco,
+                 : cols_column<KD>(c.f, I.m, k, a.xt + I.ato + (int64_t)k * c.f.n, a.bt + I.hco,
                                    a.rep_n + 2 * I.reo, a.rep_s0 + I.reo, a.rep_w + I.reo, e0, e1,
                                    a.ip + I.ipo[0], a.ip + I.ipo[1]);
     const double b = block_sum(l);
@@ -341,8 +395,8 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
     }
 }
 
-__global__ void __launch_bounds__(kFftThreads, kFftBlocks) k_fft_cols_spec(const __grid_constant__ FftDesc f,
-                                                       const float2 *xt, float2 *out) {
+__global__ void __launch_bounds__(kFftThreads, kFftBlocks)
+    k_fft_cols_spec(const __grid_constant__ FftDesc f, const float2 *xt, float2 *out) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     float2 *s = reinterpret_cast<float2 *>(sm_raw);
     const float2 *in = xt + (int64_t)blockIdx.x * f.n;
@@ -482,24 +536,33 @@ fresco_status fft_tables(FftDesc &f, std::vector<void *> &allocs, int64_t &bytes
     return FRESCO_OK;
 }
 
-// Threads (a multiple of 32, from 64) that leave the fewest idle lanes over the passes of `rows`
-// transforms, preferring more of them where it is close: cost = passes' steps x threads.
-static int fft_threads(const FftDesc &f, int rows) {
+// Steps x threads of the passes of `rows` transforms (idle lanes included), fewer threads dearer where
+// it is close.
+static double thread_cost(const FftDesc &f, int rows, int t) {
+    double cost = 0.0;
+    for (int p = 0; p < f.np; ++p) {
+        const int nb = rows * (f.n / f.r[p]);
+        cost += (double)((nb + t - 1) / t) * t * f.r[p];
+    }
+    return cost * (1.0 + 0.25 * 64.0 / t);
+}
+
+// the number of threads (a multiple of 32, from 64) of least cost
+template <class Cost>
+static int least_threads(Cost cost) {
     int best = 64;
     double best_cost = 1e300;
     for (int t = 64; t <= kFftThreads; t += 32) {
-        double cost = 0.0;
-        for (int p = 0; p < f.np; ++p) {
-            const int nb = rows * (f.n / f.r[p]);
-            cost += (double)((nb + t - 1) / t) * t * f.r[p];
-        }
-        cost *= 1.0 + 0.25 * 64.0 / t;
-        if (cost < best_cost) {
-            best_cost = cost;
+        const double c = cost(t);
+        if (c < best_cost) {
+            best_cost = c;
             best = t;
         }
     }
     return best;
+}
+static int fft_threads(const FftDesc &f, int rows) {
+    return least_threads([&](int t) { return thread_cost(f, rows, t); });
 }
 
 void fft_size_rows(FftDesc &f, int64_t rows) {
@@ -532,6 +595,9 @@ cudaError_t fft_allow_smem() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv_c, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols<true>, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols<false>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_fwd_b, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv_b, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv_cb, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_b<true>, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_b<false>, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_spec, attr, b);
@@ -544,13 +610,12 @@ bool fft_cols_fit(const FftDesc &f, bool kderiv) {
 
 constexpr double kOwnCells = 1.2e6;
 
-fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int count,
+fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int64_t rows,
                             bool always) {
-    const int64_t rows = (int64_t)nf[1] * nf[2] * count;
     // 2D single grids beyond kOwnCells stay on cuFFT, whose larger radices then outweigh its extra
     // passes over memory; ensembles (many grids, launches per size class) and the 3D rows do not.
     // Measured, x passes, y passes and mask, cuFFT against these kernels (us): 432^2 46 / 36, 784^2
-    // 53 / 38, 2500^2 95 / 109, 6480^2 448 / 471; ensemble of 128 410 / 318; the 324^3 grid's x
+    // 53 / 38, 2500^2 95 / 109, 6480^2 448 / 471; ensemble of 128 410 / 173; the 324^3 grid's x
     // passes with cuFFT's (z, y) transforms 468 / 374
     if (dim == 2 && !always && (double)nf[0] * nf[1] > kOwnCells) return FRESCO_OK;
     // (the kernels work on whole rows of nf[0] floats; nf[0] is even)
@@ -593,20 +658,16 @@ std::vector<int> rep_columns(const std::vector<int32_t> &rep_n, int dim, int kx)
 }
 
 cudaError_t fft_rows_forward(const FftDesc &f, const float *grid, float2 *xt, const float2 *tws,
-                             int64_t rows, int kx, cudaStream_t s, int batch, int64_t grid_stride,
-                             int64_t xt_stride) {
-    const dim3 g((unsigned)((rows + f.rows - 1) / f.rows), 1, (unsigned)batch);
-    k_fft_rows_fwd<<<g, f.threads, fft_bytes(f, f.rows), s>>>(f, grid, xt, tws, rows, kx,
-                                                                grid_stride, xt_stride);
+                             int64_t rows, int kx, cudaStream_t s) {
+    k_fft_rows_fwd<<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads, fft_bytes(f, f.rows), s>>>(
+        f, grid, xt, tws, rows, kx);
     return cudaGetLastError();
 }
 
 cudaError_t fft_rows_inverse(const FftDesc &f, const float2 *bt, float *grid, const float2 *tws,
-                             int64_t rows, int kx, cudaStream_t s, int batch, int64_t bt_stride,
-                             int64_t grid_stride) {
-    const dim3 g((unsigned)((rows + f.rows - 1) / f.rows), 1, (unsigned)batch);
-    k_fft_rows_inv<false><<<g, f.threads, fft_bytes(f, f.rows), s>>>(
-        f, bt, grid, tws, rows, kx, bt_stride, grid_stride, nullptr, nullptr);
+                             int64_t rows, int kx, cudaStream_t s) {
+    k_fft_rows_inv<false><<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads,
+                            fft_bytes(f, f.rows), s>>>(f, bt, grid, tws, rows, kx, nullptr, nullptr);
     return cudaGetLastError();
 }
 
@@ -614,7 +675,7 @@ cudaError_t fft_rows_inverse_w(const FftDesc &f, const float2 *bt, float *grad, 
                                int64_t rows, int kx, const float *c, const double *scal,
                                cudaStream_t s) {
     k_fft_rows_inv<true><<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads,
-                           fft_bytes(f, f.rows), s>>>(f, bt, grad, tws, rows, kx, 0, 0, c, scal);
+                           fft_bytes(f, f.rows), s>>>(f, bt, grad, tws, rows, kx, c, scal);
     return cudaGetLastError();
 }
 
@@ -626,10 +687,9 @@ cudaError_t fft_cols_weights(const FftDesc &f, const ColsArgs &a, double loss_co
 }
 
 cudaError_t fft_rows_inverse_c(const FftDesc &f, const float2 *bt, float2 *g, int64_t rows, int kx,
-                               cudaStream_t s, int batch, int64_t bt_stride, int64_t g_stride) {
-    const dim3 gr((unsigned)((rows + f.rows - 1) / f.rows), 1, (unsigned)batch);
-    k_fft_rows_inv_c<<<gr, f.threads, fft_bytes(f, f.rows), s>>>(f, bt, g, rows, kx, bt_stride,
-                                                                   g_stride);
+                               cudaStream_t s) {
+    k_fft_rows_inv_c<<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads, fft_bytes(f, f.rows),
+                       s>>>(f, bt, g, rows, kx);
     return cudaGetLastError();
 }
 
@@ -643,11 +703,63 @@ cudaError_t fft_cols_mask(const FftDesc &f, const ColsArgs &a, double loss_const
     return cudaGetLastError();
 }
 
-cudaError_t fft_cols_mask_b(const FftDesc &f, const ColsBatch &a, int count, bool kderiv,
-                            cudaStream_t s) {
-    const dim3 g((unsigned)(a.kx + 1), (unsigned)count);
-    if (kderiv) k_fft_cols_b<true><<<g, f.threads, cols_bytes(f, 1), s>>>(f, a);
-    else k_fft_cols_b<false><<<g, f.threads, cols_bytes(f, 2), s>>>(f, a);
+std::vector<FftClassSet> fft_class_sets(std::vector<FftClass> cls, int col_buffers) {
+    auto bytes = [&](const FftClass &c) {
+        return col_buffers ? cols_bytes(c.f, col_buffers) : fft_bytes(c.f, c.f.rows);
+    };
+    // the blocks that take longest first
+    std::stable_sort(cls.begin(), cls.end(), [&](const FftClass &a, const FftClass &b) {
+        return bytes(a) > bytes(b);
+    });
+    std::vector<FftClassSet> out;
+    for (const FftClass &c : cls) {
+        // a class whose blocks need much less shared memory than those that set a launch's residency
+        // (below kFftBlocks) starts another launch
+        const bool apart = !out.empty() && out.back().smem * kFftBlocks > kFftSmem &&
+                           2 * bytes(c) <= out.back().smem;
+        const int64_t blocks = (int64_t)c.blocks * c.count;
+        if (out.empty() || out.back().n == kFftClasses || apart ||
+            out.back().first[out.back().n] + blocks > 2147483647LL) {
+            out.emplace_back();
+            out.back().smem = bytes(c);
+        }
+        FftClassSet &q = out.back();
+        q.c[q.n] = c;
+        q.first[q.n + 1] = (int)(q.first[q.n] + blocks);
+        ++q.n;
+    }
+    for (FftClassSet &q : out)
+        q.threads = least_threads([&](int t) {
+            double cost = 0.0;
+            for (int i = 0; i < q.n; ++i)
+                cost += (double)q.c[i].blocks * q.c[i].count *
+                        thread_cost(q.c[i].f, q.c[i].f.rows, t);
+            return cost;
+        });
+    return out;
+}
+
+cudaError_t fft_rows_forward_b(const FftClassSet &q, const float *grid, float2 *xt,
+                               const float2 *tws, cudaStream_t s) {
+    k_fft_rows_fwd_b<<<(unsigned)q.first[q.n], q.threads, q.smem, s>>>(q, grid, xt, tws);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_rows_inverse_b(const FftClassSet &q, const float2 *bt, float *grid,
+                               const float2 *tws, cudaStream_t s) {
+    k_fft_rows_inv_b<<<(unsigned)q.first[q.n], q.threads, q.smem, s>>>(q, bt, grid, tws);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_rows_inverse_cb(const FftClassSet &q, const float2 *bt, float2 *g, cudaStream_t s) {
+    k_fft_rows_inv_cb<<<(unsigned)q.first[q.n], q.threads, q.smem, s>>>(q, bt, g);
+    return cudaGetLastError();
+}
+
+cudaError_t fft_cols_mask_b(const FftClassSet &q, const ColsBatch &a, bool kderiv, cudaStream_t s) {
+    const unsigned g = (unsigned)q.first[q.n];
+    if (kderiv) k_fft_cols_b<true><<<g, q.threads, q.smem, s>>>(q, a);
+    else k_fft_cols_b<false><<<g, q.threads, q.smem, s>>>(q, a);
     return cudaGetLastError();
 }
 

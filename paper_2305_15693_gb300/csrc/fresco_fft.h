@@ -55,16 +55,13 @@ void fft_size_cols(FftDesc &f);
 // Real rows of 2 M floats -> columns k = 0 .. kx of their half spectra, transposed: xt[k][row].
 // f: the transform of length M; tws: exp(-2 pi i k / 2M), k <= M / 2.
 cudaError_t fft_rows_forward(const FftDesc &f, const float *grid, float2 *xt, const float2 *tws,
-                             int64_t rows, int kx, cudaStream_t s, int batch = 1,
-                             int64_t grid_stride = 0, int64_t xt_stride = 0);
+                             int64_t rows, int kx, cudaStream_t s);
 // The inverse: transposed half spectra bt[k][row], k = 0 .. kx, -> real rows.
 cudaError_t fft_rows_inverse(const FftDesc &f, const float2 *bt, float *grid, const float2 *tws,
-                             int64_t rows, int kx, cudaStream_t s, int batch = 1,
-                             int64_t bt_stride = 0, int64_t grid_stride = 0);
+                             int64_t rows, int kx, cudaStream_t s);
 // Transposed columns bt[c][row], c = 0 .. 2 kx + 1 for n_x = c - kx - 1, -> complex rows of length n.
 cudaError_t fft_rows_inverse_c(const FftDesc &f, const float2 *bt, float2 *g, int64_t rows, int kx,
-                               cudaStream_t s, int batch = 1, int64_t bt_stride = 0,
-                               int64_t g_stride = 0);
+                               cudaStream_t s);
 
 // 2D column pass: for every column n_x = 0 .. kx, the forward transform along y, the mask (S, loss,
 // gradient coefficients) and the inverse transform, in shared memory.
@@ -80,10 +77,34 @@ struct ColsArgs {
 };
 cudaError_t fft_cols_mask(const FftDesc &f, const ColsArgs &a, double loss_const, double *loss,
                           unsigned *done, cudaStream_t s);
-// the same over every instance of a batch class: block (column, z) works on instance inst[z]
+// The same steps for the size classes of an ensemble, up to kFftClasses of them in a launch: blocks
+// first[i] .. first[i + 1] - 1 work on class i, `blocks` of them on each of its `count` grids.
+constexpr int kFftClasses = 16;
+struct FftClass {
+    FftDesc f;
+    int64_t in0 = 0, in_stride = 0;     // the first grid's input and the next one's, in elements
+    int64_t out0 = 0, out_stride = 0;
+    int64_t tw0 = 0;                    // row steps: the class's part of the twiddles
+    int rows = 0, kx = 0, blocks = 0, count = 0;
+    int list0 = 0;                      // column step: the class's first entry of ColsBatch::list
+};
+struct FftClassSet {
+    int n = 0, threads = 0;
+    size_t smem = 0;
+    int first[kFftClasses + 1] = {};
+    FftClass c[kFftClasses];
+};
+static_assert(sizeof(FftClassSet) <= 16384, "passed as a kernel argument");
+// launches for the classes of one step; col_buffers: buffers of a column (0: a row step)
+std::vector<FftClassSet> fft_class_sets(std::vector<FftClass> cls, int col_buffers);
+cudaError_t fft_rows_forward_b(const FftClassSet &q, const float *grid, float2 *xt,
+                               const float2 *tws, cudaStream_t s);
+cudaError_t fft_rows_inverse_b(const FftClassSet &q, const float2 *bt, float *grid,
+                               const float2 *tws, cudaStream_t s);
+cudaError_t fft_rows_inverse_cb(const FftClassSet &q, const float2 *bt, float2 *g, cudaStream_t s);
 struct ColsBatch {
     const BInst *inst;
-    const int *list;              // instances of the class
+    const int *list;              // instances, class by class
     const int *rep_first;         // per instance at rep_off[i]
     const int64_t *rep_off;
     const float2 *xt;
@@ -92,10 +113,8 @@ struct ColsBatch {
     const float *rep_s0, *rep_w, *ip;
     double *partial;              // instance i's columns at partial + part_off[i]
     const int64_t *part_off;
-    int kx;
 };
-cudaError_t fft_cols_mask_b(const FftDesc &f, const ColsBatch &a, int count, bool kderiv,
-                            cudaStream_t s);
+cudaError_t fft_cols_mask_b(const FftClassSet &q, const ColsBatch &a, bool kderiv, cudaStream_t s);
 // The weights-on-a-grid form of the two kernels (fresco_uwu_*): the columns with that form's mask
 // (a.partial [2 (kx + 1)]; scal: rho0 in, loss and F out at 2 and 3), and the rows back less (4 F /
 // rho0) c.
@@ -121,9 +140,9 @@ struct FftSet {
     std::vector<void *> allocs;
     int64_t bytes = 0;
 };
-// Chooses and builds the transforms of `count` FP32 grids; steps whose lengths do not fit keep cuFFT,
-// and, unless `always`, all of a 2D grid on which cuFFT's are the faster ones.
-fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int count,
+// Chooses and builds the transforms of an FP32 grid, `rows` rows to a launch; steps whose lengths do
+// not fit keep cuFFT, and, unless `always`, all of a 2D grid on which cuFFT's are the faster ones.
+fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int64_t rows,
                             bool always);
 void fft_set_free(FftSet *f);
 // first[k] = index of the first representative with n_x >= k, k = 0 .. kx + 1 (rep_n is n_x major)

@@ -798,7 +798,8 @@ fresco_status build_plan(fresco_plan_s *p, const Params &P, const Folded &F) {
         p->own_fft = new (std::nothrow) fresco::FftSet();
         if (!p->own_fft) return FRESCO_ERR_OOM;
         fresco::FftSet &f = *p->own_fft;
-        if ((st = fresco::fft_set_build(f, P.nf, dim, m.kderiv != 0, 1, false))) return st;
+        if ((st = fresco::fft_set_build(f, P.nf, dim, m.kderiv != 0,
+                                        (int64_t)P.nf[1] * P.nf[2], false))) return st;
         if (f.cols) {
             const std::vector<int> first = fresco::rep_columns(F.n, dim, m.kx);
             if ((st = dalloc(p, &f.rep_first, sizeof(int) * first.size()))) return st;
@@ -1643,12 +1644,14 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
     // FP32 ensembles whose every size class fits run the library's own transforms; an instance's loss
     // partials are then one per column of its class
     b->own_fft = sizeof(T) == 4;
+    int64_t all_rows = 0;
+    for (auto &K : b->cls) all_rows += (int64_t)K.nf[1] * K.count;
     for (auto &K : b->cls) {
         if (!b->own_fft) break;
         K.own = new (std::nothrow) fresco::FftSet();
         if (!K.own) return FRESCO_ERR_OOM;
         const int nf[3] = {K.nf[0], K.nf[1], 1};
-        const fresco_status st = fresco::fft_set_build(*K.own, nf, 2, b->kderiv != 0, K.count, true);
+        const fresco_status st = fresco::fft_set_build(*K.own, nf, 2, b->kderiv != 0, all_rows, true);
         if (st) return st;
         b->own_fft = K.own->cols;
     }
@@ -1803,6 +1806,37 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
                 const std::vector<int> f = fresco::rep_columns(F[i].n, dim, b->cls[cls_of[i]].kx);
                 first.insert(first.end(), f.begin(), f.end());
             }
+            // the classes of each step, together in as few launches as they fit
+            std::vector<fresco::FftClass> fwd, col, inv;
+            for (const auto &K : b->cls) {
+                const int64_t plane = K.nf[1], cells = (int64_t)K.nf[0] * plane;
+                fresco::FftClass c;
+                c.kx = K.kx;
+                c.count = K.count;
+                c.rows = K.nf[1];
+                c.tw0 = K.two0;
+                c.f = K.own->x;
+                c.blocks = (c.rows + c.f.rows - 1) / c.f.rows;
+                c.in0 = K.go0;
+                c.in_stride = cells;
+                c.out0 = K.ato0;
+                c.out_stride = plane * (K.kx + 1);
+                fwd.push_back(c);
+                c.f = b->kderiv ? K.own->x : K.own->xc;
+                c.blocks = (c.rows + c.f.rows - 1) / c.f.rows;
+                c.in0 = K.hco0;
+                c.in_stride = plane * (b->kderiv ? (int64_t)K.kx + 1 : 2 * (int64_t)K.kx + 2);
+                c.out0 = b->kderiv ? K.go0 : K.ro0;
+                c.out_stride = cells;
+                inv.push_back(c);
+                c.f = K.own->y;
+                c.blocks = K.kx + 1;
+                c.list0 = K.list0;
+                col.push_back(c);
+            }
+            b->fft_fwd = fresco::fft_class_sets(std::move(fwd), 0);
+            b->fft_col = fresco::fft_class_sets(std::move(col), b->kderiv ? 1 : 2);
+            b->fft_inv = fresco::fft_class_sets(std::move(inv), 0);
             if (!balloc(b, (void **)&b->cls_list, sizeof(int) * list.size()) ||
                 !balloc(b, (void **)&b->rep_first, sizeof(int) * first.size()) ||
                 !balloc(b, (void **)&b->rep_off, sizeof(int64_t) * off.size()))
@@ -1923,23 +1957,24 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
     }
     {
         StageScope sc(b->prof, s, ST_FFT_FWD);
+        if (b->own_fft) {
+            for (const auto &q : b->fft_fwd)
+                FR_CUDA(fresco::fft_rows_forward_b(q, (const float *)b->grid, (float2 *)b->specT,
+                                                   (const float2 *)b->tw, s));
+            // the y pass, the mask and the y pass back, column by column
+            const fresco::ColsBatch a{b->d_inst, b->cls_list, b->rep_first, b->rep_off,
+                                      (const float2 *)b->specT, (float2 *)b->bt, b->rep_n,
+                                      (const float *)b->rep_s0, (const float *)b->rep_w,
+                                      (const float *)b->ip, b->partial, b->d_mblk_first};
+            for (const auto &q : b->fft_col)
+                FR_CUDA(fresco::fft_cols_mask_b(q, a, b->kderiv != 0, s));
+            b->launches += (int64_t)(b->fft_fwd.size() + b->fft_col.size());
+        }
         for (auto &K : b->cls) {   // forward FFT of each size class
+            if (b->own_fft) break;
             const int64_t plane = K.nf[1];
             const int mh = K.nf[0] / 2;
             C2 *A = (C2 *)((T *)b->grid + K.go0), *AT = (C2 *)b->specT + K.ato0;
-            if (b->own_fft) {
-                FR_CUDA(fresco::fft_rows_forward(K.own->x, (const float *)A, (float2 *)AT,
-                                                 (const float2 *)b->tw + K.two0, plane, K.kx, s,
-                                                 K.count, 2 * plane * mh, plane * (K.kx + 1)));
-                // the y pass, the mask and the y pass back, column by column
-                fresco::ColsBatch a{b->d_inst, b->cls_list + K.list0, b->rep_first, b->rep_off,
-                                    (const float2 *)b->specT, (float2 *)b->bt, b->rep_n,
-                                    (const float *)b->rep_s0, (const float *)b->rep_w,
-                                    (const float *)b->ip, b->partial, b->d_mblk_first, K.kx};
-                FR_CUDA(fresco::fft_cols_mask_b(K.own->y, a, K.count, b->kderiv != 0, s));
-                b->launches += 2;
-                continue;
-            }
             if (sizeof(T) == 4)
                 FR_CUFFT(cufftExecC2C(K.h[0], (cufftComplex *)A, (cufftComplex *)A,
                                       CUFFT_FORWARD));
@@ -1972,18 +2007,18 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
     if (b->kderiv) {
         {
             StageScope sc(b->prof, s, ST_FFT_INV);
+            if (b->own_fft) {
+                for (const auto &q : b->fft_inv)
+                    FR_CUDA(fresco::fft_rows_inverse_b(q, (const float2 *)b->bt, (float *)b->grid,
+                                                       (const float2 *)b->tw, s));
+                b->launches += (int64_t)b->fft_inv.size();
+            }
             for (auto &K : b->cls) {   // scalar spectrum -> real field (in the spread grid's place)
+                if (b->own_fft) break;
                 const int64_t plane = K.nf[1];
                 const int mh = K.nf[0] / 2;
                 C2 *H = (C2 *)b->hc + K.hco0, *BT = (C2 *)b->bt + K.hco0;
                 C2 *Z = (C2 *)((T *)b->grid + K.go0);
-                if (b->own_fft) {
-                    FR_CUDA(fresco::fft_rows_inverse(
-                        K.own->x, (const float2 *)BT, (float *)Z, (const float2 *)b->tw + K.two0,
-                        plane, K.kx, s, K.count, plane * ((int64_t)K.kx + 1), 2 * plane * mh));
-                    b->launches += 1;
-                    continue;
-                }
                 if (sizeof(T) == 4)
                     FR_CUFFT(cufftExecC2C(K.h[2], (cufftComplex *)H, (cufftComplex *)BT,
                                           CUFFT_INVERSE));
@@ -2009,17 +2044,16 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
     }
     {
         StageScope sc(b->prof, s, ST_FFT_INV);
+        if (b->own_fft) {
+            for (const auto &q : b->fft_inv)
+                FR_CUDA(fresco::fft_rows_inverse_cb(q, (const float2 *)b->bt, (float2 *)b->g, s));
+            b->launches += (int64_t)b->fft_inv.size();
+        }
         for (auto &K : b->cls) {   // inverse FFT of each size class
+            if (b->own_fft) break;
             const int64_t plane = K.nf[1];
             C2 *H = (C2 *)b->hc + K.hco0, *BT = (C2 *)b->bt + K.hco0, *R = (C2 *)b->r + K.ro0;
             C2 *G = (C2 *)b->g + K.ro0;
-            if (b->own_fft) {
-                FR_CUDA(fresco::fft_rows_inverse_c(
-                    K.own->xc, (const float2 *)BT, (float2 *)G, plane, K.kx, s, K.count,
-                    plane * (2 * (int64_t)K.kx + 2), (int64_t)K.nf[0] * plane));
-                b->launches += 1;
-                continue;
-            }
             if (sizeof(T) == 4)
                 FR_CUFFT(cufftExecC2C(K.h[2], (cufftComplex *)H, (cufftComplex *)BT,
                                       CUFFT_INVERSE));
@@ -2382,7 +2416,7 @@ fresco_status uwu_build(fresco_uwu_s *u, const Folded &F) {
     if (sizeof(T) == 4 && dim == 2) {
         u->own = new (std::nothrow) fresco::FftSet();
         if (!u->own) return FRESCO_ERR_OOM;
-        const fresco_status st = fresco::fft_set_build(*u->own, u->M, 2, true, 1, true);
+        const fresco_status st = fresco::fft_set_build(*u->own, u->M, 2, true, u->M[1], true);
         if (st) return st;
         if (!u->own->cols) {
             fresco::fft_set_free(u->own);

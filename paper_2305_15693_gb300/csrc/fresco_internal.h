@@ -343,6 +343,7 @@ void es_poly_table(int w, double beta, EsPoly<double> &out);
 // to the library; direct_build leaves *out null where the problem is large enough for the NUFFT.
 struct DirectPlan;
 struct FftSet;   // fresco_fft.h
+struct FftClassSet;
 bool direct_wanted(int64_t n_points, const fresco_opts &o, int precision, double tol);
 fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const double *box,
                            int precision, const int32_t *mask, int64_t n_k,
@@ -518,6 +519,7 @@ struct fresco_batch_s {
     int kderiv = 0;                  // gradient mode FRESCO_GRAD_KDERIV
     int64_t n_r = 0;                 // complex elements of the row-order backward buffer
     bool own_fft = false;            // every class runs the library's own transforms
+    std::vector<fresco::FftClassSet> fft_fwd, fft_col, fft_inv;   // their launches
     int *cls_list = nullptr;         // instances, class by class
     int *rep_first = nullptr;        // per instance, first representative of every column
     int64_t *rep_off = nullptr;      // per instance, its part of rep_first
