@@ -785,7 +785,7 @@ fresco_status build_plan(fresco_plan_s *p, const Params &P, const Folded &F) {
     fresco_status st;
     if ((st = dalloc(p, &p->d_sorted, sizeof(T) * (size_t)slots * pw))) return st;
     if (sizeof(T) == 8 && (st = dalloc(p, &p->d_perm, sizeof(int) * (size_t)slots))) return st;
-    if ((st = dalloc(p, &p->d_tcur, sizeof(int) * (size_t)(g.n_tiles + 1)))) return st;
+    if (g.tcap && (st = dalloc(p, &p->d_tcur, fresco::cursor_bytes(g)))) return st;
     if ((st = dalloc(p, &p->d_tr, sizeof(int2) * (size_t)g.n_tiles))) return st;
     p->ring_slot = Launch<T>::ring_slot(g);
     if ((st = dalloc(p, &p->d_ring, sizeof(T) * (size_t)(g.n_tiles * p->ring_slot)))) return st;
@@ -956,7 +956,7 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
         // the direct form (one pass); then the tiles' record ranges, after an overflow (or in a plan
         // without the direct form) with the compact form
         if (g.tcap)
-            FR_CUDA(cudaMemsetAsync(p->d_tcur, 0, sizeof(int) * (size_t)(g.n_tiles + 1), s));
+            FR_CUDA(cudaMemsetAsync(p->d_tcur, 0, fresco::cursor_bytes(g), s));
         if (h_pts) {
             fresco_status st = stage_and_bin<T>(p, h_pts, const_cast<T *>(pts));
             if (st) return st;
@@ -1223,8 +1223,7 @@ fresco_status fresco::point_side_build(PointSide &ps, int dim, const int nf[3], 
     if (ps.bin_blocks < 1) return FRESCO_ERR_CUDA;
     bool ok = ps_alloc(ps, &ps.sorted, es * (size_t)slots * pw) &&
               (es == 4 || ps_alloc(ps, (void **)&ps.perm, sizeof(int) * (size_t)slots)) &&
-              (!g.tcap ||
-               ps_alloc(ps, (void **)&ps.tcur, sizeof(int) * (size_t)(g.n_tiles + 1))) &&
+              (!g.tcap || ps_alloc(ps, (void **)&ps.tcur, fresco::cursor_bytes(g))) &&
               ps_alloc(ps, (void **)&ps.cnt, sizeof(int) * (size_t)g.n_bins) &&
               ps_alloc(ps, (void **)&ps.off, sizeof(int) * (size_t)(g.n_bins + 1)) &&
               ps_alloc(ps, (void **)&ps.tr, sizeof(int2) * (size_t)g.n_tiles) &&
@@ -1246,7 +1245,7 @@ fresco_status fresco::point_side_spread(PointSide &ps, const T *pts, cudaStream_
     const Geom &g = ps.g;
     int nl = 1;
     if (g.tcap) {
-        FR_CUDA(cudaMemsetAsync(ps.tcur, 0, sizeof(int) * (size_t)(g.n_tiles + 1), s));
+        FR_CUDA(cudaMemsetAsync(ps.tcur, 0, fresco::cursor_bytes(g), s));
         FR_CUDA(Launch<T>::place_direct(g, pts, 0, ps.tcur, ps.sorted, ps.perm, ps.err, s));
         nl += 1;
     }
@@ -1748,7 +1747,7 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
               (sizeof(T) == 4 || balloc(b, (void **)&b->perm, sizeof(int) * N)) &&
               balloc(b, (void **)&b->key, sizeof(int) * N) &&
               balloc(b, (void **)&b->slot, sizeof(int) * N) &&
-              balloc(b, (void **)&b->cnt, sizeof(int) * b->n_bins) &&
+              balloc(b, (void **)&b->cnt, sizeof(int) * b->n_bins * fresco::kBinStride) &&
               balloc(b, (void **)&b->off, sizeof(int) * (b->n_bins + 1)) &&
               balloc(b, (void **)&b->bsum, sizeof(int) * ((b->n_bins + 1023) / 1024 + 1)) &&
               balloc(b, (void **)&b->err, sizeof(int)) &&
@@ -1943,10 +1942,11 @@ fresco_status batch_eval(fresco_batch_s *b, const T *pts, double *losses, T *gra
     const BTables &t = b->tab;
     {
         StageScope sc(b->prof, s, ST_SORT);
-        FR_CUDA(cudaMemsetAsync(b->cnt, 0, sizeof(int) * (size_t)b->n_bins, s));
+        FR_CUDA(cudaMemsetAsync(b->cnt, 0, sizeof(int) * (size_t)b->n_bins * fresco::kBinStride, s));
         FR_CUDA(Launch<T>::bin_b(t, pts, b->cnt, b->key, b->slot, b->err, s));
         int nl = 0;
-        FR_CUDA(Launch<T>::scan(b->cnt, b->off, b->bsum, b->n_bins, s, &nl));
+        FR_CUDA(Launch<T>::scan(b->cnt, b->off, b->bsum, b->n_bins, s, &nl,
+                                fresco::kBinStride));
         FR_CUDA(Launch<T>::scatter_b(t, pts, b->key, b->slot, b->off, b->sorted, b->perm, s));
         b->launches += 2 + nl;
     }

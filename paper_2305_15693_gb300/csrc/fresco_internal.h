@@ -19,7 +19,13 @@ constexpr int kMaxTileEdge = 255; // tile-relative cell must fit the 8-bit field
 constexpr int kTileCursors = 4;   // placement cursors per tile of a single plan (Geom.sub)
 constexpr int kZSegmentMax = 16;  // 3D single plans: most tiles per z-column segment (Geom.zseg)
 constexpr int kColMaxPlanes = 64; // column spread: tiles with tmax_z + w above this spread one by one
-constexpr int kDirectPointsPerThread = 8;   // points in flight per thread of k_place_direct
+// ints from one tile's cursor to the next: an L2 line each. Atomics on one line run one at a time,
+// and packed cursors of a small grid are few lines: k_place_direct, 4e5 points on 144 tiles 80 us
+// packed, 34 at a sector (8) each, 15 at a line; 10^6 on 729 tiles 108 / 38 / 34
+constexpr int kCursorStride = 32;
+// ints from one bin's count to the next in an ensemble's binning (many more bins): a sector each.
+// 2.75e6 points: 77 us packed, 50 at a sector, 52 at a line
+constexpr int kBinStride = 8;
 constexpr int kBinFinishBlocks = 1024;      // most blocks of k_bin_finish
 // fresco_loss_grad_host copies the points in up to kHostChunks pieces of at least
 // kHostChunkBytes, binning each piece while the next one is in flight
@@ -85,6 +91,11 @@ struct Geom {
     FastDiv fdp[2][2];  // division by (x tile width + width) (y tile width + width), the x and
                         // y widths tq or tq + 1
 };
+
+// the direct form's cursors and, after them, the overflow word
+inline size_t cursor_bytes(const Geom &g) {
+    return sizeof(int) * (size_t)(g.n_tiles + 1) * kCursorStride;
+}
 
 // Fills g.fdw and g.fdp from g.tq and g.width (host).
 inline void set_tile_divisors(Geom &g) {
@@ -221,11 +232,11 @@ struct StageScope {
 // return the cudaError_t of the launch. Element layouts are documented in fresco_kernels.cuh.
 template <typename T>
 struct Launch {
-    // exclusive prefix sum of cnt into off[0..n] (off[n] = total)
+    // exclusive prefix sum of cnt (stride ints apart) into off[0..n] (off[n] = total)
     static cudaError_t scan(const int *cnt, int *off, int *block_sums, int64_t n, cudaStream_t s,
-                            int *launches);
+                            int *launches, int stride = 1);
     // direct form: g.n_points points starting at caller index j0 (points points at that point)
-    // into tile slots of capacity g.tcap; tcur [n_tiles + 1] zero before the first chunk, its
+    // into tile slots of capacity g.tcap; tcur (cursor_bytes) zero before the first chunk, its
     // last entry the overflow word
     static cudaError_t place_direct(const Geom &g, const T *points, int64_t j0, int *tcur,
                                     void *sorted, int *perm, int *err, cudaStream_t s);
@@ -422,7 +433,7 @@ struct fresco_plan_s {
     int64_t ring_slot = 0;
     int *d_cnt = nullptr;            // [n_bins] points per bin, then the placement cursors
     int *d_off = nullptr;            // [n_bins + 1] exclusive prefix sum of the counts
-    int *d_tcur = nullptr;           // [n_tiles + 1] direct-form cursors, then the overflow word
+    int *d_tcur = nullptr;           // direct-form cursors, then the overflow word (cursor_bytes)
     int2 *d_tr = nullptr;            // [n_tiles] record range of every tile
     CUtensorMap tmap{};              // geom.tma: the interpolated real field as a TMA tensor
     int *d_block_sums = nullptr;     // [kBinFinishBlocks] scan scratch

@@ -233,10 +233,11 @@ __device__ __forceinline__ int strip_part(int rel, int wd, int w, int strips) {
 // blocks of 1024.
 static __global__ void __launch_bounds__(1024) k_scan_blocks(const int *__restrict__ cnt,
                                                       int *__restrict__ off,
-                                                      int *__restrict__ bsum, int64_t n) {
+                                                      int *__restrict__ bsum, int64_t n,
+                                                      int stride) {
     __shared__ int warp_tot[32];
     int64_t i = (int64_t)blockIdx.x * 1024 + threadIdx.x;
-    int v = (i < n) ? cnt[i] : 0;
+    int v = (i < n) ? cnt[i * stride] : 0;
     int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int x = v;
 #pragma unroll
@@ -348,7 +349,7 @@ __global__ void __launch_bounds__(256) k_bin_b(const BInst *__restrict__ inst,
         const BInst &I = inst[i];
         const int bin = (int)I.bo + bin_point<T, D>(I.g, pts + j * D, ok);
         key[j] = bin;
-        slot[j] = atomicAdd(&cnt[bin], 1);
+        slot[j] = atomicAdd(&cnt[(int64_t)bin * kBinStride], 1);
     }
     if (!ok) atomicOr(err, 1);
 }
@@ -1820,9 +1821,9 @@ inline int grid_for(int64_t n, int threads, int cap) {
 
 template <typename T>
 cudaError_t Launch<T>::scan(const int *cnt, int *off, int *block_sums, int64_t n, cudaStream_t s,
-                            int *launches) {
+                            int *launches, int stride) {
     const int64_t nb = (n + 1023) / 1024;
-    k_scan_blocks<<<(unsigned)nb, 1024, 0, s>>>(cnt, off, block_sums, n);
+    k_scan_blocks<<<(unsigned)nb, 1024, 0, s>>>(cnt, off, block_sums, n, stride);
     k_scan_sums<<<1, 1024, 0, s>>>(block_sums, nb, off + n);
     k_scan_add<<<(unsigned)nb, 1024, 0, s>>>(off, block_sums, n);
     *launches += 3;
@@ -1860,11 +1861,10 @@ template <typename T>
 cudaError_t Launch<T>::place_direct(const Geom &g, const T *points, int64_t j0, int *tcur,
                                     void *sorted, int *perm, int *err, cudaStream_t s) {
     using U = typename PT<T>::U;
-    constexpr int IL = kDirectPointsPerThread;
-    const bool many = g.n_points >= (int64_t)152 * 2 * 256 * IL;
-    const int grid = grid_for(many ? (g.n_points + IL - 1) / IL : g.n_points, 256, 152 * 16);
-    const auto kern = g.dim == 2 ? (many ? k_place_direct<T, 2, IL> : k_place_direct<T, 2, 1>)
-                                 : (many ? k_place_direct<T, 3, IL> : k_place_direct<T, 3, 1>);
+    const int il = g.dim == 3 && sizeof(T) == 4 ? 2 : 1;
+    const int grid = grid_for((g.n_points + il - 1) / il, 256, 152 * 16);
+    const auto kern = g.dim == 2 ? k_place_direct<T, 2, 1>
+                                 : k_place_direct<T, 3, sizeof(T) == 4 ? 2 : 1>;
     kern<<<grid, 256, 0, s>>>(g, points, j0, tcur, (U *)sorted, perm, err);
     return cudaGetLastError();
 }

@@ -3,9 +3,9 @@
 // Binning (K1). A plan whose tiles can hold their expected points plus a wide margin in a fixed
 // capacity Geom.tcap per tile places every point in one pass over the caller's points:
 //   k_place_direct  computes each point's tile and record and takes its slot from the tile's
-//                   cursor, pos = atomicAdd(&tcur[t], 1), at record t * tcap + pos;
-// the tile's points are then records [t tcap, t tcap + tcur[t]). A point whose tile is full sets
-// the overflow word tcur[n_tiles]; the compact form then runs inside the next kernel, so any input
+//                   cursor, pos = atomicAdd(cursor(tcur, t), 1), at record t * tcap + pos;
+// the tile's points are then records [t tcap, t tcap + cursor). A point whose tile is full sets
+// the overflow word (entry n_tiles); the compact form then runs inside the next kernel, so any input
 // is binned correctly and uniform inputs pay for one pass only:
 //   k_bin_finish    writes the record range of every tile, tr[t] = (first, end); after an overflow
 //                   it first counts the points of every bin, scans the counts into off[] and the
@@ -217,10 +217,10 @@ __global__ void __launch_bounds__(256) k_bin_finish(Geom g, const T *__restrict_
                                                     int2 *__restrict__ tr, int *__restrict__ err) {
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nt = (int64_t)gridDim.x * blockDim.x;
-    if (tcur && !tcur[g.n_tiles]) {
+    if (tcur && !tcur[g.n_tiles * kCursorStride]) {
         for (int64_t t = tid; t < g.n_tiles; t += nt) {
             const int b = (int)(t * g.tcap);
-            tr[t] = make_int2(b, b + tcur[t]);
+            tr[t] = make_int2(b, b + tcur[t * kCursorStride]);
         }
         return;
     }
@@ -273,11 +273,14 @@ __global__ void __launch_bounds__(256) k_bin_finish(Geom g, const T *__restrict_
     place_points<T, D>(g, pts, cnt, sorted, perm);
 }
 
+// tile t's cursor (t = n_tiles: the overflow word)
+__device__ __forceinline__ int *cursor(int *tcur, int64_t t) { return tcur + t * kCursorStride; }
+
 // One pass of the direct form: points j0 .. j0 + g.n_points - 1 of the caller's array (pts points
-// at point j0), each to its tile's next slot. tcur[n_tiles] is the overflow word.
-// IL: points in flight per thread; the returning cursor atomics are what it waits for, so a large
-// array takes eight, and a small one one, for more blocks (20011 FP64 points in 3D: ten blocks, 47
-// us, now 9; 100003 in 2D 16.6, now 15.1; no difference from 4e5 on).
+// at point j0), each to its tile's next slot.
+// IL: points in flight per thread. Warps hide the returning atomics better than points per thread do
+// (one point 22 us at 10^6 and 153 at 10^7 in 2D, four 24 and 184, eight 34 and 229; in 3D FP32 two
+// are best: 2 10^6 points 52 / 50 / 54 / 70 for one, two, four, eight).
 template <typename T, int D, int IL>
 __global__ void __launch_bounds__(256) k_place_direct(Geom g, const T *__restrict__ pts,
                                                       int64_t j0, int *__restrict__ tcur,
@@ -317,11 +320,11 @@ __global__ void __launch_bounds__(256) k_place_direct(Geom g, const T *__restric
                 const unsigned grp = __match_any_sync(0xffffffffu, tile[k]);
                 const int lane = threadIdx.x & 31, leader = __ffs(grp) - 1;
                 int base = 0;
-                if (in && lane == leader) base = atomicAdd(&tcur[t], __popc(grp));
+                if (in && lane == leader) base = atomicAdd(cursor(tcur, t), __popc(grp));
                 base = __shfl_sync(grp, base, leader);
                 pos[k] = base + __popc(grp & ((1u << lane) - 1u));
             } else {
-                pos[k] = in ? atomicAdd(&tcur[t], 1) : 0;
+                pos[k] = in ? atomicAdd(cursor(tcur, t), 1) : 0;
             }
         }
 #pragma unroll
@@ -336,7 +339,7 @@ __global__ void __launch_bounds__(256) k_place_direct(Geom g, const T *__restric
         }
     }
     if (!ok) atomicOr(err, 1);
-    if (over) atomicOr(&tcur[g.n_tiles], 1);
+    if (over) atomicOr(cursor(tcur, g.n_tiles), 1);
 }
 
 // Shared-memory accesses of the window loops, written as PTX on 32-bit shared-space addresses
