@@ -184,6 +184,9 @@ fresco_status fresco_status_check(fresco_plan_t p);
  * each stage of every later call; fresco_profile_read returns accumulated milliseconds and
  * call counts per stage (synchronises first) and resets them. Stages, in order:
  * 0 sort, 1 spread, 2 forward FFT, 3 mask/loss, 4 loss finalize, 5 inverse FFT, 6 interpolate.
+ * Steps that share a kernel count under the first one's stage: a plan with its own 2D transforms
+ * has the column kernel (mask, loss and the y pass back too) under 2; a small plan's direct sums
+ * are under 1, 3 and 6. The loss is summed by the mask's last block, so 4 stays zero there.
  * ms and counts have room for FRESCO_N_STAGES entries each (counts may be NULL). */
 #define FRESCO_N_STAGES 7
 fresco_status fresco_profile(fresco_plan_t p, int enable);
@@ -322,8 +325,9 @@ fresco_status fresco_lbfgs_destroy(fresco_lbfgs_t s);
  * A batch plan holds n_inst independent 2D problems (points, box, mask, S0, W each their own,
  * the same precision and tolerance). Their points are packed one instance after the other in a
  * single device array; every stage (sort, spread, mask, interpolation) runs as one launch over
- * all instances, and the uniform FFTs run per size class (fine grids rounded up to 2^k or 3 2^k),
- * one batched cuFFT call per class and direction. The result for instance i is exactly what
+ * all instances. The uniform FFTs run per size class (fine grids rounded up to 2^k or 3 2^k): FP32
+ * in the library's own kernels, up to sixteen classes in a launch; FP64 as one batched cuFFT call
+ * per class and direction. The result for instance i is exactly what
  * fresco_plan / fresco_loss_grad give for that problem alone (up to the larger fine grid). */
 typedef struct fresco_batch_s *fresco_batch_t;
 
