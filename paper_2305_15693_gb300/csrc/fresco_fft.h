@@ -123,7 +123,7 @@ cudaError_t fft_cols_weights(const FftDesc &f, const ColsArgs &a, double loss_co
 cudaError_t fft_rows_inverse_w(const FftDesc &f, const float2 *bt, float *grad, const float2 *tws,
                                int64_t rows, int kx, const float *c, const double *scal,
                                cudaStream_t s);
-// the column spectra themselves: out[k][row] = forward transform of xt[k] along y, in place allowed
+// the column spectra themselves: out[k][row] = forward transform of xt[k] along y
 cudaError_t fft_cols_spectrum(const FftDesc &f, const float2 *xt, float2 *out, int kx,
                               cudaStream_t s);
 // whether a column (with its scratch) fits a block

@@ -505,7 +505,7 @@ void release(fresco_plan_s *p) {
     if (p->stream) cudaStreamSynchronize(p->stream);
     else cudaDeviceSynchronize();
     void *bufs[] = {p->d_sorted, p->d_perm, p->d_ring, p->d_cnt, p->d_off, p->d_tcur, p->d_tr,
-                    p->d_block_sums, p->d_grid, p->d_tw, p->d_specT, p->d_bt[0], p->d_bt[1],
+                    p->d_block_sums, p->d_grid, p->d_tw, p->d_specT, p->d_spec, p->d_bt[0], p->d_bt[1],
                     p->d_hc[0], p->d_hc[1], p->d_r[0],
                     p->d_r[1], p->d_g[0], p->d_g[1], p->d_rep_n, p->d_rep_s0, p->d_rep_w,
                     p->d_ip[0], p->d_ip[1], p->d_ip[2], p->d_partial, p->d_done, p->d_err,
@@ -1003,7 +1003,6 @@ fresco_status forward_impl(fresco_plan_s *p, const T *pts, double *loss,
                                (const float *)p->d_ip[1], p->d_partial};
             FR_CUDA(fresco::fft_cols_mask(own->y, a, p->info.loss_const, loss, p->d_done, s));
             p->launches += 1;
-            p->spec_ready = false;
             p->forward_done = true;
             return FRESCO_OK;
         }
@@ -1454,11 +1453,19 @@ fresco_status fresco_get_rho_S(fresco_plan_t p, void *d_rho, void *d_S) {
                 ? fresco::direct_rho_s<double>(p->direct, (double *)d_rho, (double *)d_S, p->stream)
                 : fresco::direct_rho_s<float>(p->direct, (float *)d_rho, (float *)d_S, p->stream));
     }
-    if (p->own_fft && p->own_fft->cols && !p->spec_ready) {
-        // the column kernel keeps its spectra on chip: transform the columns here, once per forward
+    const void *spec = p->d_specT;
+    if (p->own_fft && p->own_fft->cols) {
+        // the column kernel keeps its spectra on chip: transform the columns here, into a buffer of
+        // their own on every call. (In place, once per forward, would need the host to know when the
+        // columns are new, and a replayed graph rewrites them without a call to forward_impl.)
+        if (!p->d_spec) {
+            const fresco_status st = dalloc(
+                p, &p->d_spec, sizeof(float2) * (size_t)(p->mgeom.plane * (p->mgeom.kx + 1)));
+            if (st) return st;
+        }
         FR_CUDA(fresco::fft_cols_spectrum(p->own_fft->y, (const float2 *)p->d_specT,
-                                          (float2 *)p->d_specT, p->mgeom.kx, p->stream));
-        p->spec_ready = true;
+                                          (float2 *)p->d_spec, p->mgeom.kx, p->stream));
+        spec = p->d_spec;
         p->launches += 1;
     }
     if (!p->d_mask_orig) {
@@ -1469,12 +1476,12 @@ fresco_status fresco_get_rho_S(fresco_plan_t p, void *d_rho, void *d_S) {
     }
     cudaError_t e;
     if (p->precision == FRESCO_F64)
-        e = Launch<double>::rho_s(p->mgeom, p->d_mask_orig, p->n_k, p->d_specT,
+        e = Launch<double>::rho_s(p->mgeom, p->d_mask_orig, p->n_k, spec,
                                   (const double *)p->d_ip[0], (const double *)p->d_ip[1],
                                   (const double *)p->d_ip[2], (double *)d_rho, (double *)d_S,
                                   p->stream);
     else
-        e = Launch<float>::rho_s(p->mgeom, p->d_mask_orig, p->n_k, p->d_specT,
+        e = Launch<float>::rho_s(p->mgeom, p->d_mask_orig, p->n_k, spec,
                                  (const float *)p->d_ip[0], (const float *)p->d_ip[1],
                                  (const float *)p->d_ip[2], (float *)d_rho, (float *)d_S,
                                  p->stream);

@@ -441,6 +441,7 @@ struct fresco_plan_s {
     void *d_grid = nullptr;          // real fine grid (spread output)
     void *d_tw = nullptr;            // exp(-2 pi i k / nf0), k = 0..nf0/4 (real-row split/merge)
     void *d_specT = nullptr;         // its columns x = 0..kx transposed: [kx+1][plane]
+    void *d_spec = nullptr;          // those transformed along y (own 2D columns, fresco_get_rho_S)
     void *d_hc[2] = {nullptr, nullptr};   // transposed compact backward spectra [2kx+2][plane]
     void *d_bt[2] = {nullptr, nullptr};   // after the (z,)y pass, still transposed
     void *d_r[2] = {nullptr, nullptr};    // transposed back to [plane][nf0]; other columns zero
@@ -474,7 +475,6 @@ struct fresco_plan_s {
     bool have_fft[4] = {false, false, false, false};
 
     fresco::FftSet *own_fft = nullptr;      // FP32 plans: the library's own transforms
-    bool spec_ready = false;                // d_specT holds the transformed columns (own_fft->cols)
     fresco::DirectPlan *direct = nullptr;   // small problems: direct sums, none of the above
     fresco::StageProfile prof;
     int64_t launches = 0;
