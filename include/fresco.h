@@ -267,7 +267,7 @@ fresco_status fresco_pair_destroy(fresco_pair_t p);
  * iteration: d = -H g by the two-loop recursion (H0 = (s.y)/(y.y) I; steepest descent when the
  * history is empty or d is not a descent direction); step t0 = min(1, max_step / max_j |d_j|);
  * backtracking t = t0, t0/2, ... until L(x + t d) <= L(x) + c1 t g.d; the pair (s, y) is kept when
- * s.y > 0. The host reads one or two scalars per line-search trial. */
+ * s.y > 0. The host reads a few scalars per line-search trial, in one copy. */
 typedef struct fresco_lbfgs_s *fresco_lbfgs_t;
 
 typedef struct {
@@ -301,7 +301,7 @@ typedef struct {
 
 void fresco_lbfgs_opts_default(fresco_lbfgs_opts *opts);
 
-/* Create a solver for a plan (the plan must outlive it). Allocates (2m + 4) vectors of N * dim
+/* Create a solver for a plan (the plan must outlive it). Allocates (2m + 6) vectors of N * dim
  * elements of the plan's precision. Returns FRESCO_ERR_ARG or FRESCO_ERR_OOM. */
 fresco_status fresco_lbfgs_create(fresco_lbfgs_t *out, fresco_plan_t plan,
                                   const fresco_lbfgs_opts *opts);

@@ -35,6 +35,7 @@ constexpr int kRedThreads = 256;
 enum Slot {
     SL_GD = 0,      // g.d
     SL_DMAX,        // max |d_j|
+    SL_GMAX,        // max |d_j| of d = -g, where g.d is not below 0
     SL_LOSS,        // loss at the trial point
     SL_SY,          // s.y of the candidate pair
     SL_YY,          // y.y of the candidate pair
@@ -168,7 +169,9 @@ struct History {
 };
 
 // Two-loop recursion, d = -H g, with g.d, max |d|, and the first trial point xt = x + t d,
-// t = min(1, max_step / max |d|), for vectors that fit the registers of one cluster: kTlBlocks
+// t = min(1, max_step / max |d|); where d is not a descent direction (g.d >= 0, or not a number after
+// a pair whose s.y is next to nothing), d = -g instead: a trial runs before the host has seen g.d, and
+// must not run on points along a direction that is dropped. For vectors that fit the registers of one cluster: kTlBlocks
 // blocks of kTlThreads threads with up to E elements each. Every dot product is a sum per warp and
 // one exchange of these over the cluster's shared memory. A launch per vector operation costs more than these
 // operations up to about 3e4 elements (20 points of history: 60 launches, 190 us, against one of
@@ -277,16 +280,19 @@ __global__ void __cluster_dims__(kTlBlocks, 1, 1) __launch_bounds__(kTlThreads)
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         v[e] = T(-1) * v[e];
-        if (i0 + e * ST < n) {
-            acc.add(g[i0 + e * ST], v[e]);
-            mx = fmax(mx, fabs(v[e]));
-        }
+        if (i0 + e * ST < n) acc.add(g[i0 + e * ST], v[e]);
     }
     const double gd = total(acc.value(), false);
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (i0 + e * ST < n) {
+            if (!(gd < 0.0)) v[e] = T(-1) * g[i0 + e * ST];
+            mx = fmax(mx, fabs(v[e]));
+        }
     const double dmax = total((double)mx, true);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc[SL_GD] = gd;
-        sc[SL_DMAX] = dmax;
+        sc[SL_DMAX] = sc[SL_GMAX] = dmax;
     }
     const T t = (T)fmin(1.0, max_step / dmax);
 #pragma unroll
@@ -300,7 +306,7 @@ __global__ void __cluster_dims__(kTlBlocks, 1, 1) __launch_bounds__(kTlThreads)
 
 // One step of the recursion over a vector of any length: v = in (+ c a), c = sign (*c0 - *c1),
 // times *scale, negated if neg; then, in the same pass, v.b times *mul into *out and, if out_max,
-// max |v|. Null pointers leave their part out.
+// max |v| and max |b| into its two entries. Null pointers leave their part out.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_two_loop_step(
     T *__restrict__ v, const T *in, const T *__restrict__ a, const double *__restrict__ c0,
@@ -310,7 +316,7 @@ __global__ void __launch_bounds__(kRedThreads) k_two_loop_step(
     const T c = a ? (T)(sign * (*c0 - (c1 ? *c1 : 0.0))) : T(0);
     const T st = scale ? (T)*scale : T(1);
     fresco::DotAcc<T> acc;
-    T mx = T(0);
+    T mx = T(0), bx = T(0);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         T u = in[i];
@@ -320,33 +326,35 @@ __global__ void __launch_bounds__(kRedThreads) k_two_loop_step(
         v[i] = u;
         if (b) acc.add(b[i], u);
         mx = fmax(mx, fabs(u));
+        if (out_max) bx = fmax(bx, fabs(b[i]));
     }
     double r[1] = {acc.value()};
     if (b && grid_reduce<1>(r, false, part, done)) *out = r[0] * (mul ? *mul : 1.0);
     if (!out_max) return;
     // (a second pass over the blocks' counters: the sum's is zero again only once its last block
-    // is done, so the maximum has its own)
-    double q[1] = {(double)mx};
-    if (grid_reduce<1>(q, true, part + gridDim.x, done + 1)) *out_max = q[0];
+    // is done, so the maxima have their own)
+    double q[2] = {(double)mx, (double)bx};
+    if (grid_reduce<2>(q, true, part + gridDim.x, done + 1)) {
+        out_max[0] = q[0];
+        out_max[1] = q[1];
+    }
 }
 
-// y = s0 x
+// z = x + min(1, max_step / max |d|) d; d = -g first where it is not a descent direction (k_two_loop
+// has the reason). sc: the device scalars
 template <typename T>
-__global__ void k_scale_copy(T *y, const T *x, int64_t n, double s0) {
-    const T ct = (T)s0;
+__global__ void k_first_trial(T *__restrict__ z, const T *__restrict__ x, T *__restrict__ d,
+                              const T *__restrict__ g, int64_t n, double max_step,
+                              const double *__restrict__ sc) {
+    const bool steepest = !(sc[SL_GD] < 0.0);
+    const T tt = (T)fmin(1.0, max_step / (steepest ? sc[SL_GMAX] : sc[SL_DMAX]));
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = ct * x[i];
-}
-
-// z = x + min(1, max_step / *dmax) b
-template <typename T>
-__global__ void k_first_trial(T *__restrict__ z, const T *__restrict__ x, const T *__restrict__ b,
-                              int64_t n, double max_step, const double *__restrict__ dmax) {
-    const T tt = (T)fmin(1.0, max_step / *dmax);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        z[i] = fma(tt, b[i], x[i]);
+         i += (int64_t)gridDim.x * blockDim.x) {
+        T u;
+        if (steepest) d[i] = u = T(-1) * g[i];
+        else u = d[i];
+        z[i] = fma(tt, u, x[i]);
+    }
 }
 
 // z = a + t * b
@@ -401,14 +409,11 @@ struct Ops {
         k_absmax<T><<<grid(), kRedThreads, 0, s->stream>>>((const T *)a, s->n, s->part, s->done,
                                                            out);
     }
-    void scale_copy(void *y, const void *x, double s0) {
-        k_scale_copy<T><<<grid(), kRedThreads, 0, s->stream>>>((T *)y, (const T *)x, s->n, s0);
-    }
     int slots() const { return s->opts.history + 1; }
     double *gamma() const { return s->scal + SL_GAMMA; }
     double *rho() const { return gamma() + slots(); }
     double *alpha() const { return rho() + slots(); }
-    // d = -H g, g.d, max |d| and the first trial point xt
+    // d = -H g (or -g), g.d, max |d| and the first trial point xt
     void direction(const void *x) {
         History h;
         h.count = s->count;
@@ -460,8 +465,8 @@ struct Ops {
                          sc + SL_GD, sc + SL_DMAX);
             }
         }
-        k_first_trial<T><<<grid(), kRedThreads, 0, s->stream>>>(xt, xp, d, s->n, s->opts.max_step,
-                                                                sc + SL_DMAX);
+        k_first_trial<T><<<grid(), kRedThreads, 0, s->stream>>>(xt, xp, d, g, s->n,
+                                                                s->opts.max_step, sc);
     }
     // the trial point's candidate pair, in the free slot
     void candidate(const void *x) {
@@ -616,20 +621,21 @@ fresco_status run_impl(fresco_lbfgs_s *s, void *x_caller, int64_t max_iter,
         const double grms = std::sqrt(gg / (double)s->n);
         if (s->opts.gtol > 0.0 && grms < s->opts.gtol) { status = 1; break; }
         if (s->opts.ftol > 0.0 && fx < s->opts.ftol) { status = 2; break; }
+        if (!(gg > 0.0)) {   // (a gradient of zeros: no direction, and nothing to evaluate)
+            op.absmax(s->g, sc + SL_GMAX);
+            if (!(read_scalars(s)[SL_GMAX] > 0.0)) {
+                s->count = 0;
+                status = 1;
+                break;
+            }
+        }
         op.direction(x);   // two-loop recursion, and xt at the first step length
         if ((st = trial())) return st;
         double gd = hs[SL_GD], dmax = hs[SL_DMAX];
-        if (!(gd < 0.0)) {   // not a descent direction: restart from steepest descent
+        if (!(gd < 0.0)) {   // not a descent direction: the device has taken the steepest descent
             s->count = 0;
-            s->head = 0;
-            op.scale_copy(s->d, s->g, -1.0);
             gd = -gg;
-            op.absmax(s->d, sc + SL_DMAX);
-            dmax = read_scalars(s)[SL_DMAX];
-            if (dmax > 0.0) {
-                op.lincomb(s->xt, x, s->d, std::min(1.0, s->opts.max_step / dmax));
-                if ((st = trial())) return st;
-            }
+            dmax = hs[SL_GMAX];
         }
         if (!(dmax > 0.0)) { status = 1; break; }
         double t = std::min(1.0, s->opts.max_step / dmax);
