@@ -407,9 +407,9 @@ fresco_status fresco_uwu_plan(fresco_uwu_t *out, int dim, const int64_t *grid, c
                               int64_t n_k, const double *S0, const double *W, int precision,
                               void *stream);
 /* d_c: device [M_{d-1}]..[M_0] of the plan's precision (x fastest, not all zero); d_loss: device
- * double; d_grad: device, same layout as d_c, or NULL. Asynchronous on the plan's stream. The loss
- * is summed in a fixed order and the type-1 spread adds in fixed point (integers scaled per tile
- * by a power of two below the tile's largest possible cell sum), so repeated calls agree bitwise. */
+ * double; d_grad: device, same layout as d_c, or NULL. d_c must be aligned to two elements, as cuFFT's
+ * real transforms ask (FP32 plans: FRESCO_ERR_CUFFT otherwise); d_grad to one. Asynchronous on the
+ * plan's stream. All sums run in a fixed order, so repeated calls agree bitwise. */
 fresco_status fresco_uwu_loss_grad(fresco_uwu_t u, const void *d_c, double *d_loss, void *d_grad);
 fresco_status fresco_uwu_destroy(fresco_uwu_t u);
 

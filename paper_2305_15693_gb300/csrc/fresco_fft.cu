@@ -58,8 +58,9 @@ __device__ __forceinline__ void rows_fwd(const FftDesc &f, const float *__restri
 }
 
 // WEIGHTS: the result less (4 F / rho0) c, c the weights on the same grid and scal[0] = rho0, scal[3]
-// = F (the weight gradient's second term)
-template <bool WEIGHTS>
+// = F (the weight gradient's second term). PAIRS: grid lies on an 8-byte boundary (the plans' own grids
+// do; a caller's gradient need not).
+template <bool WEIGHTS, bool PAIRS>
 __device__ __forceinline__ void rows_inv(const FftDesc &f, const float2 *__restrict__ bt,
                                          float *__restrict__ grid, const float2 *__restrict__ tws,
                                          int64_t rows, int64_t r0, int kx,
@@ -70,7 +71,16 @@ __device__ __forceinline__ void rows_inv(const FftDesc &f, const float2 *__restr
     const int M = f.n, pitch = f.words;
     const int nr = (int)min((int64_t)f.rows, rows - r0);
     bt += r0;
-    float2 *out = reinterpret_cast<float2 *>(grid) + r0 * M;
+    float *out = grid + 2 * r0 * M;
+    auto store = [&](int row, int i, float2 v) {
+        float *p = out + 2 * ((int64_t)row * M + i);
+        if constexpr (PAIRS) {
+            *reinterpret_cast<float2 *>(p) = v;
+        } else {
+            p[0] = v.x;
+            p[1] = v.y;
+        }
+    };
     // Z[k] = P + i Q, Z[M - k] = conj P + i conj Q (as k_rfft_merge_rows), parts exchanged
     const int half = M / 2, shift = __popc(f.rows - 1);
     for (int t = threadIdx.x; t < (half + 1) << shift; t += blockDim.x) {
@@ -93,11 +103,10 @@ __device__ __forceinline__ void rows_inv(const FftDesc &f, const float2 *__restr
         const float2 *cr = reinterpret_cast<const float2 *>(c) + r0 * M;
         fft_adjoint(f, nr, s, pitch, [&](int row, int i, float2 v) {
             const float2 w = cr[(int64_t)row * M + i];
-            out[(int64_t)row * M + i] = {v.y - coef * w.x, v.x - coef * w.y};
+            store(row, i, {v.y - coef * w.x, v.x - coef * w.y});
         });
     } else {
-        fft_adjoint(f, nr, s, pitch,
-                    [&](int row, int i, float2 v) { out[(int64_t)row * M + i] = {v.y, v.x}; });
+        fft_adjoint(f, nr, s, pitch, [&](int row, int i, float2 v) { store(row, i, {v.y, v.x}); });
     }
 }
 
@@ -131,12 +140,12 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
     rows_fwd(f, grid, xt, tws, rows, (int64_t)blockIdx.x * f.rows, kx);
 }
 
-template <bool WEIGHTS>
+template <bool WEIGHTS, bool PAIRS>
 __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
     k_fft_rows_inv(const __grid_constant__ FftDesc f, const float2 *__restrict__ bt,
                    float *__restrict__ grid, const float2 *__restrict__ tws, int64_t rows, int kx,
                    const float *__restrict__ c, const double *__restrict__ scal) {
-    rows_inv<WEIGHTS>(f, bt, grid, tws, rows, (int64_t)blockIdx.x * f.rows, kx, c, scal);
+    rows_inv<WEIGHTS, PAIRS>(f, bt, grid, tws, rows, (int64_t)blockIdx.x * f.rows, kx, c, scal);
 }
 
 __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
@@ -171,9 +180,9 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
     int b;
     const FftClass &c = q.c[class_of(q, b)];
     const int z = b / c.blocks;
-    rows_inv<false>(c.f, bt + c.in0 + z * c.in_stride, grid + c.out0 + z * c.out_stride,
-                    tws + c.tw0, c.rows, (int64_t)(b - z * c.blocks) * c.f.rows, c.kx, nullptr,
-                    nullptr);
+    rows_inv<false, true>(c.f, bt + c.in0 + z * c.in_stride, grid + c.out0 + z * c.out_stride,
+                          tws + c.tw0, c.rows, (int64_t)(b - z * c.blocks) * c.f.rows, c.kx,
+                          nullptr, nullptr);
 }
 
 __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
@@ -589,8 +598,9 @@ cudaError_t fft_allow_smem() {
     const int b = (int)kFftSmem;
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(k_fft_rows_fwd, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv<false>, attr, b);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv<true>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv<false, true>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv<true, true>, attr, b);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv<true, false>, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols_w, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_rows_inv_c, attr, b);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_cols<true>, attr, b);
@@ -666,16 +676,19 @@ cudaError_t fft_rows_forward(const FftDesc &f, const float *grid, float2 *xt, co
 
 cudaError_t fft_rows_inverse(const FftDesc &f, const float2 *bt, float *grid, const float2 *tws,
                              int64_t rows, int kx, cudaStream_t s) {
-    k_fft_rows_inv<false><<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads,
-                            fft_bytes(f, f.rows), s>>>(f, bt, grid, tws, rows, kx, nullptr, nullptr);
+    k_fft_rows_inv<false, true><<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads,
+                                  fft_bytes(f, f.rows), s>>>(f, bt, grid, tws, rows, kx, nullptr,
+                                                             nullptr);
     return cudaGetLastError();
 }
 
 cudaError_t fft_rows_inverse_w(const FftDesc &f, const float2 *bt, float *grad, const float2 *tws,
                                int64_t rows, int kx, const float *c, const double *scal,
                                cudaStream_t s) {
-    k_fft_rows_inv<true><<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads,
-                           fft_bytes(f, f.rows), s>>>(f, bt, grad, tws, rows, kx, c, scal);
+    const auto kern = (uintptr_t)grad % sizeof(float2) ? k_fft_rows_inv<true, false>
+                                                       : k_fft_rows_inv<true, true>;
+    kern<<<(unsigned)((rows + f.rows - 1) / f.rows), f.threads, fft_bytes(f, f.rows), s>>>(
+        f, bt, grad, tws, rows, kx, c, scal);
     return cudaGetLastError();
 }
 

@@ -2634,6 +2634,9 @@ fresco_status fresco_uwu_plan(fresco_uwu_t *out, int dim, const int64_t *grid, c
 fresco_status fresco_uwu_loss_grad(fresco_uwu_t u, const void *d_c, double *d_loss, void *d_grad) {
     fresco::clear_pending_error();
     if (!u || !d_c || !d_loss) return FRESCO_ERR_ARG;
+    // (weights are loaded in pairs; cuFFT, which takes the other grids, asks for the same and answers
+    // with this error)
+    if (u->own && !aligned(d_c, sizeof(float2))) return FRESCO_ERR_CUFFT;
     if (u->precision == FRESCO_F64)
         return uwu_eval<double>(u, (const double *)d_c, d_loss, (double *)d_grad);
     return uwu_eval<float>(u, (const float *)d_c, d_loss, (float *)d_grad);
