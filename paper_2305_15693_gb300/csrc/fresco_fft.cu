@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
 
 // The columns of the weights-on-a-grid form (exact transforms, no kernel): S = |rho|^2 / rho0, the
 // loss and F = sum W S (S - S0), and (E / 2) rho, E = 4 W (S - S0) / rho0, back along y. Both sums
-// keep float pairs (products and sums with their errors) as the point form's loss does. scal[0] =
-// rho0 on entry; the last block leaves the loss (and its constant) in scal[2] and *loss, F in scal[3].
+// run in FP64 term by term, as in the cuFFT form (k_uwu_mask). scal[0] = rho0 on entry; the last
+// block leaves the loss (and its constant) in scal[2] and *loss, F in scal[3].
 __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
     k_fft_cols_w(const __grid_constant__ FftDesc f, const __grid_constant__ ColsArgs a,
                  double loss_const, double *__restrict__ scal, double *__restrict__ loss,
@@ -344,25 +344,15 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
         fft_forward(f, 1, s, 0, [&](int, int i) { return in[i]; });
         const double inv_rho0 = 1.0 / scal[0];
         const float inv = (float)inv_rho0;
-        float lh = 0.f, ll = 0.f, fh = 0.f, fl = 0.f;
         for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
             const int ny = a.rep_n[2 * e + 1];
             const int p = fft_place(f, __ldg(f.pos + (ny < 0 ? ny + n : ny)));
             const float2 F = s[p];
-            const float S = (F.x * F.x + F.y * F.y) * inv, w = a.rep_w[e];
-            float dh, dl, sh, se;
-            two_sum(S, -a.rep_s0[e], dh, dl);
-            const float pr = dh * dh, pl = fmaf(2.f * dh, dl, fmaf(dh, dh, -pr));
-            const float th = w * pr, tl = fmaf(w, pl, fmaf(w, pr, -th));
-            two_sum(lh, th, sh, se);
-            lh = sh;
-            ll += se + tl;
-            const float ws = w * S, wse = fmaf(w, S, -ws);
-            const float uh = ws * dh, ul = fmaf(ws, dl, fmaf(wse, dh, fmaf(ws, dh, -uh)));
-            two_sum(fh, uh, sh, se);
-            fh = sh;
-            fl += se + ul;
-            const float h = (float)(2.0 * (double)w * ((double)dh + (double)dl) * inv_rho0);
+            const float S = (F.x * F.x + F.y * F.y) * inv;
+            const double w = (double)a.rep_w[e], d = (double)S - (double)a.rep_s0[e];
+            bl = fma(w * d, d, bl);
+            bf = fma(w * (double)S, d, bf);
+            const float h = (float)(2.0 * w * d * inv_rho0);
             s[p] = {h * F.y, h * F.x};   // parts exchanged for the inverse
             atomicOr(&bits[p >> 5], 1u << (p & 31));
             if (k == 0) {
@@ -377,8 +367,8 @@ __global__ void __launch_bounds__(kFftThreads, kFftBlocks)
         __syncthreads();
         float2 *out = a.bt + (int64_t)k * n;
         fft_adjoint(f, 1, s, 0, [&](int, int i, float2 v) { out[i] = {v.y, v.x}; });
-        bl = block_sum((double)lh + (double)ll);
-        bf = block_sum((double)fh + (double)fl);
+        bl = block_sum(bl);
+        bf = block_sum(bf);
     }
     if (threadIdx.x == 0) {
         a.partial[k] = bl;

@@ -2271,18 +2271,19 @@ __device__ __forceinline__ double uwu_block_sum(double v) {
     return b;
 }
 
-// *out = sum c^2; the block that finishes last adds the partial sums in a fixed order
+// *out = sum c^2, every square in FP64 (in FP32 those of weights below 1e-19 lose their digits and
+// below 3e-23 vanish); the block that finishes last adds the partial sums in a fixed order
 template <typename T>
 __global__ void __launch_bounds__(256) k_uwu_sumsq(const T *__restrict__ c, int64_t n,
                                                    double *__restrict__ part,
                                                    unsigned *__restrict__ done,
                                                    double *__restrict__ out) {
     __shared__ bool s_last;
-    fresco::DotAcc<T> acc;
+    double acc = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        acc.add(c[i], c[i]);
-    const double b = uwu_block_sum(acc.value());
+        acc = fma((double)c[i], (double)c[i], acc);
+    const double b = uwu_block_sum(acc);
     if (threadIdx.x == 0) {
         part[blockIdx.x] = b;
         __threadfence();
