@@ -626,28 +626,6 @@ fresco_status make_ffts(fresco_plan_s *p) {
 // also takes up to 4 KB of static shared state and 1 KB the hardware reserves; 228 KB per SM).
 int tile_blocks_per_sm(size_t dyn) { return (int)((228 * 1024) / (dyn + 5 * 1024)); }
 
-// Tiles per z-column segment of the 3D column spread. A block walks one segment, so the segments
-// set the number of blocks: the length taken makes (waves of blocks) x (tiles of a segment + 1)
-// smallest, the 1 standing for a segment's start and end (zeroing, the extra planes, the z fold).
-// Small and middle grids no longer end in a nearly empty wave; large ones, with tens of waves, come
-// out near the former fixed length of 6. Measured: 20011 FP64 points (100 columns of 10 tiles),
-// 6 -> 4; 2^21 FP32 points (144 columns of 27), 6 -> 14.
-int z_segment(const Geom &g, size_t smem) {
-    const int64_t slots = 152 * std::min(2, std::max(1, tile_blocks_per_sm(smem)));
-    const int64_t cols = (int64_t)g.nb[0] * g.nb[1];
-    int best = 1;
-    double best_cost = 1e300;
-    for (int zs = std::min(2, g.nb[2]); zs <= std::min(kZSegmentMax, g.nb[2]); ++zs) {
-        const int64_t blocks = cols * ((g.nb[2] + zs - 1) / zs);
-        const double cost = (double)((blocks + slots - 1) / slots) * (zs + 1);
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = zs;
-        }
-    }
-    return best;
-}
-
 // TMA staging of the kernel-derivative interpolation (FP32 plans): the real field h, [nf2][nf1]
 // [nf0] floats, as a tensor whose boxes cover a tile's region from the 16-byte boundary at or
 // below its first column (rows up to 3 elements wider than the region). Sets g.tma and g.tbox
@@ -739,7 +717,9 @@ fresco_status build_plan(fresco_plan_s *p, const Params &P, const Folded &F) {
     g.sub = kTileCursors;   // own-points spread: no border strips; sub-cursors per tile
     g.zseg = dim == 3 && P.tmax[2] + P.width <= kColMaxPlanes ? 1 : 0;
     g.width = P.width;
-    if (g.zseg) g.zseg = z_segment(g, (size_t)Launch<T>::spread_own_smem(g));
+    if (g.zseg)
+        g.zseg = z_segment(g.nb, tile_blocks_per_sm((size_t)Launch<T>::spread_own_smem(g)),
+                           sizeof(T) == 4);
     for (int a = 0; a < 3; ++a) g.strips[a] = 0;
     g.n_bins = g.n_tiles * g.sub;
     if (g.n_bins >= 2147483647LL) return FRESCO_ERR_UNSUPPORTED;
@@ -1205,8 +1185,11 @@ fresco_status fresco::point_side_build(PointSide &ps, int dim, const int nf[3], 
     g.width = width;
     g.zseg = dim == 3 && P.tmax[2] + width <= kColMaxPlanes ? 1 : 0;
     if (g.zseg)
-        g.zseg = z_segment(g, es == 8 ? (size_t)Launch<double>::spread_own_smem(g)
-                                      : (size_t)Launch<float>::spread_own_smem(g));
+        g.zseg = z_segment(g.nb,
+                           tile_blocks_per_sm(es == 8
+                                                  ? (size_t)Launch<double>::spread_own_smem(g)
+                                                  : (size_t)Launch<float>::spread_own_smem(g)),
+                           es == 4);
     g.n_bins = g.n_tiles * g.sub;
     g.n_points = n_points;
     g.beta = beta;

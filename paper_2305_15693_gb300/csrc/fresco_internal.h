@@ -17,7 +17,8 @@ constexpr int kMaxWidth = 16;     // largest ES kernel width instantiated
 constexpr int kMinWidth = 2;
 constexpr int kMaxTileEdge = 255; // tile-relative cell must fit the 8-bit field of a packed coordinate
 constexpr int kTileCursors = 4;   // placement cursors per tile of a single plan (Geom.sub)
-constexpr int kZSegmentMax = 16;  // 3D single plans: most tiles per z-column segment (Geom.zseg)
+// 3D single plans: most tiles per z-column segment (Geom.zseg, z_segment)
+constexpr int kZSegmentFixed = 6, kZSegmentMax = 16;
 constexpr int kColMaxPlanes = 64; // column spread: tiles with tmax_z + w above this spread one by one
 // ints from one tile's cursor to the next: an L2 line each. Atomics on one line run one at a time,
 // and packed cursors of a small grid are few lines: k_place_direct, 4e5 points on 144 tiles 80 us
@@ -95,6 +96,31 @@ struct Geom {
 // the direct form's cursors and, after them, the overflow word
 inline size_t cursor_bytes(const Geom &g) {
     return sizeof(int) * (size_t)(g.n_tiles + 1) * kCursorStride;
+}
+
+// Tiles per z-column segment of the 3D column spread. A block walks one segment, so the segments
+// set the number of blocks: the length taken makes (waves of blocks) x (tiles of a segment + 1)
+// smallest, the 1 standing for a segment's start and end (zeroing, the extra planes, the z fold), so
+// that a small grid does not end in a nearly empty wave (20011 FP64 points, 100 columns of 10 tiles:
+// segments of 4). fixed: the spread adds in fixed point (FP32), and the tiles of a segment share the
+// scale that its most crowded tile sets, or all fall back to float atomics when that tile is too
+// crowded for any. Longer segments would hand a crowded tile's coarser quantum to more tiles, so
+// these stay at kZSegmentFixed (2^21 uniform points, 144 columns of 27 tiles, run fastest at 14).
+inline int z_segment(const int nb[3], int blocks_per_sm, bool fixed) {
+    const int64_t slots = 152 * std::min(2, std::max(1, blocks_per_sm));
+    const int64_t cols = (int64_t)nb[0] * nb[1];
+    const int most = std::min(fixed ? kZSegmentFixed : kZSegmentMax, nb[2]);
+    int best = 1;
+    double best_cost = 1e300;
+    for (int zs = std::min(2, nb[2]); zs <= most; ++zs) {
+        const int64_t blocks = cols * ((nb[2] + zs - 1) / zs);
+        const double cost = (double)((blocks + slots - 1) / slots) * (zs + 1);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = zs;
+        }
+    }
+    return best;
 }
 
 // Fills g.fdw and g.fdp from g.tq and g.width (host).
