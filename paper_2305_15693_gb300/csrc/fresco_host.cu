@@ -673,23 +673,6 @@ void setup_interp_tma(fresco_plan_s *p, const void *field) {
     g = t;
 }
 
-// Records per tile of the direct binning form: the expected points of the widest tile (uniform
-// density) plus eight Poisson standard deviations and 32, so that uniform and near-uniform inputs
-// never overflow a tile. 0 (compact form only) where the slots would not be indexable in 32 bits
-// or would take more than four times the points' records.
-int direct_tile_capacity(const Geom &g) {
-    double cells = 1.0, tile = 1.0;
-    for (int a = 0; a < g.dim; ++a) {
-        cells *= (double)g.nf[a];
-        tile *= (double)g.tmax[a];
-    }
-    const double mu = (double)g.n_points / cells * tile;
-    const double cap = std::ceil(mu + 8.0 * std::sqrt(mu) + 32.0);
-    const double slots = cap * (double)g.n_tiles;
-    if (slots >= 2147483647.0 || slots > 4.0 * (double)g.n_points + 1048576.0) return 0;
-    return (int)cap;
-}
-
 template <typename T>
 fresco_status build_plan(fresco_plan_s *p, const Params &P, const Folded &F) {
     using C2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
@@ -725,7 +708,8 @@ fresco_status build_plan(fresco_plan_s *p, const Params &P, const Folded &F) {
     if (g.n_bins >= 2147483647LL) return FRESCO_ERR_UNSUPPORTED;
     g.n_points = p->n_points;
     g.beta = P.beta;
-    g.tcap = direct_tile_capacity(g);
+    const double all[3] = {(double)g.nf[0], (double)g.nf[1], (double)g.nf[2]};
+    g.tcap = direct_tile_capacity(g, all);
     set_tile_divisors(g);
 
     MaskGeom &m = p->mgeom;
@@ -1144,8 +1128,8 @@ void fresco::point_side_free(PointSide &ps) {
 }
 
 fresco_status fresco::point_side_build(PointSide &ps, int dim, const int nf[3], const double box[3],
-                                       int64_t n_points, int width, double beta, int precision,
-                                       cudaStream_t s) {
+                                       const double extent[3], int64_t n_points, int width,
+                                       double beta, int precision, cudaStream_t s) {
     Params P{};
     P.dim = dim;
     P.precision = precision;
@@ -1193,7 +1177,7 @@ fresco_status fresco::point_side_build(PointSide &ps, int dim, const int nf[3], 
     g.n_bins = g.n_tiles * g.sub;
     g.n_points = n_points;
     g.beta = beta;
-    g.tcap = direct_tile_capacity(g);
+    g.tcap = direct_tile_capacity(g, extent);
     set_tile_divisors(g);
     ps.precision = precision;
     const int64_t cells = (int64_t)g.nf[0] * g.nf[1] * g.nf[2];

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "fresco.h"
@@ -121,6 +122,26 @@ inline int z_segment(const int nb[3], int blocks_per_sm, bool fixed) {
         }
     }
     return best;
+}
+
+// Records per tile of the direct binning form: the expected points of the widest tile (points uniform
+// over `extent` cells per axis: the whole grid of a periodic plan, the box's cells where the grid has
+// spare ones around it) plus eight Poisson standard deviations and 32, so that uniform and
+// near-uniform inputs never overflow a tile (an overflow pays for the direct pass and then for the
+// compact form). 0 (compact form only) where the slots would not be indexable in 32 bits or would
+// take more than four times the points' records.
+inline int direct_tile_capacity(const Geom &g, const double extent[3]) {
+    double cells = 1.0, tile = 1.0;
+    for (int a = 0; a < g.dim; ++a) {
+        const double e = std::min(std::max(extent[a], 1.0), (double)g.nf[a]);
+        cells *= e;
+        tile *= std::min((double)g.tmax[a], e);
+    }
+    const double mu = (double)g.n_points / cells * tile;
+    const double cap = std::ceil(mu + 8.0 * std::sqrt(mu) + 32.0);
+    const double slots = cap * (double)g.n_tiles;
+    if (slots >= 2147483647.0 || slots > 4.0 * (double)g.n_points + 1048576.0) return 0;
+    return (int)cap;
 }
 
 // Fills g.fdw and g.fdp from g.tq and g.width (host).
@@ -359,9 +380,10 @@ struct PointSide {
     int64_t device_bytes = 0;
     std::vector<void *> allocs;
 };
+// extent: cells per axis the points lie in (the grid keeps spare ones beyond them), 1 beyond dim.
 fresco_status point_side_build(PointSide &ps, int dim, const int nf[3], const double box[3],
-                               int64_t n_points, int width, double beta, int precision,
-                               cudaStream_t s);
+                               const double extent[3], int64_t n_points, int width, double beta,
+                               int precision, cudaStream_t s);
 void point_side_free(PointSide &ps);
 template <typename T>
 fresco_status point_side_spread(PointSide &ps, const T *pts, cudaStream_t s, int64_t *launches);

@@ -1356,12 +1356,13 @@ fresco_status nu_build(fresco_nuwnu_s *p, const double *kvec, const double *S0, 
     UN_CUDA(cudaMemcpy(u->scal, &norm, sizeof(double), cudaMemcpyHostToDevice));
     // point side: the n1 grid over the periodic box n1 h
     int n1[3] = {1, 1, 1};
-    double pbox[3] = {1, 1, 1};
+    double pbox[3] = {1, 1, 1}, extent[3] = {1, 1, 1};
     for (int a = 0; a < dim; ++a) {
         n1[a] = u->g.M[a];
         pbox[a] = (double)n1[a] * p->h[a];
+        extent[a] = p->box[a] / p->h[a];
     }
-    st = fresco::point_side_build(p->ps, dim, n1, pbox, p->n_points, u->width, u->beta,
+    st = fresco::point_side_build(p->ps, dim, n1, pbox, extent, p->n_points, u->width, u->beta,
                                   p->precision, p->stream);
     if (st) return st;
     UN_CUDA(cudaDeviceSynchronize());
