@@ -840,15 +840,14 @@ fresco_status un_build(fresco_uwnu_s *u, const double *nu, const double *S0, con
     const int dim = g.dim;
     const int64_t nk = u->n_k;
     const int w = u->width;
-    // real grids (2D FP32) whose transforms fit the shared memory of the library's own kernels; the
-    // margins of the half plane must not overlap
-    u->real = dim == 2 && sizeof(T) == 4 && g.nf[0] >= 4 * w + 2 &&
+    // real grids (2D FP32) whose transforms fit the shared memory of the library's own kernels, with
+    // tiles enough for the constraints; the margins of the half plane must not overlap
+    u->real = dim == 2 && sizeof(T) == 4 && g.nf[0] >= 4 * w + 2 && half_plane_pays(g.nf, w, nk) &&
               fresco::fft_describe(g.nf[0] / 2, u->fx) && fresco::fft_describe(g.nf[1], u->fy);
     u->ug = g;
     if (u->real) {
         u->rg = RealGrid{g.M[0], g.M[1], g.nf[0], g.nf[1], w, centred};
-        u->ug.nf[0] = g.nf[1];
-        u->ug.nf[1] = g.nf[0] / 2 + 2 * w + 1;
+        half_plane_cells(g.nf, w, u->ug.nf);
         u->fine = (int64_t)u->ug.nf[0] * u->ug.nf[1];
     }
     const int *tnf = u->ug.nf;   // the constraint side's grid

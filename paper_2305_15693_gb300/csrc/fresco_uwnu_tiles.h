@@ -44,6 +44,29 @@ inline UTiles utiles_for(int dim, const int nf[3]) {
     return tl;
 }
 
+// Cells of the half plane that the real 2D form keeps of a fine grid: rows l_x = -w .. nf_x / 2 + w,
+// transposed (axis 0 is y).
+inline void half_plane_cells(const int nf[3], int w, int h[3]) {
+    h[0] = nf[1];
+    h[1] = nf[0] / 2 + 2 * w + 1;
+    h[2] = 1;
+}
+
+// Whether a real 2D plan of n_k constraints runs on the half plane. Its transforms save about 30 us,
+// but its constraint side has about half as many tiles, each with twice the constraints, and a block
+// takes one tile: where the tiles are too few to fill the chip twice over, crowded tiles cost more
+// than the transforms save. Measured on GB300, whole plane / half plane (us; tiles of the half plane,
+// constraints per such tile): 64^2 weights (12 tiles) 10^4 constraints (833) 81 / 79, 10^5 240 / 377;
+// 112^2 (28) 10^4 (357) 72 / 60, 10^5 (3571) 126 / 163; 160^2 (60) 10^5 (1667) 99 / 110; 256^2 (144)
+// 10^5 (694) 89 / 79, 10^6 (6944) 204 / 279; 400^2 (350) 10^6 190 / 168.
+inline bool half_plane_pays(const int nf[3], int w, int64_t n_k) {
+    int h[3];
+    half_plane_cells(nf, w, h);
+    const UTiles tl = utiles_for(2, h);
+    const int64_t tiles = (int64_t)tl.nt[0] * tl.nt[1];
+    return tiles >= 2 * 152 || n_k <= 700 * tiles;
+}
+
 // origin and extent of tile t
 inline void utile_box(const UTiles &tl, const int nf[3], int64_t t, int o[3], int len[3]) {
     const int tc[3] = {(int)(t % tl.nt[0]), (int)((t / tl.nt[0]) % tl.nt[1]),
