@@ -327,8 +327,8 @@ fresco_status fresco_lbfgs_destroy(fresco_lbfgs_t s);
  * the same precision and tolerance). Their points are packed one instance after the other in a
  * single device array; every stage (sort, spread, mask, interpolation) runs as one launch over
  * all instances. The uniform FFTs run per size class (fine grids rounded up to 2^k or 3 2^k): FP32
- * in the library's own kernels, up to sixteen classes in a launch; FP64 as one batched cuFFT call
- * per class and direction. The result for instance i is exactly what
+ * in the library's own kernels, up to sixteen classes in a launch, unless few classes hold very many
+ * cells; those, and FP64, as one batched cuFFT call per class and direction. The result for instance i is exactly what
  * fresco_plan / fresco_loss_grad give for that problem alone (up to the larger fine grid). */
 typedef struct fresco_batch_s *fresco_batch_t;
 

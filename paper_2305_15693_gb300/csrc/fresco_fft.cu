@@ -613,10 +613,10 @@ constexpr double kOwnCells = 1.2e6;
 fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int64_t rows,
                             bool always) {
     // 2D single grids beyond kOwnCells stay on cuFFT, whose larger radices then outweigh its extra
-    // passes over memory; ensembles (many grids, launches per size class) and the 3D rows do not.
+    // passes over memory; ensembles (fft_ensemble_pays) and the 3D rows have rules of their own.
     // Measured, x passes, y passes and mask, cuFFT against these kernels (us): 432^2 46 / 36, 784^2
-    // 53 / 38, 2500^2 95 / 109, 6480^2 448 / 471; ensemble of 128 410 / 173; the 324^3 grid's x
-    // passes with cuFFT's (z, y) transforms 468 / 374
+    // 53 / 38, 2500^2 95 / 109, 6480^2 448 / 471; the 324^3 grid's x passes with cuFFT's (z, y)
+    // transforms 468 / 374
     if (dim == 2 && !always && (double)nf[0] * nf[1] > kOwnCells) return FRESCO_OK;
     // (the kernels work on whole rows of nf[0] floats; nf[0] is even)
     f.fwd = fft_describe(nf[0] / 2, f.x);

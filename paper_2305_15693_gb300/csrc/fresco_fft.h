@@ -144,6 +144,16 @@ struct FftSet {
 // not fit keep cuFFT, and, unless `always`, all of a 2D grid on which cuFFT's are the faster ones.
 fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int64_t rows,
                             bool always);
+// Whether an FP32 ensemble of `cells` fine-grid cells in all, in so many size classes, runs these
+// transforms: they save the library form's launches, six and more for every class, and cost more per
+// cell (the direct mode's above all, with two columns and complex rows back). Measured on GB300,
+// transforms and mask, cuFFT / these kernels (us). kderiv: one class of 4.2e6 cells 58 / 55, 9.4e6
+// (3072^2) 129 / 111, 1.7e7 (16 grids of 1024^2) 127 / 146, 6.7e7 (64 of 1024^2) 434 / 515, 7.5e7 (two
+// of 6144^2) 634 / 655; nine classes of 1.6e7 together 427 / 160. Direct: 2.4e6 73 / 71, 4.2e6 (four of
+// 1024^2) 76 / 82, 9.4e6 163 / 176, 6.7e7 573 / 830; nine classes 488 / 299, two of 2.1e7 278 / 316.
+inline bool fft_ensemble_pays(double cells, int classes, bool kderiv) {
+    return cells <= (kderiv ? 1.0e7 : 4.0e6) * classes;
+}
 void fft_set_free(FftSet *f);
 // first[k] = index of the first representative with n_x >= k, k = 0 .. kx + 1 (rep_n is n_x major)
 std::vector<int> rep_columns(const std::vector<int32_t> &rep_n, int dim, int kx);

@@ -1614,11 +1614,15 @@ fresco_status batch_build(fresco_batch_s *b, const std::vector<Params> &P,
         reo += nrep;
         I.loss_const = F[i].loss_const;
     }
-    // FP32 ensembles whose every size class fits run the library's own transforms; an instance's loss
-    // partials are then one per column of its class
-    b->own_fft = sizeof(T) == 4;
-    int64_t all_rows = 0;
-    for (auto &K : b->cls) all_rows += (int64_t)K.nf[1] * K.count;
+    // FP32 ensembles whose every size class fits run the library's own transforms where these pay; an
+    // instance's loss partials are then one per column of its class
+    int64_t all_rows = 0, all_cells = 0;
+    for (auto &K : b->cls) {
+        all_rows += (int64_t)K.nf[1] * K.count;
+        all_cells += (int64_t)K.nf[0] * K.nf[1] * K.count;
+    }
+    b->own_fft = sizeof(T) == 4 && fresco::fft_ensemble_pays((double)all_cells, (int)b->cls.size(),
+                                                             b->kderiv != 0);
     for (auto &K : b->cls) {
         if (!b->own_fft) break;
         K.own = new (std::nothrow) fresco::FftSet();
