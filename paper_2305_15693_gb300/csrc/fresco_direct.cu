@@ -21,8 +21,9 @@
 // (the NUFFT adds its kernel's truncation).
 //
 // What bounds it: FP64 the FP64 pipe; FP32 shared-memory loads; at the smallest sizes the three
-// launches. The line between the two forms (kDirectWork) lies where they measured equal on GB300;
-// see direct_build.
+// launches; with few points the gradient's walk over all cells, which every block makes for its
+// eight points. The line between the two forms (kDirectWork, kDirectCost) lies where they measured
+// equal on GB300; see direct_build.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -472,6 +473,25 @@ struct DirectPlan {
 // 29, 3.0e7: 82 / 46, 6.0e7: 91 / 67; 3D, 1.7e7: 123 / 41, 4.6e7: 134 / 99. FP64, 2D, 3.2e6: 206 /
 // 81, 4.9e6: 279 / 111, 1.3e7: 200 / 252; 3D, 6.1e6: 391 / 198.
 static constexpr double kDirectWork[2] = {4.0e7, 9.0e6};   // FP32, FP64
+// With few points most SMs idle, the time is that of one block and the wavevectors alone decide;
+// the product above does not see it (100 points and K = 500 took 1226 us, the NUFFT 185). Estimates
+// of both forms in us, [precision][dimension - 2]; the NUFFT's without its points, few in every plan
+// that gets here. Fitted to 170 pairs of plans of 1 to 8000 points with disks, balls, strips and
+// sparse masks of |n| up to 4000, on both sides of the line. Direct sums / NUFFT: 2D FP32, 300
+// points, K = 60 31 / 55, 100 55 / 57, 130 75 / 58, 200 160 / 70; 10 points, 30 wavevectors of |n| up
+// to 2000 170 / 1315, a strip of 4000 x 1 163 / 94; 2D FP64, 300 points, K = 60 100 / 142, 80 156 /
+// 136; K = 50 and 1000 points 100 / 130, 2000 points 157 / 134; 3D, K = 12, 2000 points 35 / 127,
+// FP64 221 / 369.
+struct DirectCost {
+    double fixed, quad, row;         // launches; a quad, a quad row of one block's walk
+    double pt_quad, pt_phase;        // a point's share of the sums over a quad, of one phase
+    double nufft, nufft_cell;        // the NUFFT's launches, 10^6 cells of its fine grid
+};
+static constexpr DirectCost kDirectCost[2][2] = {
+    {{18.0, 0.0152, 0.11, 2.0e-6, 1.4e-5, 55.0, 20.0},
+     {15.0, 0.029, 0.11, 6.5e-6, 1.4e-5, 100.0, 100.0}},
+    {{22.0, 0.097, 0.15, 3.4e-5, 6.0e-5, 110.0, 250.0},
+     {25.0, 0.27, 0.15, 3.4e-5, 6.0e-5, 190.0, 900.0}}};
 // Tolerances the plan may ask for: the direct sums carry the working precision, so a plan that
 // states a looser tolerance keeps the NUFFT whose error it expects (and its speed at that width).
 static constexpr double kDirectTol[2] = {1.0e-5, 1.0e-9};
@@ -545,9 +565,10 @@ static fresco_status build_t(DirectPlan *d, const std::vector<int2> &cols,
 }
 
 // Builds the direct form of a plan, or leaves *out null where the NUFFT is the better one. mask:
-// the caller's rows; rep_n, rep_s0, rep_w: the folded representatives (n_x >= 0 half).
+// the caller's rows; rep_n, rep_s0, rep_w: the folded representatives (n_x >= 0 half); fine_cells:
+// cells of the fine grid the NUFFT would use.
 fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const double *box,
-                           int precision, const int32_t *mask, int64_t n_k,
+                           int precision, double fine_cells, const int32_t *mask, int64_t n_k,
                            const std::vector<int32_t> &rep_n, const std::vector<double> &rep_s0,
                            const std::vector<double> &rep_w, double loss_const) {
     *out = nullptr;
@@ -614,6 +635,13 @@ fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const do
     g.n_col = (int)cols.size();
     g.n_quad = (int)quads.size();
     if (8.0 * g.n_quad * (double)n_points > 1.25 * work) return FRESCO_OK;
+    const DirectCost &c = kDirectCost[precision == FRESCO_F64][dim - 2];
+    // FP64: the walk is bound by the FP64 pipe, which further blocks on an SM share
+    const double turns =
+        precision == FRESCO_F64 ? std::max(1.0, (double)n_points / (152.0 * 8.0)) : 1.0;
+    const double sums = c.fixed + c.quad * g.n_quad * turns + c.row * (g.nx4 / 4) +
+                        (double)n_points * (c.pt_quad * g.n_quad + c.pt_phase * (g.nx4 + g.n_col));
+    if (sums > c.nufft + c.nufft_cell * fine_cells * 1e-6) return FRESCO_OK;
     // one point's phases must fit the shared memory of both kernels
     const size_t es = precision == FRESCO_F64 ? 8 : 4;
     if ((precision == FRESCO_F64 ? direct_rho_smem<double>(g, 1) : direct_rho_smem<float>(g, 1)) >

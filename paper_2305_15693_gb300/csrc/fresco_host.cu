@@ -1350,8 +1350,9 @@ fresco_status fresco_plan(fresco_plan_t *out, int dim, const double *box, int64_
     fresco_opts_default(&o);
     if (opts) o = *opts;
     if (fresco::direct_wanted(n_points, o, P.precision, P.tol))
-        st = fresco::direct_build(&p->direct, dim, n_points, box, P.precision, mask, n_k, F.n, F.s0,
-                                  F.w, F.loss_const);
+        st = fresco::direct_build(&p->direct, dim, n_points, box, P.precision,
+                                  (double)P.nf[0] * P.nf[1] * P.nf[2], mask, n_k, F.n, F.s0, F.w,
+                                  F.loss_const);
     if (!st && p->direct) {
         p->device_bytes += fresco::direct_bytes(p->direct);
         st = dalloc(p, &p->d_err, sizeof(int));

@@ -405,7 +405,7 @@ struct FftSet;   // fresco_fft.h
 struct FftClassSet;
 bool direct_wanted(int64_t n_points, const fresco_opts &o, int precision, double tol);
 fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const double *box,
-                           int precision, const int32_t *mask, int64_t n_k,
+                           int precision, double fine_cells, const int32_t *mask, int64_t n_k,
                            const std::vector<int32_t> &rep_n, const std::vector<double> &rep_s0,
                            const std::vector<double> &rep_w, double loss_const);
 void direct_free(DirectPlan *d);
