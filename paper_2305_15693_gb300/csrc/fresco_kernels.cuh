@@ -975,7 +975,7 @@ __device__ __forceinline__ void interp_tile(const Geom &g, const EsPoly<T> &ep,
 
     const T scale = grad_out ? (T)(*grad_out) : T(1);
     if constexpr (sizeof(T) == 8 && D == 3) {
-        if (p1 - p0 <= kWarpPointMax) {
+        if (p1 - p0 <= warp_point_max(W, false)) {
             // one warp per point (spread_points_owned above has the reason): a lane takes every 32nd
             // (y, z) row of the window. 3D, 20011 points, w = 13: interpolation 2038 -> 541 us
             double *sw = reinterpret_cast<double *>(sm_raw + (sizeof(C) + sizeof(T)) * (size_t)cells);
@@ -1452,7 +1452,7 @@ __device__ __forceinline__ void interp_tile_kd(const Geom &g, const EsPoly<T> &e
     __syncthreads();
     if (!ok) return;
     if constexpr (sizeof(T) == 8 && D == 3) {
-        if (p1 - p0 <= kWarpPointMax) {
+        if (p1 - p0 <= warp_point_max(W, true)) {
             // one warp per point, as in interp_tile
             double *sw = reinterpret_cast<double *>(sm_raw + interp_kd_tile_bytes(g, sizeof(T)));
             int *si = reinterpret_cast<int *>(sw + kOwnedChunkInterp * D * 2 * W);
@@ -1875,9 +1875,10 @@ int Launch<T>::spread_own_smem(const Geom &g) {
     // packed window start and D kernel offsets
     const size_t region = g.dim == 3 && g.zseg > 0 ? spread_col_tile_bytes(g, sizeof(T))
                                                    : spread_own_tile_bytes(g, sizeof(T));
-    // (FP32), or the staged weights of a chunk of points (FP64)
-    return (int)(region + (sizeof(T) == 4 ? (size_t)(1 + g.dim) * 4 * (size_t)g.list_cap
-                                          : owned_bytes(kOwnedChunk, g.dim, g.width, false)));
+    // (FP32), or the staged weights of a chunk of points (FP64 kernels wide enough, kOwnedSpread)
+    return (int)(region + (sizeof(T) == 4       ? (size_t)(1 + g.dim) * 4 * (size_t)g.list_cap
+                           : g.width >= kOwnedWidth ? owned_bytes(kOwnedChunk, g.dim, g.width, false)
+                                                : 0));
 }
 
 template <typename T>

@@ -623,10 +623,16 @@ __device__ __forceinline__ int residue_lists(const typename PT<T>::U *__restrict
 // multiply-add per window cell.
 constexpr int kOwnedChunk = 32;       // spread: points whose weights are staged at once
 constexpr int kOwnedChunkInterp = 8;  // interpolation: one point per warp (the field leaves little room)
-// Interpolation tiles of more points than this go back to one thread per point: a full block of
-// 256 points takes 472 us (direct) or 353 us (kernel derivative) at w = 13 on one SM, a point
-// taken by a warp 2.7 us.
-constexpr int kWarpPointMax = 128;
+// 3D interpolation tiles of at most this many points give each a warp, others a thread: a warp's time
+// per point hardly falls with the kernel's width, a thread's falls with its cube. Where the two meet,
+// from the interpolation stage of 180 plans (3000 to 3 10^5 points, w = 3 .. 13), threads / warps (us):
+// kernel derivative, w = 3, 6 points a tile 26 / 24, 10 77 / 97, 50 83 / 286; w = 5, 15 72 / 51, 36
+// 205 / 340; w = 7, 21 92 / 73, 36 418 / 477; w = 10, 31 206 / 148, 45 829 / 862; w = 13, 38 5491 /
+// 4073, 51 3615 / 4058; direct, w = 4, 10 137 / 112, 15 98 / 102; w = 7, 36 621 / 536, 51 1379 / 1570;
+// w = 12, 51 9421 / 5012.
+__host__ __device__ constexpr int warp_point_max(int w, bool kderiv) {
+    return kderiv ? (w < 9 ? 6 * (w - 2) : 42) : 10 * (w - 3) + 3;
+}
 
 // bytes of the staged weights (and derivatives) and window starts of n points, 16-byte aligned
 __host__ __device__ inline size_t owned_bytes(int n, int dim, int w, bool deriv) {
@@ -684,8 +690,9 @@ __device__ __forceinline__ void stage_point_weights(const EsPoly<double> &ep,
 
 // The FP64 spread takes a tile's points this way when a window row pair fills enough threads; with
 // narrow kernels (W^2 < 64 threads of 256) one thread per point with atomics is the better one.
+constexpr int kOwnedWidth = 8;
 template <typename T, int W>
-constexpr bool kOwnedSpread = sizeof(T) == 8 && W >= 8;
+constexpr bool kOwnedSpread = sizeof(T) == 8 && W >= kOwnedWidth;
 
 // Adds the windows of points [p0, p1) to the region (planes of Sxy elements, rows of Ex) without
 // atomics: thread (a, b) owns every cell with x = a and y = b modulo W, of which each window holds
