@@ -162,7 +162,7 @@ fresco_status fresco_backward(fresco_plan_t p, const double *d_grad_out, void *d
 /* After fresco_forward: rho (interleaved re, im: device [n_k][2]) and S (device [n_k]) for the
  * mask rows in the order given to fresco_plan, in the plan's precision. Either may be NULL.
  * The first call uploads the mask and, in 2D FP32 plans with their own transforms, allocates a
- * second spectrum (allocates once). */
+ * second spectrum (allocates once; plans that run direct sums allocate nothing). */
 fresco_status fresco_get_rho_S(fresco_plan_t p, void *d_rho, void *d_S);
 
 /* End-to-end variant on host buffers: copies h_points (host, [N][dim] plan type) to the device,

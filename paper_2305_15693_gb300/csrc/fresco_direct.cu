@@ -462,8 +462,8 @@ struct DirectPlan {
     void *tab = nullptr;
     double *lpart = nullptr;
     unsigned *done = nullptr;
-    int *row_idx = nullptr;            // mask rows -> cell entries (fresco_get_rho_S, lazily)
-    std::vector<int> h_row_idx;
+    int *row_idx = nullptr;            // [n_k] mask rows -> cell entries (fresco_get_rho_S)
+    int64_t n_k = 0;
     int n_mask_blk = 0;
     int64_t bytes = 0;
 };
@@ -512,8 +512,10 @@ bool direct_wanted(const int64_t n_points, const fresco_opts &o, int precision, 
 template <typename T>
 static fresco_status build_t(DirectPlan *d, const std::vector<int2> &cols,
                              const std::vector<int2> &quads, const std::vector<int> &qbase,
-                             const std::vector<double> &s0, const std::vector<double> &w) {
+                             const std::vector<double> &s0, const std::vector<double> &w,
+                             const std::vector<int> &row_idx) {
     DirectGeom &g = d->g;
+    d->n_k = (int64_t)row_idx.size();
     size_chunks<T>(g);
     const size_t cells = 4 * (size_t)g.n_quad;
     const size_t n_part = (size_t)g.n_blk;
@@ -530,6 +532,7 @@ static fresco_status build_t(DirectPlan *d, const std::vector<int2> &cols,
     if (!(A((void **)&d->cols, sizeof(int2) * cols.size()) &&
           A((void **)&d->quads, sizeof(int2) * quads.size()) &&
           A((void **)&d->qbase, sizeof(int) * qbase.size()) &&
+          A((void **)&d->row_idx, sizeof(int) * row_idx.size()) &&
           A(&d->cell_s0, sizeof(T) * 2 * cells) && A(&d->cell_w, sizeof(T) * 2 * cells) &&
           A(&d->part, sizeof(T) * 4 * cells * n_part) && A(&d->dco, sizeof(T) * 4 * cells) &&
           A(&d->rho, sizeof(T) * 4 * cells) &&
@@ -547,6 +550,8 @@ static fresco_status build_t(DirectPlan *d, const std::vector<int2> &cols,
               cudaMemcpy(d->quads, quads.data(), sizeof(int2) * quads.size(),
                          cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(d->qbase, qbase.data(), sizeof(int) * qbase.size(),
+                         cudaMemcpyHostToDevice) == cudaSuccess &&
+              cudaMemcpy(d->row_idx, row_idx.data(), sizeof(int) * row_idx.size(),
                          cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(d->cell_s0, ts.data(), sizeof(T) * ts.size(), cudaMemcpyHostToDevice) ==
                   cudaSuccess &&
@@ -669,15 +674,15 @@ fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const do
     DirectPlan *d = new (std::nothrow) DirectPlan();
     if (!d) return FRESCO_ERR_OOM;
     d->g = g;
-    d->h_row_idx.resize((size_t)n_k);
+    std::vector<int> row_idx((size_t)n_k);
     for (int64_t q = 0; q < n_k; ++q) {
         const Entry e = entry(mask + q * dim);
         const int c = cell(e);
-        d->h_row_idx[(size_t)q] = e.neg ? -(c + 1) : c;
+        row_idx[(size_t)q] = e.neg ? -(c + 1) : c;
     }
     const fresco_status st = precision == FRESCO_F64
-                                 ? build_t<double>(d, cols, quads, qbase, s0, w)
-                                 : build_t<float>(d, cols, quads, qbase, s0, w);
+                                 ? build_t<double>(d, cols, quads, qbase, s0, w, row_idx)
+                                 : build_t<float>(d, cols, quads, qbase, s0, w, row_idx);
     if (st) {
         direct_free(d);
         return st;
@@ -721,18 +726,8 @@ cudaError_t direct_grad(DirectPlan *d, const double *grad_out, T *grad, cudaStre
 
 template <typename T>
 cudaError_t direct_rho_s(DirectPlan *d, T *rho, T *S, cudaStream_t s) {
-    const int64_t n_k = (int64_t)d->h_row_idx.size();
-    if (!d->row_idx) {
-        cudaError_t e = cudaMalloc((void **)&d->row_idx, sizeof(int) * (size_t)n_k);
-        if (e != cudaSuccess) return e;
-        d->allocs.push_back(d->row_idx);
-        d->bytes += (int64_t)sizeof(int) * n_k;
-        e = cudaMemcpyAsync(d->row_idx, d->h_row_idx.data(), sizeof(int) * (size_t)n_k,
-                            cudaMemcpyHostToDevice, s);
-        if (e != cudaSuccess) return e;
-    }
-    k_direct_rho_s<T><<<(unsigned)((n_k + 255) / 256), 256, 0, s>>>(
-        n_k, d->row_idx, (const Cx<T> *)d->rho, (T)d->g.inv_n, rho, S);
+    k_direct_rho_s<T><<<(unsigned)((d->n_k + 255) / 256), 256, 0, s>>>(
+        d->n_k, d->row_idx, (const Cx<T> *)d->rho, (T)d->g.inv_n, rho, S);
     return cudaGetLastError();
 }
 

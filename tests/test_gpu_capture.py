@@ -17,6 +17,31 @@ def _built():
     _build.build()
 
 
+def test_first_read_of_a_small_plan_can_be_recorded():
+    """A direct plan's first read of rho and S inside the recorded work: it allocates and uploads
+    nothing, and a read that was recorded and never replayed leaves nothing behind for later ones."""
+    import torch
+    from paper_2305_15693_gb300 import fresco
+    mask = inputs.ball_mask(9, 2)
+    x = torch.from_numpy(inputs.uniform_points(300, 2, 3)).cuda()
+    stream = torch.cuda.Stream()
+    loss = torch.zeros((), dtype=torch.float64, device="cuda")
+    rho = torch.zeros(len(mask), 2, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream), fresco.Plan(1.0, mask, np.zeros(len(mask)), np.ones(len(mask)),
+                                                300, precision="f64", stream=stream) as plan:
+        fresco.fresco_forward(plan.handle, x, loss)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            fresco.fresco_forward(plan.handle, x, loss)
+            fresco.fresco_get_rho_S(plan.handle, rho, None)
+        want, _ = plan.rho_S()          # (before any replay)
+        graph.replay()
+        stream.synchronize()
+        assert plan.launch_count() > 0 and torch.equal(rho, want)
+
+
 @pytest.mark.parametrize("mode", ["kderiv", "direct"])
 @pytest.mark.parametrize("dim,width,precision", [(2, 7, "f32"), (2, 0, "f32"), (3, 7, "f32"),
                                                  (2, 13, "f64")])
