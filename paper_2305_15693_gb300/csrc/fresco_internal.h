@@ -453,6 +453,23 @@ struct DotAcc<double> {
     __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
     __device__ __forceinline__ double value() const { return v; }
 };
+
+// A sum of floats no less exact than one in FP64: three floats, the parts that each addition drops kept
+// by two-sums (about 70 bits), without the narrow FP64 pipe. Terms and sum must stay well inside FP32's
+// range; the callers take others to FP64. (Additions by intrinsics: a product passed as x must not be
+// fused into them.)
+struct Sum3 {
+    float h = 0.f, m = 0.f, l = 0.f;
+    static __device__ __forceinline__ float add_rest(float &a, float b) {   // a += b; what that drops
+        const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+        a = s;
+        return e;
+    }
+    __device__ __forceinline__ void add_low(float x) { l += add_rest(m, x); }   // x << the sum
+    __device__ __forceinline__ void add(float x) { add_low(add_rest(h, x)); }
+    __device__ __forceinline__ double value() const { return ((double)l + (double)m) + (double)h; }
+};
 #endif
 
 }  // namespace fresco
