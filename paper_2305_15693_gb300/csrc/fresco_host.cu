@@ -2406,7 +2406,12 @@ fresco_status uwu_build(fresco_uwu_s *u, const Folded &F) {
     u->n_rep = (int64_t)F.s0.size();
     u->n_mask_blocks = std::max<int64_t>(1, std::min<int64_t>((u->n_rep + 255) / 256, kUwuBlocks));
     const size_t specT_n = (size_t)(u->kx + 1) * (size_t)u->plane;
-    if (sizeof(T) == 4 && dim == 2) {
+    // (columns of 16384, the one power of two that leaves an SM a single block, lose to cuFFT's on the
+    // largest grids: 16384^2, K = 1000 / 1500 / 4000, cuFFT 2800 / 2985 / 4350 us, own 2974 / 3294 / 5341;
+    // 8192 x 16384 1553 / 1447, 15360^2 3114 / 2700, 18432^2 4365 / 3500)
+    const bool lib_columns = u->M[1] >= 16384 && (u->M[1] & (u->M[1] - 1)) == 0 &&
+                             u->cells >= (1ll << 28);
+    if (sizeof(T) == 4 && dim == 2 && !lib_columns) {
         u->own = new (std::nothrow) fresco::FftSet();
         if (!u->own) return FRESCO_ERR_OOM;
         const fresco_status st = fresco::fft_set_build(*u->own, u->M, 2, true, u->M[1], true);
