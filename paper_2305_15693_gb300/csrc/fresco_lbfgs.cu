@@ -275,21 +275,23 @@ __global__ void __cluster_dims__(kTlBlocks, 1, 1) __launch_bounds__(kTlThreads)
 #pragma unroll
             for (int e = 0; e < E; ++e) bs[e] = nx[e];
     }
-    T mx = T(0);
+    T mx = T(0), gx = T(0);
     fresco::DotAcc<T> acc;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         v[e] = T(-1) * v[e];
-        if (i0 + e * ST < n) acc.add(g[i0 + e * ST], v[e]);
+        if (i0 + e * ST < n) {
+            const T ge = g[i0 + e * ST];
+            acc.add(ge, v[e]);
+            mx = fmax(mx, fabs(v[e]));
+            gx = fmax(gx, fabs(ge));
+        }
     }
     const double gd = total(acc.value(), false);
+    if (!(gd < 0.0))
 #pragma unroll
-    for (int e = 0; e < E; ++e)
-        if (i0 + e * ST < n) {
-            if (!(gd < 0.0)) v[e] = T(-1) * g[i0 + e * ST];
-            mx = fmax(mx, fabs(v[e]));
-        }
-    const double dmax = total((double)mx, true);
+        for (int e = 0; e < E; ++e) v[e] = i0 + e * ST < n ? T(-1) * g[i0 + e * ST] : T(0);
+    const double dmax = total((double)(gd < 0.0 ? mx : gx), true);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc[SL_GD] = gd;
         sc[SL_DMAX] = sc[SL_GMAX] = dmax;
