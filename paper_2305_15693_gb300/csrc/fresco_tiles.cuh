@@ -693,6 +693,14 @@ __device__ __forceinline__ void stage_point_weights(const EsPoly<double> &ep,
 constexpr int kOwnedWidth = 8;
 template <typename T, int W>
 constexpr bool kOwnedSpread = sizeof(T) == 8 && W >= kOwnedWidth;
+// In 2D a point's window fills W^2 threads with one cell each, so crowded tiles of the narrower kernels
+// go back to a thread per point, whose time falls with the width: points of a tile from which on they do.
+// Spread stage, a thread per point / owned cells (us), few tiles: w = 8, 250 points a tile 50 / 50, 1000
+// 132 / 167, 10^4 999 / 1421; w = 9, 1000 156 / 210; w = 10, 300 77 / 75, 1000 182 / 216; w = 11, 300 91 /
+// 78, 1000 212 / 224, 10^4 1653 / 1844; w = 12, 300 101 / 78, 10^4 1910 / 1873; w = 16, 10^4 2942 / 2009.
+__host__ __device__ constexpr int owned_point_max_2d(int w) {
+    return w < 10 ? 256 : (w == 10 ? 384 : (w == 11 ? 768 : 2147483647));
+}
 
 // Adds the windows of points [p0, p1) to the region (planes of Sxy elements, rows of Ex) without
 // atomics: thread (a, b) owns every cell with x = a and y = b modulo W, of which each window holds
@@ -798,11 +806,15 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_spread_own(
             for (int a = 0; a < D; ++a) x1[a] = (T)l_x1[a * cap + h];
             spread_point_own<T, W, D>(ep, i0, x1, Ex, Exy, ftile, itile, true, fscale);
         }
-    } else if constexpr (kOwnedSpread<T, W>) {
-        spread_points_owned<W, D>(ep, sorted, p0, p1, Ex, Exy, 0, 0, ftile,
-                                  sm_raw + spread_own_tile_bytes(g, sizeof(T)));
     } else {
-        for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
+        bool owned = false;
+        if constexpr (kOwnedSpread<T, W>) {
+            owned = D == 3 || p1 - p0 <= owned_point_max_2d(W);
+            if (owned)
+                spread_points_owned<W, D>(ep, sorted, p0, p1, Ex, Exy, 0, 0, ftile,
+                                          sm_raw + spread_own_tile_bytes(g, sizeof(T)));
+        }
+        for (int p = owned ? p1 : p0 + (int)threadIdx.x; p < p1; p += blockDim.x) {
             U u[3];
             load_packed<T, D>(sorted, p, u);
             int i0[3];
