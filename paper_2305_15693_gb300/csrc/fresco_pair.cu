@@ -161,7 +161,7 @@ __device__ __forceinline__ void add_pair(const PairGeom &g, T r2, const T (&dx)[
                                          T eps, T alpha, T eps_alpha, bool harmonic, bool hertz,
                                          EnergySum<T> &e, T (&f)[3]) {
     const T r = sqrt(r2);
-    const T u = T(1) - r * inv_sig;
+    const T u = fmax(T(1) - r * inv_sig, T(0));   // (r2 < sigma^2 may still round to r > sigma)
     T up;   // u^(alpha - 1)
     if (harmonic) up = u;
     else if (hertz) up = u * sqrt(u);
@@ -187,10 +187,10 @@ constexpr int kPairSegs = D == 3 ? 18 : 6;
 // for the largest total (about 1.6 times the mean at 14 candidates) and not for the largest count
 // of every cell in turn. What bounds it is that imbalance and the instructions per candidate (a
 // prefetch of the next candidate's record changed nothing). 2^21 points in 3D, sigma = 0.8
-// spacings, FP32, GB300: 222 us; the whole term 674 -> 323 us against one loop per cell with a
-// division per candidate and axis. With two cells along an axis (sigma above a third of the box) a
-// candidate's shift is not known from its cell: the general form scans the distinct cells one by
-// one and rounds to the nearest image.
+// spacings, FP32, GB300, the whole term: 741 -> 378 us against one loop per cell with a division per
+// candidate and axis and an FP64 addition per pair. With two cells along an axis (sigma above a
+// third of the box) a candidate's shift is not known from its cell: the general form scans the
+// distinct cells one by one and rounds to the nearest image.
 template <typename T, int D, bool ROWS>
 __global__ void __launch_bounds__(128) k_pair(PairGeom g, const T *__restrict__ sorted,
                                               const int *__restrict__ perm,
