@@ -82,7 +82,13 @@ typedef struct {
 #define FRESCO_GRAD_DIRECT 0
 #define FRESCO_GRAD_KDERIV 1
 
-/* Plan parameters, filled by fresco_plan_query and fresco_get_info. */
+/* Small plans. Where the options leave the choice to the library (no width_override, no tile, a
+ * tolerance of at most 1e-5 in FP32 or 1e-9 in FP64) and direct sums over points and wavevectors are
+ * estimated to take less time than the NUFFT, a plan runs them: three launches, no grid, errors those
+ * of the arithmetic alone. Every entry point works alike on such a plan; tile_order has no effect. */
+
+/* Plan parameters, filled by fresco_plan_query and fresco_get_info. Grid, kernel and tiles are those
+ * of the NUFFT (of a plan that runs direct sums: those it would have). */
 typedef struct {
     int dim;
     int precision;
@@ -328,8 +334,9 @@ fresco_status fresco_lbfgs_destroy(fresco_lbfgs_t s);
  * single device array; every stage (sort, spread, mask, interpolation) runs as one launch over
  * all instances. The uniform FFTs run per size class (fine grids rounded up to 2^k or 3 2^k): FP32
  * in the library's own kernels, up to sixteen classes in a launch, unless few classes hold very many
- * cells; those, and FP64, as one batched cuFFT call per class and direction. The result for instance i is exactly what
- * fresco_plan / fresco_loss_grad give for that problem alone (up to the larger fine grid). */
+ * cells; those, and FP64, as one batched cuFFT call per class and direction. The result for
+ * instance i is what the NUFFT of fresco_plan / fresco_loss_grad gives for that problem alone (up to
+ * the larger fine grid). */
 typedef struct fresco_batch_s *fresco_batch_t;
 
 /* boxes: host [n_inst][dim]; n_points, n_modes: host [n_inst]; masks: host int32, the instances'
