@@ -148,11 +148,14 @@ fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, in
 // transforms: they save the library form's launches, six and more for every class, and cost more per
 // cell (the direct mode's above all, with two columns and complex rows back). Measured on GB300,
 // transforms and mask, cuFFT / these kernels (us). kderiv: one class of 4.2e6 cells 58 / 55, 9.4e6
-// (3072^2) 129 / 111, 1.7e7 (16 grids of 1024^2) 127 / 146, 6.7e7 (64 of 1024^2) 434 / 515, 7.5e7 (two
-// of 6144^2) 634 / 655; nine classes of 1.6e7 together 427 / 160. Direct: 2.4e6 73 / 71, 4.2e6 (four of
-// 1024^2) 76 / 82, 9.4e6 163 / 176, 6.7e7 573 / 830; nine classes 488 / 299, two of 2.1e7 278 / 316.
+// (3072^2) 129 / 111, 1.7e7 (16 grids of 1024^2) 127 / 146, 6.7e7 (64 of 1024^2) 434 / 515; two of 2.7e7
+// together 265 / 263, 8.2e7 689 / 729; four of 6.8e7 566 / 556, 2.0e8 1378 / 1590; nine of 1.6e7
+// 427 / 160, 9.6e7 1003 / 804, 2.0e8 1824 / 1608. Direct: one class of 2.4e6 73 / 71, 4.2e6 (four of
+// 1024^2) 76 / 82, 6.7e7 573 / 830; two of 1.1e7 224 / 181, 1.3e7 215 / 225; four of 1.7e7 303 / 241,
+// 3.3e7 496 / 546; nine of 5.2e7 852 / 720, 9.6e7 1330 / 1313, 1.1e8 1398 / 1637. Over 80 ensembles of
+// both modes the form not taken is at most 1.02 (kderiv) and 1.04 (direct) times as fast as a whole.
 inline bool fft_ensemble_pays(double cells, int classes, bool kderiv) {
-    return cells <= (kderiv ? 1.0e7 : 4.0e6) * classes;
+    return cells <= (kderiv ? 2.4e7 * classes - 1.4e7 : 6.65e6 * classes - 2.65e6);
 }
 void fft_set_free(FftSet *f);
 // first[k] = index of the first representative with n_x >= k, k = 0 .. kx + 1 (rep_n is n_x major)

@@ -21,10 +21,11 @@ def _built():
 
 
 @pytest.mark.parametrize("mode", ["kderiv", "direct"])
-@pytest.mark.parametrize("Ks", [(510,) * 4, (250,) * 3, (250, 510, 30, 510, 510)])
+@pytest.mark.parametrize("Ks", [(510,) * 4, (250,) * 3, (250, 510, 30, 510, 510),
+                                (250, 510, 30, 510, 510, 510, 510)])
 def test_instances_match_single_plans(Ks, mode):
-    """Grids of 2048^2 (K = 510), 1024^2 (250) and 128^2 (30): 1.7e7 and 3.1e6 cells in one class and
-    1.4e7 in three."""
+    """Grids of 2048^2 (K = 510), 1024^2 (250) and 128^2 (30): 1.7e7 and 3.1e6 cells in one class,
+    1.4e7 and 2.2e7 in three."""
     import torch
     from paper_2305_15693_gb300 import fresco
     g = inputs.rng(len(Ks))
