@@ -682,6 +682,14 @@ def constraint_side_bytes(dim: int, n_k: int, fine: int, esize: int, dq: bool) -
             "spread": n_k * (per_k_in + 2 * esize) + fine * 2 * esize}
 
 
+def constraint_side_cells(n_fine: list, width: int, esize: int) -> int:
+    """Cells of the fine grid that the constraint side reads or writes: all, but of a 2D FP32 grid
+    (real rows, enough tiles) only the half plane l_x = -w .. n_x / 2 + w."""
+    if len(n_fine) == 2 and esize == 4:
+        return n_fine[1] * (n_fine[0] // 2 + 2 * width + 1)
+    return int(np.prod(n_fine))
+
+
 def constraint_side_roofline(stages: dict, dim: int, n_k: int, fine: int, esize: int, dq: bool,
                              calls: int, workload: str) -> dict:
     """HBM roofline of the slower of the two constraint-side kernels (stage times from the
@@ -811,7 +819,7 @@ def run_nuwnu(args, fw, rank, world, local_rank, dist_on):
     info = plan.info
     stages = profile_stages(plan, args.steps, lambda: plan.loss_grad(pts))
     esize = 4 if fw.dtype == "f32" else 8
-    fine = int(np.prod(info["n_fine"][:fw.dim]))
+    fine = constraint_side_cells(info["n_fine"][:fw.dim], info["width"], esize)
     roof = constraint_side_roofline(stages, fw.dim, k.shape[0], fine, esize, True, args.steps,
                                     fw.name)
     # accuracy on a subsample the oracle finishes in seconds: 4096 points, all wavevectors
@@ -947,7 +955,7 @@ def run_uwnu(args, fw, rank, world, local_rank, dist_on):
     info = plan.info
     stages = profile_stages(plan, args.steps, lambda: plan.loss_grad(c))
     esize = 4 if fw.dtype == "f32" else 8
-    fine = int(np.prod(info["n_fine"][:fw.dim]))
+    fine = constraint_side_cells(info["n_fine"][:fw.dim], info["width"], esize)
     roof = constraint_side_roofline(stages, fw.dim, fw.n_k, fine, esize, False, args.steps,
                                     fw.name)
     # accuracy and the oracle's rate on a sample the oracle finishes in seconds: every weight
