@@ -475,23 +475,26 @@ struct DirectPlan {
 static constexpr double kDirectWork[2] = {4.0e7, 9.0e6};   // FP32, FP64
 // With few points most SMs idle, the time is that of one block and the wavevectors alone decide;
 // the product above does not see it (100 points and K = 500 took 1226 us, the NUFFT 185). Estimates
-// of both forms in us, [precision][dimension - 2]; the NUFFT's without its points, few in every plan
-// that gets here. Fitted to 170 pairs of plans of 1 to 8000 points with disks, balls, strips and
-// sparse masks of |n| up to 4000, on both sides of the line. Direct sums / NUFFT: 2D FP32, 300
-// points, K = 60 31 / 55, 100 55 / 57, 130 75 / 58, 200 160 / 70; 10 points, 30 wavevectors of |n| up
-// to 2000 170 / 1315, a strip of 4000 x 1 163 / 94; 2D FP64, 300 points, K = 60 100 / 142, 80 156 /
-// 136; K = 50 and 1000 points 100 / 130, 2000 points 157 / 134; 3D, K = 12, 2000 points 35 / 127,
-// FP64 221 / 369.
+// of both forms in us, [precision][dimension - 2]. Fitted to 170 pairs of plans of 1 to 8000 points with
+// disks, balls, strips and sparse masks of |n| up to 4000, and to 1380 of 30 to 10^6 points with disks and
+// balls, on both sides of the line. Direct sums / NUFFT: 2D FP32, 300 points, K = 60 31 / 55, 100 55 / 57,
+// 130 75 / 58, 200 160 / 70; 120000 points, K = 10 62 / 91; 10 points, 30 wavevectors of |n| up to 2000
+// 170 / 1315, a strip of 4000 x 1 163 / 94; 2D FP64, 300 points, K = 60 100 / 142, 80 156 / 136; K = 50
+// and 1000 points 100 / 130, 2000 points 157 / 134; K = 10 and 3000 points 48 / 1295, 30000 157 / 12123;
+// 3D, K = 18 and 3000 points 109 / 139; FP64, K = 10 and 1000 points 114 / 212, 3000 189 / 284.
 struct DirectCost {
     double fixed, quad, row;         // launches; a quad, a quad row of one block's walk
+    double turn;                     // points from which on an SM's blocks wait for its FP64 pipe
     double pt_quad, pt_phase;        // a point's share of the sums over a quad, of one phase
     double nufft, nufft_cell;        // the NUFFT's launches, 10^6 cells of its fine grid
+    double nufft_pt;                 // a point (FP64: few enough tiles that all of them count)
+    double nufft_dense, crowd;       // more than a point a cell; points per 10^6 cells (few tiles)
 };
 static constexpr DirectCost kDirectCost[2][2] = {
-    {{18.0, 0.0152, 0.11, 2.0e-6, 1.4e-5, 55.0, 20.0},
-     {15.0, 0.029, 0.11, 6.5e-6, 1.4e-5, 100.0, 100.0}},
-    {{22.0, 0.097, 0.15, 3.4e-5, 6.0e-5, 110.0, 250.0},
-     {25.0, 0.27, 0.15, 3.4e-5, 6.0e-5, 190.0, 900.0}}};
+    {{18.0, 0.0152, 0.11, 0.0, 2.0e-6, 1.4e-5, 55.0, 20.0, 0.0, 30.0, 1.5e-7},
+     {15.0, 0.029, 0.11, 0.0, 3.0e-6, 1.0e-5, 100.0, 100.0, 0.0, 0.0, 1.5e-7}},
+    {{22.0, 0.097, 0.15, 1216.0, 3.4e-5, 6.0e-5, 122.0, 250.0, 0.0, 0.0, 3.3e-4},
+     {25.0, 0.27, 0.15, 2000.0, 1.0e-5, 3.0e-5, 180.0, 900.0, 0.035, 0.0, 1.5e-4}}};
 // Tolerances the plan may ask for: the direct sums carry the working precision, so a plan that
 // states a looser tolerance keeps the NUFFT whose error it expects (and its speed at that width).
 static constexpr double kDirectTol[2] = {1.0e-5, 1.0e-9};
@@ -641,12 +644,13 @@ fresco_status direct_build(DirectPlan **out, int dim, int64_t n_points, const do
     g.n_quad = (int)quads.size();
     if (8.0 * g.n_quad * (double)n_points > 1.25 * work) return FRESCO_OK;
     const DirectCost &c = kDirectCost[precision == FRESCO_F64][dim - 2];
-    // FP64: the walk is bound by the FP64 pipe, which further blocks on an SM share
-    const double turns =
-        precision == FRESCO_F64 ? std::max(1.0, (double)n_points / (152.0 * 8.0)) : 1.0;
+    const double n = (double)n_points, mcells = fine_cells * 1e-6;
+    const double turns = c.turn > 0.0 ? std::max(1.0, n / c.turn) : 1.0;
     const double sums = c.fixed + c.quad * g.n_quad * turns + c.row * (g.nx4 / 4) +
-                        (double)n_points * (c.pt_quad * g.n_quad + c.pt_phase * (g.nx4 + g.n_col));
-    if (sums > c.nufft + c.nufft_cell * fine_cells * 1e-6) return FRESCO_OK;
+                        n * (c.pt_quad * g.n_quad + c.pt_phase * (g.nx4 + g.n_col));
+    const double nufft = c.nufft + c.nufft_cell * mcells + c.nufft_pt * n +
+                         (n > fine_cells ? c.nufft_dense : 0.0) + c.crowd * n / mcells;
+    if (sums > nufft) return FRESCO_OK;
     // one point's phases must fit the shared memory of both kernels
     const size_t es = precision == FRESCO_F64 ? 8 : 4;
     if ((precision == FRESCO_F64 ? direct_rho_smem<double>(g, 1) : direct_rho_smem<float>(g, 1)) >

@@ -22,8 +22,8 @@ def _built():
 
 
 def _mask(form, K):
-    if form == "disk":
-        return inputs.ball_mask(K, 2)
+    if form in ("disk", "ball"):
+        return inputs.ball_mask(K, 2 if form == "disk" else 3)
     if form == "sparse":
         m = inputs.rng(K).integers(-K, K + 1, (30, 2))
     else:   # strip
@@ -38,14 +38,15 @@ def _mask(form, K):
     ("disk", 100, 50, "f64", True), ("disk", 50, 100, "f64", False),
     ("disk", 2000, 50, "f64", False), ("sparse", 10, 500, "f32", True),
     ("sparse", 10, 500, "f64", True), ("strip", 20, 2000, "f32", False),
-    ("strip", 20, 100, "f32", True)])
+    ("strip", 20, 100, "f32", True), ("disk", 12000, 10, "f64", True),
+    ("disk", 100000, 6, "f32", True), ("ball", 3000, 8, "f64", True), ("ball", 4000, 10, "f32", True)])
 def test_form_and_parity(form, n, K, precision, direct):
     import torch
     from paper_2305_15693_gb300 import fresco
     g = inputs.rng(n + K)
     dt = np.float64 if precision == "f64" else np.float32
     mask = _mask(form, K)
-    pts = g.random((n, 2)).astype(dt)
+    pts = g.random((n, mask.shape[1])).astype(dt)
     S0, W = 0.3 * g.random(len(mask)), 0.5 + g.random(len(mask))
     want_l, want_g, _, want_rho = oracle.loss_grad(pts, mask, S0, W)
     with fresco.Plan(1.0, mask, S0, W, n, precision=precision) as plan:
