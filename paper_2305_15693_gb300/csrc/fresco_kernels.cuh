@@ -975,7 +975,7 @@ __device__ __forceinline__ void interp_tile(const Geom &g, const EsPoly<T> &ep,
 
     const T scale = grad_out ? (T)(*grad_out) : T(1);
     if constexpr (sizeof(T) == 8 && D == 3) {
-        if (p1 - p0 <= warp_point_max(W, false)) {
+        if (by_warps(W, false, g, p1 - p0)) {
             // one warp per point (spread_points_owned above has the reason): a lane takes every 32nd
             // (y, z) row of the window. 3D, 20011 points, w = 13: interpolation 2038 -> 541 us
             double *sw = reinterpret_cast<double *>(sm_raw + (sizeof(C) + sizeof(T)) * (size_t)cells);
@@ -1452,7 +1452,7 @@ __device__ __forceinline__ void interp_tile_kd(const Geom &g, const EsPoly<T> &e
     __syncthreads();
     if (!ok) return;
     if constexpr (sizeof(T) == 8 && D == 3) {
-        if (p1 - p0 <= warp_point_max(W, true)) {
+        if (by_warps(W, true, g, p1 - p0)) {
             // one warp per point, as in interp_tile
             double *sw = reinterpret_cast<double *>(sm_raw + interp_kd_tile_bytes(g, sizeof(T)));
             int *si = reinterpret_cast<int *>(sw + kOwnedChunkInterp * D * 2 * W);

@@ -623,15 +623,35 @@ __device__ __forceinline__ int residue_lists(const typename PT<T>::U *__restrict
 // multiply-add per window cell.
 constexpr int kOwnedChunk = 32;       // spread: points whose weights are staged at once
 constexpr int kOwnedChunkInterp = 8;  // interpolation: one point per warp (the field leaves little room)
-// 3D interpolation tiles of at most this many points give each a warp, others a thread: a warp's time
-// per point hardly falls with the kernel's width, a thread's falls with its cube. Where the two meet,
-// from the interpolation stage of 180 plans (3000 to 3 10^5 points, w = 3 .. 13), threads / warps (us):
-// kernel derivative, w = 3, 6 points a tile 26 / 24, 10 77 / 97, 50 83 / 286; w = 5, 15 72 / 51, 36
-// 205 / 340; w = 7, 21 92 / 73, 36 418 / 477; w = 10, 31 206 / 148, 45 829 / 862; w = 13, 38 5491 /
-// 4073, 51 3615 / 4058; direct, w = 4, 10 137 / 112, 15 98 / 102; w = 7, 36 621 / 536, 51 1379 / 1570;
-// w = 12, 51 9421 / 5012.
-__host__ __device__ constexpr int warp_point_max(int w, bool kderiv) {
-    return kderiv ? (w < 9 ? 6 * (w - 2) : 42) : 10 * (w - 3) + 3;
+// Mean points a tile up to which 3D interpolation gives every point a warp, and beyond it a thread. A warp
+// per point keeps the FP64 pipe busy by itself, so its time grows with the points of all blocks on the SM;
+// a thread per point costs a window's latency whatever the points, up to 64 of them, and blocks on the
+// same SM hide each other's. Where the two meet therefore lies about twice as far for a block that has its
+// SM to itself (`alone`: large tiles, or no more tiles than SMs). Interpolation stage with equal tiles,
+// threads / warps (us). Two or more blocks, 1000 to 3024 tiles, kernel derivative: w = 3, 8 points a tile
+// 76 / 72, 12 76 / 107; w = 5, 20 199 / 201 (direct); w = 7, 32 432 / 426, 36 453 / 485; w = 10, 40 722 /
+// 677, 48 722 / 808; w = 13, 48 1216 / 1160, 56 1216 / 1350; w = 15, 56 1203 / 1096, 64 1203 / 1248;
+// direct, w = 7, 40 601 / 526, 48 601 / 625; w = 9, 56 788 / 876 or 670 / 652; w = 10, 48 1168 / 1161, 56
+// 1169 / 1343. Alone, kernel derivative: w = 15, 1000 tiles, 84 2066 / 1761, 96 2117 / 1998, 112 2132 /
+// 2328; 64 to 144 tiles, w = 3, 12 16 / 14, 16 15 / 15; w = 7, 48 49 / 44, 56 48 / 50; w = 10, 72 107 /
+// 100, 84 105 / 117; direct, w = 7, 64 64 / 64; w = 13, 1000 tiles, 96 2042 / 1791, 112 2051 / 2064.
+__host__ __device__ constexpr int warp_point_max(int w, bool kderiv, bool alone) {
+    const int two_kd = 6 * w - 10 < 2 * w + 26 ? 6 * w - 10 : 2 * w + 26;
+    const int two_direct = w < 6 ? 6 * w - 10 : (w < 10 ? 10 * w - 28 : 50);
+    const int one_kd = 11 * w - 20 < 5 * w + 27 ? 11 * w - 20 : 5 * w + 27;
+    const int one_direct = 13 * w - 23 < 5 * w + 45 ? 13 * w - 23 : 5 * w + 45;
+    return alone ? (kderiv ? one_kd : one_direct) : (kderiv ? two_kd : two_direct);
+}
+// Whether a block of the interpolation (one per tile) takes its n points by warps. The plan's mean decides
+// for all tiles but the crowded and the nearly empty: where a launch mixes both forms, blocks of the one
+// hold up their SM's blocks of the other (uniform points, w = 14, 41 a tile, limit 54: 585 us by the mean,
+// 630 with the limit for each tile). An SM has 228 KB of shared memory, each block takes 1 KB of its own.
+__device__ __forceinline__ bool by_warps(int w, bool kderiv, const Geom &g, int n) {
+    unsigned bytes;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(bytes));
+    const int most = warp_point_max(w, kderiv,
+                                    gridDim.x <= 152 || 2 * (bytes + 1024) > 228 * 1024);
+    return g.n_points <= most * g.n_tiles ? n <= 2 * most : 2 * n <= most;
 }
 
 // bytes of the staged weights (and derivatives) and window starts of n points, 16-byte aligned

@@ -22,14 +22,15 @@ def _built():
     _build.build()
 
 
+@pytest.mark.parametrize("K,n", [(6, 900), (14, 9000)])   # (fewer tiles than SMs, and more)
 @pytest.mark.parametrize("mode", ["direct", "kderiv"])
 @pytest.mark.parametrize("width", [2, 3, 4, 5, 6, 7, 8, 10, 12])
-def test_copies_of_points_share_the_gradient(width, mode):
+def test_copies_of_points_share_the_gradient(width, mode, K, n):
     import torch
     from paper_2305_15693_gb300 import fresco
-    n, copies = 900, 8
+    copies = 8
     g = inputs.rng(width)
-    mask = inputs.ball_mask(6, 3)
+    mask = inputs.ball_mask(K, 3)
     S0, W = g.random(len(mask)), 0.5 + g.random(len(mask))
     pts = g.random((n, 3))
     out = []
