@@ -609,6 +609,7 @@ bool fft_cols_fit(const FftDesc &f, bool kderiv) {
 }
 
 constexpr double kOwnCells = 1.2e6;
+constexpr int kOwnRow = 9000;
 
 fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, int64_t rows,
                             bool always) {
@@ -616,8 +617,10 @@ fresco_status fft_set_build(FftSet &f, const int nf[3], int dim, bool kderiv, in
     // passes over memory; ensembles (fft_ensemble_pays) and the 3D rows have rules of their own.
     // Measured, x passes, y passes and mask, cuFFT against these kernels (us): 432^2 46 / 36, 784^2
     // 53 / 38, 2500^2 95 / 109, 6480^2 448 / 471; the 324^3 grid's x passes with cuFFT's (z, y)
-    // transforms 468 / 374
-    if (dim == 2 && !always && (double)nf[0] * nf[1] > kOwnCells) return FRESCO_OK;
+    // transforms 468 / 374. So do grids of few rows longer than kOwnRow, each of which one block
+    // transforms by itself: 8064 x 14 48 / 47, 12096 x 14 51 / 67, 16128 x 42 57 / 81
+    if (dim == 2 && !always && ((double)nf[0] * nf[1] > kOwnCells || nf[0] > kOwnRow))
+        return FRESCO_OK;
     // (the kernels work on whole rows of nf[0] floats; nf[0] is even)
     f.fwd = fft_describe(nf[0] / 2, f.x);
     f.inv = kderiv ? f.fwd : fft_describe(nf[0], f.xc);

@@ -37,7 +37,7 @@ def _mask(form, K):
     ("disk", 100, 300, "f32", False), ("disk", 150, 130, "f32", False),
     ("disk", 100, 50, "f64", True), ("disk", 50, 100, "f64", False),
     ("disk", 2000, 50, "f64", False), ("sparse", 10, 500, "f32", True),
-    ("sparse", 10, 500, "f64", True), ("strip", 20, 2000, "f32", False),
+    ("sparse", 10, 500, "f64", True), ("strip", 20, 2000, "f32", False), ("strip", 20, 3000, "f32", False),
     ("strip", 20, 100, "f32", True), ("disk", 12000, 10, "f64", True),
     ("disk", 100000, 6, "f32", True), ("ball", 3000, 8, "f64", True), ("ball", 4000, 10, "f32", True)])
 def test_form_and_parity(form, n, K, precision, direct):
